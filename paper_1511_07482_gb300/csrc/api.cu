@@ -230,6 +230,16 @@ static bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// device memory of this GPU that its kernels may write
+static bool is_local_device_ptr(const void* p, int device) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 // ============================================================ small FP64 matrices (row stride 4)
 struct Mat {
     int d = 0;
@@ -4111,40 +4121,34 @@ int kdefft_kde_grid(kdefft_ds ds, const double* H, double* out) {
     int L[4] = {0, 0, 0, 0}, P[4];
     KCHK(plan_for(ds, Hm, L, P));
     const KdeDesc g = kde_desc(ds, L);
-    // stencil K_H(delta (.) l), last axis fastest, FP64 on the host
     Mat inv;
     double det;
     spd_inv_det(Hm, inv, det);
-    const double nrm = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
-    std::vector<float> tab((size_t)g.nstencil);
-    for (long long s = 0; s < g.nstencil; ++s) {
-        long long r = s;
-        double x[4] = {0, 0, 0, 0};
-        for (int k = d - 1; k >= 0; --k) {
-            const int w = 2 * L[k] + 1;
-            x[k] = ds->delta[k] * (double)((int)(r % w) - L[k]);
-            r /= w;
-        }
-        double q = 0.0;
-        for (int a = 0; a < d; ++a)
-            for (int b = 0; b < d; ++b) q += x[a] * inv(a, b) * x[b];
-        tab[(size_t)s] = (float)(nrm * std::exp(-0.5 * q));
-    }
-    const size_t bt = (sizeof(float) * tab.size() + 255) & ~(size_t)255;
-    KCHK(c->kdebuf.ensure(bt + sizeof(double) * (size_t)ds->ncells));
+    KdeKernel kn;
+    std::memset(&kn, 0, sizeof(kn));
+    kn.nrm = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
+    for (int a = 0; a < d; ++a)
+        for (int b = 0; b < d; ++b) kn.lam[a * MAXD + b] = inv(a, b);
+    // the kernel writes a device output itself (FP64-aligned memory of this
+    // GPU); any other output takes a copy from the context's buffer
+    const bool direct = is_local_device_ptr(out, c->device) && ((uintptr_t)out & 7) == 0;
+    const size_t bt = (sizeof(float) * (size_t)g.nstencil + 255) & ~(size_t)255;
+    KCHK(c->kdebuf.ensure(bt + (direct ? 0 : sizeof(double) * (size_t)ds->ncells)));
     float* dtab = (float*)c->kdebuf.p;
-    double* dout = (double*)((unsigned char*)c->kdebuf.p + bt);
-    KCU(cudaMemcpyAsync(dtab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice, c->stream));
-    c->h2d += (int64_t)(sizeof(float) * tab.size());
+    double* dout = direct ? out : (double*)((unsigned char*)c->kdebuf.p + bt);
+    c->launches++;   // the stencil table
     cudaEvent_t ev = prof_start(c);
+    KCU(launch_kde_table(g, kn, dtab, c->stream));
     KCU(launch_kde_grid((const float*)ds->counts.p, g, dtab, dout, c->nsm, c->stream));
     prof_stop(c, ev, "kde_grid", 8.0 * (double)ds->ncells + 4.0 * (double)g.nstencil,
               2.0 * (double)ds->ncells * (double)g.nstencil);
-    if (is_device_ptr(out)) {
-        KCU(cudaMemcpyAsync(out, dout, sizeof(double) * ds->ncells, cudaMemcpyDeviceToDevice, c->stream));
-    } else {
-        KCU(cudaMemcpyAsync(out, dout, sizeof(double) * ds->ncells, cudaMemcpyDeviceToHost, c->stream));
-        c->d2h += (int64_t)(sizeof(double) * ds->ncells);
+    if (!direct) {
+        if (is_device_ptr(out)) {
+            KCU(cudaMemcpyAsync(out, dout, sizeof(double) * ds->ncells, cudaMemcpyDeviceToDevice, c->stream));
+        } else {
+            KCU(cudaMemcpyAsync(out, dout, sizeof(double) * ds->ncells, cudaMemcpyDeviceToHost, c->stream));
+            c->d2h += (int64_t)(sizeof(double) * ds->ncells);
+        }
     }
     KCU(cudaStreamSynchronize(c->stream));
     prof_flush(c);

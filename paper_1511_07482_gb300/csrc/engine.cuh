@@ -362,6 +362,12 @@ struct MixComp {                 // w (2 pi)^{-d/2} |S|^{-1/2} exp(-(x - mu)^T S
     double nrm;                  // (2 pi)^{-d/2} |S|^{-1/2}
     double w;
 };
+struct KdeKernel {               // nrm exp(-x^T lam x / 2)
+    double lam[MAXD * MAXD];     // H^-1, row stride MAXD
+    double nrm;                  // (2 pi)^{-d/2} |H|^{-1/2}
+};
+// tab[l] = K_H(delta (.) l) over the stencil, last axis fastest
+cudaError_t launch_kde_table(const KdeDesc& g, const KdeKernel& kn, float* tab, cudaStream_t st);
 // out[g] = n^-1 sum_l c[g - l] ktab[l] for every grid node (ktab: the stencil,
 // last axis fastest); counts FP32
 cudaError_t launch_kde_grid(const float* counts, const KdeDesc& g, const float* ktab, double* out, int nsm,
