@@ -3431,14 +3431,14 @@ int kdefft_bin(kdefft_ctx c, const double* X, int64_t n, int d, const double* lo
         dX = (const double*)xbuf.p;
     }
     // outside counter | block partials of the moments
-    const int mblk = moments_blocks(n, c->nsm);
+    const int mblk = bin_blocks(n, c->nsm);
     const int nv = d + d * d;
     DevBuf misc(&c->cache);
     KCHK(misc.ensure(sizeof(double) * (16 + (size_t)mblk * nv)));
     unsigned long long* dOut = (unsigned long long*)misc.p;
     double* dPart = (double*)misc.p + 16;
     const bool dbl = o.precision == KDEFFT_FP64;
-    // covariance for the normal-scale start point, in one pass shifted by the
+    // covariance for the normal-scale start point, from moments shifted by the
     // grid's centre (block partials summed in block order: the same start
     // point from run to run)
     Shift sh{};
@@ -3446,14 +3446,14 @@ int kdefft_bin(kdefft_ctx c, const double* X, int64_t n, int d, const double* lo
     unsigned long long nout = 0;
     std::vector<double> part((size_t)mblk * nv);
     if (!dbl && o.binning != KDEFFT_BIN_SIMPLE) {
-        // FP32 linear binning: the launch sequence (zeroing, binning, fixed
-        // point to FP32, moments, copies of the outside count and the moment
-        // partials to pinned memory) replays as a CUDA graph when its
+        // FP32 linear binning: the launch sequence (zeroing, binning with
+        // the moments, fixed point to FP32, one copy of the outside count and
+        // the moment partials to pinned memory) replays as a CUDA graph when its
         // pointers and sizes repeat
         int K = 32;   // fixed point with K fractional bits; a cell's total (<= n 2^K) stays below 2^63
         while (K > 8 && (double)n * std::ldexp(1.0, K) >= std::ldexp(1.0, 63)) --K;
         DevBuf& fix = c->binfix;
-        KCHK(fix.ensure(8 * (size_t)ds->ncells));
+        KCHK(fix.ensure(8 * ((size_t)ds->ncells + 1)));   // the accumulators, then the outside counter
         KCHK(ds->counts.ensure(4 * (size_t)ds->ncells));
         // the outside counter and the moment partials come back in one copy
         // of the whole work buffer (counter at 0, partials from 16)
@@ -3471,17 +3471,15 @@ int kdefft_bin(kdefft_ctx c, const double* X, int64_t n, int d, const double* lo
             sig.insert(sig.end(), {bits[0], bits[1], bits[2], g.M[k]});
         }
         auto issue = [&]() -> int {
-            KCU(cudaMemsetAsync(misc.p, 0, sizeof(double) * 16, c->stream));
-            KCU(cudaMemsetAsync(fix.p, 0, 8 * (size_t)ds->ncells, c->stream));
+            unsigned long long* acc = (unsigned long long*)fix.p;
+            KCU(cudaMemsetAsync(acc, 0, 8 * ((size_t)ds->ncells + 1), c->stream));
             cudaEvent_t evb = prof_start(c);
             c->launches++;   // the fixed-point-to-FP32 conversion
-            KCU(launch_bin_linear<unsigned long long>(dX, n, g, (unsigned long long*)fix.p, ds->ncells, dOut,
-                                                      std::ldexp(1.0, K), c->nsm, c->stream));
-            KCU(launch_fix_to_f32((const unsigned long long*)fix.p, (float*)ds->counts.p, ds->ncells,
-                                  std::ldexp(1.0, -K), c->stream));
+            KCU(launch_bin_fixed(dX, n, g, sh, acc, ds->ncells, acc + ds->ncells, std::ldexp(1.0, K), dPart, c->nsm,
+                                 c->stream));
+            KCU(launch_fix_to_f32(acc, (float*)ds->counts.p, ds->ncells, std::ldexp(1.0, -K), acc + ds->ncells, dOut,
+                                  c->nsm, c->stream));
             prof_stop(c, evb, "bin", (double)n * d * 8.0 + (double)ds->ncells * 4.0, (double)n * (1 << d) * 2.0);
-            c->launches += 1;
-            KCU(launch_moments_shifted(dX, n, d, sh, dPart, c->nsm, c->stream));
             KCU(cudaMemcpyAsync(hres, misc.p, sizeof(double) * nres, cudaMemcpyDeviceToHost, c->stream));
             return KDEFFT_OK;
         };
@@ -3501,17 +3499,15 @@ int kdefft_bin(kdefft_ctx c, const double* X, int64_t n, int d, const double* lo
             c->launches++;   // the integer-to-real conversion
             KCHK(ds->counts_i.ensure(4 * (size_t)ds->ncells));
             KCU(cudaMemsetAsync(ds->counts_i.p, 0, 4 * (size_t)ds->ncells, c->stream));
-            KCU(launch_bin_simple(dX, n, g, (int*)ds->counts_i.p, ds->ncells, dOut, c->nsm, c->stream));
+            KCU(launch_bin_simple(dX, n, g, sh, (int*)ds->counts_i.p, ds->ncells, dOut, dPart, c->nsm, c->stream));
             if (dbl)
                 KCU(launch_int_to_real<double>((int*)ds->counts_i.p, (double*)ds->counts.p, ds->ncells, c->stream));
             else
                 KCU(launch_int_to_real<float>((int*)ds->counts_i.p, (float*)ds->counts.p, ds->ncells, c->stream));
         } else {
-            KCU(launch_bin_linear<double>(dX, n, g, (double*)ds->counts.p, ds->ncells, dOut, 1.0, c->nsm, c->stream));
+            KCU(launch_bin_f64(dX, n, g, sh, (double*)ds->counts.p, ds->ncells, dOut, dPart, c->nsm, c->stream));
         }
         prof_stop(c, evb, "bin", (double)n * d * 8.0 + (double)ds->ncells * (dbl ? 8.0 : 4.0), (double)n * (1 << d) * 2.0);
-        c->launches += 1;
-        KCU(launch_moments_shifted(dX, n, d, sh, dPart, c->nsm, c->stream));
         KCU(cudaMemcpyAsync(&nout, dOut, sizeof(nout), cudaMemcpyDeviceToHost, c->stream));
         KCU(cudaMemcpyAsync(part.data(), dPart, sizeof(double) * mblk * nv, cudaMemcpyDeviceToHost, c->stream));
         KCU(cudaStreamSynchronize(c->stream));
@@ -3576,7 +3572,9 @@ int kdefft_bin_many(kdefft_ctx c, int nds, const double* const* X, const int64_t
         ds.opts = o;
         BinJob& jb = jobs[i];
         std::memset(&jb, 0, sizeof(jb));
-        jb.g.d = d;
+        GridDesc g;
+        std::memset(&g, 0, sizeof(g));
+        g.d = d;
         ds.ncells = 1;
         for (int k = 0; k < d; ++k) {
             const double l = lo[(size_t)i * d + k], h = hi[(size_t)i * d + k];
@@ -3587,12 +3585,13 @@ int kdefft_bin_many(kdefft_ctx c, int nds, const double* const* X, const int64_t
             ds.hi[k] = h;
             ds.M[k] = m;
             ds.delta[k] = (h - l) / (double)(m - 1);   // Eq. 16
-            jb.g.lo[k] = l;
-            jb.g.hi[k] = h;
-            jb.g.delta[k] = ds.delta[k];
-            jb.g.M[k] = m;
+            g.lo[k] = l;
+            g.hi[k] = h;
+            g.delta[k] = ds.delta[k];
+            g.M[k] = m;
             ds.ncells *= m;
         }
+        bin_axes(g, jb.ax);
         if (ds.ncells > (1LL << 31)) return fail(KDEFFT_ERR_UNSUPPORTED, "grid too large");
         while (K > 8 && (double)n[i] * std::ldexp(1.0, K) >= std::ldexp(1.0, 63)) --K;
         if (!is_device_ptr(X[i])) {
@@ -3603,7 +3602,8 @@ int kdefft_bin_many(kdefft_ctx c, int nds, const double* const* X, const int64_t
         totcells += (ds.ncells + 3) & ~3LL;   // 16-byte aligned views
         jb.n = n[i];
         jb.ncells = ds.ncells;
-        jb.mblk = (int)std::min<long long>(64, (n[i] + 255) / 256);
+        // few datasets share the chip with more blocks each
+        jb.mblk = (int)std::min<long long>(std::max(64, bin_blocks(n[i], c->nsm) / nds), (n[i] + 255) / 256);
     }
     // device memory: the samples given on the host, the counts of every
     // dataset (one pool the datasets share), fixed-point accumulators, and
@@ -3623,7 +3623,7 @@ int kdefft_bin_many(kdefft_ctx c, int nds, const double* const* X, const int64_t
     KCU(cudaMemsetAsync(c->binfix.p, 0, 8 * (size_t)totcells, c->stream));
     unsigned long long* dOut = (unsigned long long*)misc.p;
     double* dPart = (double*)misc.p + nds;
-    KCHK(c->binjobs.ensure(sizeof(BinJob) * nds * 4));
+    KCHK(c->binjobs.ensure(sizeof(BinJob) * nds));
     BinJob* jd = (BinJob*)c->binjobs.p;
     long long po = 0;
     for (int i = 0; i < nds; ++i) {
@@ -3652,17 +3652,15 @@ int kdefft_bin_many(kdefft_ctx c, int nds, const double* const* X, const int64_t
         fl += (double)n[i] * (1 << d) * 2.0;
     }
     cudaEvent_t evb = prof_start(c);
-    c->launches++;   // phases 0 and 1
-    KCU(launch_bin_many(jobs.data(), jd, nds, 0, qscale, c->stream));
-    KCU(launch_bin_many(jobs.data(), jd + nds, nds, 1, qscale, c->stream));
+    c->launches++;   // the fixed-point-to-FP32 conversion
+    KCU(launch_bin_many(jobs.data(), jd, nds, d, qscale, c->stream));
     prof_stop(c, evb, "bin", by, fl);
-    c->launches += 1;   // the one-pass covariance
-    KCU(launch_bin_many(jobs.data(), jd + 2 * nds, nds, 2, qscale, c->stream));
-    std::vector<double> part((size_t)totpart);
-    std::vector<unsigned long long> nout(nds);
-    KCU(cudaMemcpyAsync(nout.data(), dOut, sizeof(unsigned long long) * nds, cudaMemcpyDeviceToHost, c->stream));
-    KCU(cudaMemcpyAsync(part.data(), dPart, sizeof(double) * totpart, cudaMemcpyDeviceToHost, c->stream));
+    std::vector<double> res(nmisc);   // outside counters | moment partials
+    KCU(cudaMemcpyAsync(res.data(), misc.p, sizeof(double) * nmisc, cudaMemcpyDeviceToHost, c->stream));
     KCU(cudaStreamSynchronize(c->stream));
+    const double* part = res.data() + nds;
+    std::vector<unsigned long long> nout(nds);
+    std::memcpy(nout.data(), res.data(), sizeof(unsigned long long) * nds);
     prof_flush(c);
     po = 0;
     for (int i = 0; i < nds; ++i) {

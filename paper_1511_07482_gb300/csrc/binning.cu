@@ -12,9 +12,10 @@
 // (x_k - lo_k) / delta_k itself, so that the cells match the oracle's bit for
 // bit.
 //
-// Grids that fit in shared memory are accumulated per block there (one
-// privatised histogram per block, flushed with global atomics of the nonzero
-// cells); larger grids use global atomics directly.
+// The sample is read once: the same pass takes the moments that the
+// normal-scale start needs (its FP64 work hides behind the atomics).  Its
+// counts go to a histogram of its own in each block's shared memory where the
+// grid fits, else to global atomics in L2.
 //
 // FP32 counts are accumulated in 64-bit fixed point (each weight rounded to
 // a multiple of 2^-K, K = 32 for samples below 2^31 points): integer sums do
@@ -23,133 +24,294 @@
 // corner weights are FP32 products of the FP64 fractions rounded to FP32: a
 // weight's relative error of a few 2^-24 matches the FP32 rounding of the
 // count itself.  FP64 counts use FP64 weights and FP64 atomics.
+#include <cstring>
 #include <type_traits>
 
+#include "devutil.cuh"
 #include "engine.cuh"
 
 namespace kdefft {
 
-// Linear binning locates a point with t = (x - lo) * (1 / delta): one FP64
-// multiply instead of a division (FP64 is slow on this part).  t is within
-// two ulps of the oracle's (x - lo) / delta, so a point moves to the next
-// cell only within two ulps of a node, where its weight there is ~1e-16.
-struct Recip {
-    double v[MAXD];
-};
+// ------------------------------------------------------------ one point
+// Order-preserving integer of a double: a < b as doubles iff key(a) < key(b)
+// for ordered values; NaN lies beyond both infinities.
+__host__ __device__ __forceinline__ long long order_key(long long bits) {
+    return bits ^ ((bits >> 63) & 0x7fffffffffffffffLL);
+}
 
-__device__ __forceinline__ bool locate(const double* __restrict__ x, const GridDesc& g, const Recip& inv, long long* l,
-                                       double* f, long long* base) {
-    long long b = 0;
-    for (int k = 0; k < g.d; ++k) {
-        if (!(x[k] >= g.lo[k] && x[k] <= g.hi[k])) return false;   // NaN fails too
-        const double top = (double)(g.M[k] - 1);
-        const double t = fmin(__dmul_rn(__dsub_rn(x[k], g.lo[k]), inv.v[k]), top);
-        double lk = floor(t);
-        if (lk >= top) lk = top - 1.0;
-        f[k] = __dsub_rn(t, lk);
-        l[k] = (long long)lk;
-        b = b * g.M[k] + l[k];
+void bin_axes(const GridDesc& g, BinAxes& ax) {
+    std::memset(&ax, 0, sizeof(ax));
+    unsigned int s = 1;
+    for (int k = g.d - 1; k >= 0; --k) {
+        ax.lo[k] = g.lo[k];
+        ax.delta[k] = g.delta[k];
+        ax.inv[k] = 1.0 / g.delta[k];
+        // a bound at zero admits both of its signs
+        const double lo = g.lo[k] == 0.0 ? -0.0 : g.lo[k], hi = g.hi[k] == 0.0 ? 0.0 : g.hi[k];
+        long long b;
+        std::memcpy(&b, &lo, 8);
+        ax.klo[k] = order_key(b);
+        std::memcpy(&b, &hi, 8);
+        ax.khi[k] = order_key(b);
+        ax.top[k] = (int)g.M[k] - 2;
+        ax.stride[k] = s;
+        s *= (unsigned int)g.M[k];
     }
-    *base = b;
-    return true;
 }
 
-// Fixed-point weight of a corner (units of 2^-K, qscale = 2^K) from FP32
-// factors: the location t, l, f stays FP64 as above, but the corner product
-// only feeds an FP32 count, and a few FP32 roundings of the weight stay at
-// the level of that count's own rounding (FP64 arithmetic is slow here).
-__device__ __forceinline__ unsigned long long corner_fixed(int d, int c, const float* ff, const float* gg,
-                                                           float qscale) {
-    float w = 1.f;
-    for (int k = 0; k < d; ++k) w *= ((c >> k) & 1) ? ff[k] : gg[k];
-    return __float2ull_rn(w * qscale);
+// FP64 arithmetic is what a point costs on this part (2 lanes a cycle and SM,
+// 64 for integer operations), so only t = (x - lo) * (1 / delta) is FP64: the
+// bounds are integer comparisons, and cell and fraction come from t's bits.
+// t is within two ulps of the oracle's (x - lo) / delta, so a point moves to
+// the next cell only within two ulps of a node, where its weight there is
+// ~1e-16.  x is inside iff lo <= x <= hi on every axis (NaN is not).
+__device__ __forceinline__ bool inside(double x, long long klo, long long khi) {
+    const long long key = order_key(__double_as_longlong(x));
+    return key >= klo && key <= khi;
 }
 
-template <typename acc>
-__global__ void __launch_bounds__(256) k_bin_linear(const double* __restrict__ X, long long n, GridDesc g, Recip inv,
-                                                    acc* __restrict__ counts, long long ncells,
-                                                    unsigned long long* __restrict__ outside, int use_smem,
-                                                    double qscale) {
+// Cell l = min(floor(t), M - 2) and fraction t - l (1 where t reaches M - 1,
+// which the rounding of delta can push past it) of t >= 0, below 2^31: t is
+// m 2^-sh with a 53-bit m, so the cell is m >> sh and the fraction the bits
+// below, one rounding from FP32 (t < 2^-74 gives a fraction below 2^-73
+// instead of its own, and a weight of zero either way).
+__device__ __forceinline__ int cell_f32(double t, int top, float& f) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(t);
+    const unsigned long long m = (b & 0xfffffffffffffULL) | 0x10000000000000ULL;
+    const int sh = min(1075 - (int)((b >> 52) & 0x7ff), 126);   // the sign of -0 does not matter
+    const int s = min(sh, 63);
+    int l = (int)(m >> s);
+    f = __ull2float_rn(m & ((1ULL << s) - 1)) * __int_as_float((127 - sh) << 23);
+    if (l > top) {
+        l = top;
+        f = 1.f;
+    }
+    return l;
+}
+// the same with the fraction in FP64 (t + 2^52 rounded down holds floor(t))
+__device__ __forceinline__ int cell_f64(double t, int top, double& f) {
+    const double u = __dadd_rd(t, 4503599627370496.0);
+    int l = (int)__double_as_longlong(u);
+    f = __dsub_rn(t, __dsub_rn(u, 4503599627370496.0));
+    if (l > top) {
+        l = top;
+        f = 1.0;
+    }
+    return l;
+}
+
+// Nearest node floor(min(t, M - 1) + 1/2) with t the quotient (x - lo) / delta
+// itself.  t * (1 / delta) is within two ulps of it: the division is only
+// needed within 2^-30 of a tie.
+__device__ __forceinline__ int nearest(double x, double lo, double delta, double inv, int top) {
+    const double y = __dsub_rn(x, lo);
+    double t = __dmul_rn(y, inv);
+    const double h = __dadd_rn(t, 0.5), u = __dadd_rd(h, 4503599627370496.0);
+    const double r = __dsub_rn(h, __dsub_rn(u, 4503599627370496.0));   // in [0, 1)
+    int l = (int)__double_as_longlong(u);
+    if (r < 1e-9 || r > 1.0 - 1e-9) {
+        t = fmin(__ddiv_rn(y, delta), (double)(top + 1));
+        l = (int)floor(__dadd_rn(t, 0.5));
+    }
+    return min(l, top + 1);
+}
+
+// ------------------------------------------------------------ the pass
+// Points i0 + threadIdx.x, + stride, .. below n: their counts into `counts`
+// (kind 0: fixed point, kind 1: FP64, kind 2: whole points), and the block's
+// sums of x - s and (x - s)(x - s)^T to part.
+//
+// A linear-binned point is 2^d 64-bit atomic additions to scattered cells,
+// and what L2 is limited by is the 32-byte sectors they touch (58 G/s on
+// 128^3 with a point per lane).  So a warp spreads its 32 points over lane
+// pairs, half of them at a time, and a pair adds the two neighbours along the
+// last axis with one instruction: three times out of four they share a sector.
+// What is left is FP64: 2 d operations to locate a point and 2 d + d (d + 1) / 2
+// for its moments, 84 % of the FP64 pipe.  Binning and moments with their
+// launches, against a thread per point with run-time dimensions, FP64
+// comparisons and floor, and a second pass for the moments: 1e7 points on
+// 512^2 363 us (866), 1e6 on 128^3 103 us (206), 1e6 on 48^4 142 us (336);
+// FP64 counts, 1e6 on 256^2 97 us (161).
+template <int D, int KIND, typename acc>
+__device__ __forceinline__ void bin_pass(const double* __restrict__ X, long long n, long long i0, long long stride,
+                                         const BinAxes& ax, const double* __restrict__ shift, acc* counts,
+                                         unsigned long long* __restrict__ outside, double qscale,
+                                         double* __restrict__ part) {
+    constexpr int NV = D + D * (D + 1) / 2;
+    constexpr int NP = NV <= 2 ? 2 : NV <= 8 ? 8 : 16;   // sums padded to a power of two
+    const int lane = threadIdx.x & 31;
+    const float qs = (float)qscale;   // 2^K, exact
+    const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    double sum[NP];
+#pragma unroll
+    for (int v = 0; v < NP; ++v) sum[v] = 0.0;
+    unsigned int nout = 0;
+    auto load = [&](long long i, double* x) {
+        if constexpr (D % 2 == 0) {
+            if (vec) {
+#pragma unroll
+                for (int k = 0; k < D; k += 2) {
+                    const double2 v = *reinterpret_cast<const double2*>(X + i * D + k);
+                    x[k] = v.x;
+                    x[k + 1] = v.y;
+                }
+                return;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < D; ++k) x[k] = X[i * D + k];
+    };
+    double xn[D];
+    long long i = i0 + threadIdx.x;
+    if (i < n) load(i, xn);
+    for (; i - lane < n; i += stride) {   // a warp's lanes leave together
+        const bool have = i < n;
+        double x[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) x[k] = xn[k];
+        if (i + stride < n) load(i + stride, xn);   // the next point is on its way meanwhile
+        bool in = have;
+        if (have) {
+#pragma unroll
+            for (int k = 0; k < D; ++k) in = in && inside(x[k], ax.klo[k], ax.khi[k]);
+            if (!in) ++nout;
+        }
+        unsigned int base = 0;
+        if constexpr (KIND == 2) {
+            if (in) {
+#pragma unroll
+                for (int k = 0; k < D; ++k)
+                    base += (unsigned int)nearest(x[k], ax.lo[k], ax.delta[k], ax.inv[k], ax.top[k]) * ax.stride[k];
+                atomicAdd(counts + base, acc(1));
+            }
+        } else {
+            using real = typename std::conditional<KIND == 0, float, double>::type;
+            real f[D];
+#pragma unroll
+            for (int k = 0; k < D; ++k) {
+                const double t = in ? __dmul_rn(__dsub_rn(x[k], ax.lo[k]), ax.inv[k]) : 0.0;
+                if constexpr (KIND == 0)
+                    base += (unsigned int)cell_f32(t, ax.top[k], f[k]) * ax.stride[k];
+                else
+                    base += (unsigned int)cell_f64(t, ax.top[k], f[k]) * ax.stride[k];
+            }
+            if (!in) base = 0xffffffffu;   // no cell: the grid has at most 2^31
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int src = half * 16 + (lane >> 1);
+                const unsigned int b = __shfl_sync(0xffffffffu, base, src);
+                real ff[D], gg[D];
+#pragma unroll
+                for (int k = 0; k < D; ++k) {
+                    ff[k] = __shfl_sync(0xffffffffu, f[k], src);
+                    if constexpr (KIND == 0)
+                        gg[k] = 1.f - ff[k];
+                    else
+                        gg[k] = __dsub_rn(1.0, ff[k]);
+                }
+                if (b == 0xffffffffu) continue;
+                const real last = (lane & 1) ? ff[D - 1] : gg[D - 1];
+#pragma unroll
+                for (int c = 0; c < (1 << (D - 1)); ++c) {
+                    unsigned int idx = b + (lane & 1);
+                    real w = real(1);
+#pragma unroll
+                    for (int k = 0; k < D - 1; ++k) {
+                        if ((c >> k) & 1) idx += ax.stride[k];
+                        const real v = ((c >> k) & 1) ? ff[k] : gg[k];
+                        if constexpr (KIND == 0)
+                            w = k == 0 ? v : w * v;
+                        else
+                            w = k == 0 ? v : __dmul_rn(w, v);
+                    }
+                    if constexpr (KIND == 0) {
+                        w = D == 1 ? last : w * last;
+                        atomicAdd(counts + idx, (acc)__float2ull_rn(w * qs));
+                    } else {
+                        w = D == 1 ? last : __dmul_rn(w, last);
+                        atomicAdd(counts + idx, (acc)w);
+                    }
+                }
+            }
+        }
+        if (have) {   // moments: every point, inside or not
+#pragma unroll
+            for (int k = 0; k < D; ++k) x[k] -= shift[k];
+#pragma unroll
+            for (int k = 0; k < D; ++k) sum[k] += x[k];
+            int v = D;
+#pragma unroll
+            for (int a = 0; a < D; ++a)
+#pragma unroll
+                for (int b = a; b < D; ++b) sum[v++] += x[a] * x[b];
+        }
+    }
+    nout = __reduce_add_sync(0xffffffffu, nout);
+    if (nout && lane == 0) atomicAdd(outside, (unsigned long long)nout);
+    // Sums over the warp, for all values together: at each step a lane keeps
+    // half of its values and adds the other lane's share of them, which takes
+    // about as many FP64 additions as there are values instead of five for
+    // each.  The pairs added are those of a shuffle-down tree, so the bits
+    // are its bits; the eight warps are then added in order.
+    int held = NP, first = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (held > 1) {
+            const bool upper = (lane & o) != 0;
+            held >>= 1;
+#pragma unroll
+            for (int v = 0; v < NP / 2; ++v) {
+                if (v < held) {
+                    const double keep = upper ? sum[v + held] : sum[v];
+                    const double give = upper ? sum[v] : sum[v + held];
+                    sum[v] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+            }
+            if (upper) first += held;
+        } else {
+            sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], o);
+        }
+    }
+    __shared__ double red[8][NP];
+    constexpr int LOW = 32 / NP;   // lanes that hold the same value
+    if ((lane & (LOW - 1)) == 0) red[threadIdx.x >> 5][first] = sum[0];
+    __syncthreads();
+    constexpr int NF = D + D * D;
+    if (threadIdx.x < NF) {
+        int v = threadIdx.x;
+        if (v >= D) {   // the full product matrix from its upper triangle
+            const int p = (v - D) / D, q = (v - D) % D, a = p < q ? p : q, b = p < q ? q : p;
+            v = D + a * D - a * (a - 1) / 2 + (b - a);
+        }
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w][v];
+        part[threadIdx.x] = t;   // block partial; summed in block order by the host
+    }
+}
+
+template <int D, int KIND, typename acc>
+__global__ void __launch_bounds__(256) k_bin(const double* __restrict__ X, long long n,
+                                             const __grid_constant__ BinAxes ax, const __grid_constant__ Shift sh,
+                                             acc* __restrict__ counts, unsigned int smem_cells,
+                                             unsigned long long* __restrict__ outside, double qscale,
+                                             double* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     acc* hist = reinterpret_cast<acc*>(smem_raw);
-    if (use_smem) {
-        for (long long c = threadIdx.x; c < ncells; c += blockDim.x) hist[c] = acc(0);
+    for (unsigned int c = threadIdx.x; c < smem_cells; c += blockDim.x) hist[c] = acc(0);
+    if (smem_cells) __syncthreads();
+    const long long i0 = (long long)blockIdx.x * blockDim.x, stride = (long long)gridDim.x * blockDim.x;
+    double* out = part + (size_t)blockIdx.x * (D + D * D);
+    if (smem_cells)
+        bin_pass<D, KIND, acc>(X, n, i0, stride, ax, sh.s, hist, outside, qscale, out);
+    else
+        bin_pass<D, KIND, acc>(X, n, i0, stride, ax, sh.s, counts, outside, qscale, out);
+    if (smem_cells) {
         __syncthreads();
-    }
-    long long stride[MAXD];
-    {
-        long long s = 1;
-        for (int k = g.d - 1; k >= 0; --k) {
-            stride[k] = s;
-            s *= g.M[k];
-        }
-    }
-    const int ncorner = 1 << g.d;
-    constexpr bool fixed = std::is_same<acc, unsigned long long>::value;
-    const float qs = (float)qscale;   // 2^K, exact
-    unsigned long long nout = 0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        double x[MAXD], f[MAXD];
-        long long l[MAXD], base;
-        for (int k = 0; k < g.d; ++k) x[k] = X[i * g.d + k];
-        if (!locate(x, g, inv, l, f, &base)) {
-            ++nout;
-            continue;
-        }
-        float ff[MAXD], gg[MAXD];
-        if constexpr (fixed)
-            for (int k = 0; k < g.d; ++k) {
-                ff[k] = (float)f[k];
-                gg[k] = 1.f - ff[k];
-            }
-        for (int b = 0; b < ncorner; ++b) {
-            long long idx = base;
-            for (int k = 0; k < g.d; ++k) idx += ((b >> k) & 1) * stride[k];
-            acc* dst = use_smem ? hist + idx : counts + idx;
-            if constexpr (fixed) {
-                atomicAdd(dst, corner_fixed(g.d, b, ff, gg, qs));
-            } else {
-                double w = 1.0;
-                for (int k = 0; k < g.d; ++k) w = __dmul_rn(w, ((b >> k) & 1) ? f[k] : __dsub_rn(1.0, f[k]));
-                atomicAdd(dst, w);
-            }
-        }
-    }
-    if (nout) atomicAdd(outside, nout);
-    if (use_smem) {
-        __syncthreads();
-        for (long long c = threadIdx.x; c < ncells; c += blockDim.x) {
+        for (unsigned int c = threadIdx.x; c < smem_cells; c += blockDim.x) {
             const acc v = hist[c];
             if (v != acc(0)) atomicAdd(counts + c, v);
         }
     }
-}
-
-__global__ void __launch_bounds__(256) k_bin_simple(const double* __restrict__ X, long long n, GridDesc g,
-                                                    int* __restrict__ counts, unsigned long long* __restrict__ outside) {
-    unsigned long long nout = 0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        long long idx = 0;
-        bool ok = true;
-        for (int k = 0; k < g.d; ++k) {
-            const double x = X[i * g.d + k];
-            if (!(x >= g.lo[k] && x <= g.hi[k])) {
-                ok = false;
-                break;
-            }
-            const double t = fmin(__ddiv_rn(__dsub_rn(x, g.lo[k]), g.delta[k]), (double)(g.M[k] - 1));
-            const long long lk = (long long)floor(__dadd_rn(t, 0.5));
-            idx = idx * g.M[k] + lk;
-        }
-        if (!ok) {
-            ++nout;
-            continue;
-        }
-        atomicAdd(counts + idx, 1);
-    }
-    if (nout) atomicAdd(outside, nout);
 }
 
 __global__ void k_f32_to_f64(const float* __restrict__ src, double* __restrict__ dst, long long n) {
@@ -165,17 +327,37 @@ cudaError_t launch_f32_to_f64(const float* src, double* dst, long long n, cudaSt
     return cudaGetLastError();
 }
 
-__global__ void k_fix_to_f32(const unsigned long long* __restrict__ src, float* __restrict__ dst, long long n,
-                             double unit) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        dst[i] = (float)((double)src[i] * unit);
+// Fixed point to FP32, four cells a thread (16-byte loads and stores; both
+// arrays are 16-byte aligned): one correctly rounded conversion and an exact
+// product with a power of two.
+__device__ __forceinline__ void fix_cells(const unsigned long long* __restrict__ src, float* __restrict__ dst,
+                                          long long c, long long n, float unit) {
+    if (c + 4 <= n) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(src + c);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(src + c + 2);
+        *reinterpret_cast<float4*>(dst + c) = make_float4(__ull2float_rn(a.x) * unit, __ull2float_rn(a.y) * unit,
+                                                          __ull2float_rn(b.x) * unit, __ull2float_rn(b.y) * unit);
+    } else {
+        for (; c < n; ++c) dst[c] = __ull2float_rn(src[c]) * unit;
+    }
 }
 
-cudaError_t launch_fix_to_f32(const unsigned long long* src, float* dst, long long n, double unit, cudaStream_t st) {
+__global__ void __launch_bounds__(256) k_fix_to_f32(const unsigned long long* __restrict__ src,
+                                                    float* __restrict__ dst, long long n, float unit,
+                                                    const unsigned long long* __restrict__ outside,
+                                                    unsigned long long* __restrict__ outside_copy) {
+    for (long long c = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); c < n;
+         c += 4LL * gridDim.x * blockDim.x)
+        fix_cells(src, dst, c, n, unit);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *outside_copy = *outside;
+}
+
+cudaError_t launch_fix_to_f32(const unsigned long long* src, float* dst, long long n, double unit,
+                              const unsigned long long* outside, unsigned long long* outside_copy, int nsm,
+                              cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    long long b = (n + 255) / 256;
-    if (b > 4096) b = 4096;
-    k_fix_to_f32<<<(int)b, 256, 0, st>>>(src, dst, n, unit);
+    const long long b = (n + 1023) / 1024, cap = (long long)nsm * 8;
+    k_fix_to_f32<<<(unsigned)(b < cap ? b : cap), 256, 0, st>>>(src, dst, n, (float)unit, outside, outside_copy);
     return cudaGetLastError();
 }
 
@@ -183,42 +365,6 @@ template <typename real>
 __global__ void k_int_to_real(const int* __restrict__ src, real* __restrict__ dst, long long n) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         dst[i] = (real)src[i];
-}
-
-static int blocks_for(long long n, int nsm, int per_sm) {
-    long long b = (n + 255) / 256;
-    const long long cap = (long long)nsm * per_sm;
-    if (b > cap) b = cap;
-    if (b < 1) b = 1;
-    return (int)b;
-}
-
-template <typename acc>
-cudaError_t launch_bin_linear(const double* X, long long n, const GridDesc& g, acc* counts, long long ncells,
-                              unsigned long long* outside, double qscale, int nsm, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    const size_t hist_bytes = sizeof(acc) * (size_t)ncells;
-    const int use_smem = hist_bytes <= 96 * 1024;
-    size_t sm = 0;
-    int grid;
-    if (use_smem) {
-        sm = hist_bytes;   // within the 96 KB set once by prepare_binning (no attribute call here: graph capture)
-        grid = blocks_for(n, nsm, 2);
-    } else {
-        grid = blocks_for(n, nsm, 8);
-    }
-    Recip inv{};
-    for (int k = 0; k < g.d; ++k) inv.v[k] = 1.0 / g.delta[k];
-    k_bin_linear<acc><<<grid, 256, sm, st>>>(X, n, g, inv, counts, ncells, outside, use_smem, qscale);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_bin_simple(const double* X, long long n, const GridDesc& g, int* counts, long long ncells,
-                              unsigned long long* outside, int nsm, cudaStream_t st) {
-    (void)ncells;
-    if (n <= 0) return cudaSuccess;
-    k_bin_simple<<<blocks_for(n, nsm, 8), 256, 0, st>>>(X, n, g, counts, outside);
-    return cudaGetLastError();
 }
 
 template <typename real>
@@ -230,172 +376,130 @@ cudaError_t launch_int_to_real(const int* src, real* dst, long long n, cudaStrea
     return cudaGetLastError();
 }
 
-// Sample covariance for the normal-scale start point, in one pass: FP64
-// block sums of x - s and (x - s)(x - s)^T
-// with a fixed shift s inside the data (the grid's centre), from which
-// cov = (S2 - S1 S1^T / n) / (n - 1); with s near the mean the subtraction
-// loses little.  out: per block d + d^2 values.
-__global__ void __launch_bounds__(256) k_moments_shifted(const double* __restrict__ X, long long n, int d, Shift sh,
-                                                         double* __restrict__ out) {
-    double acc[MAXD + MAXD * MAXD];
-    const int nv = d + d * d;
-    for (int v = 0; v < nv; ++v) acc[v] = 0.0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        double x[MAXD];
-        for (int k = 0; k < d; ++k) x[k] = X[i * d + k] - sh.s[k];
-        for (int k = 0; k < d; ++k) acc[k] += x[k];
-        for (int a = 0; a < d; ++a)
-            for (int b = 0; b < d; ++b) acc[d + a * d + b] += x[a] * x[b];
-    }
-    __shared__ double red[8][MAXD + MAXD * MAXD];
-    for (int v = 0; v < nv; ++v) {
-        double t = acc[v];
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][v] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x < nv) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
-        out[(size_t)blockIdx.x * nv + threadIdx.x] = t;   // block partial; summed in block order by the host
-    }
+// Counts that fit in kBinSmem (two blocks an SM) go to a histogram per block.
+// Against global atomics for these it is never slower (a pass over 1000 points
+// on 100^2 35 against 37 us with its launches, 2e6 points 103 against 145 us),
+// and where many points share few cells it takes the contention out of L2
+// (8e6 points on 512 nodes 161 against 2224 us).
+constexpr int kBinSmem = 96 * 1024;
+
+// blocks of a binning pass: at most two per SM (the moments' block partials,
+// which the host adds in block order, keep their number and their points)
+int bin_blocks(long long n, int nsm) {
+    long long b = (n + 255) / 256;
+    const long long cap = 2LL * nsm;
+    if (b > cap) b = cap;
+    if (b < 1) b = 1;
+    return (int)b;
 }
 
-cudaError_t launch_moments_shifted(const double* X, long long n, int d, const Shift& sh, double* out, int nsm,
-                                   cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    k_moments_shifted<<<moments_blocks(n, nsm), 256, 0, st>>>(X, n, d, sh, out);
+template <int D, int KIND, typename acc>
+static cudaError_t bin_go(const double* X, long long n, const BinAxes& ax, const Shift& sh, acc* counts,
+                          long long ncells, unsigned long long* outside, double qscale, double* part, int nsm,
+                          cudaStream_t st) {
+    const int grid = bin_blocks(n, nsm);
+    const long long bytes = (long long)sizeof(acc) * ncells;
+    const bool smem = bytes <= kBinSmem;
+    k_bin<D, KIND, acc><<<grid, 256, smem ? (size_t)bytes : 0, st>>>(X, n, ax, sh, counts, smem ? (unsigned)ncells : 0u,
+                                                                     outside, qscale, part);
     return cudaGetLastError();
 }
 
-int moments_blocks(long long n, int nsm) { return blocks_for(n, nsm, 2); }
+template <int KIND, typename acc>
+static cudaError_t bin_d(const double* X, long long n, const GridDesc& g, const Shift& sh, acc* counts,
+                         long long ncells, unsigned long long* outside, double qscale, double* part, int nsm,
+                         cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    BinAxes ax;
+    bin_axes(g, ax);
+    switch (g.d) {
+        case 1: return bin_go<1, KIND, acc>(X, n, ax, sh, counts, ncells, outside, qscale, part, nsm, st);
+        case 2: return bin_go<2, KIND, acc>(X, n, ax, sh, counts, ncells, outside, qscale, part, nsm, st);
+        case 3: return bin_go<3, KIND, acc>(X, n, ax, sh, counts, ncells, outside, qscale, part, nsm, st);
+        case 4: return bin_go<4, KIND, acc>(X, n, ax, sh, counts, ncells, outside, qscale, part, nsm, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
 
+cudaError_t launch_bin_fixed(const double* X, long long n, const GridDesc& g, const Shift& sh,
+                             unsigned long long* counts, long long ncells, unsigned long long* outside, double qscale,
+                             double* part, int nsm, cudaStream_t st) {
+    return bin_d<0, unsigned long long>(X, n, g, sh, counts, ncells, outside, qscale, part, nsm, st);
+}
+cudaError_t launch_bin_f64(const double* X, long long n, const GridDesc& g, const Shift& sh, double* counts,
+                           long long ncells, unsigned long long* outside, double* part, int nsm, cudaStream_t st) {
+    return bin_d<1, double>(X, n, g, sh, counts, ncells, outside, 1.0, part, nsm, st);
+}
+cudaError_t launch_bin_simple(const double* X, long long n, const GridDesc& g, const Shift& sh, int* counts,
+                              long long ncells, unsigned long long* outside, double* part, int nsm, cudaStream_t st) {
+    return bin_d<2, int>(X, n, g, sh, counts, ncells, outside, 1.0, part, nsm, st);
+}
 
 // ------------------------------------------------------------ batched binning
-__device__ __forceinline__ int bin_job_of(const BinJob* __restrict__ jobs, int n, long long b) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (jobs[mid].blk0 <= b)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
+constexpr int kCellsPerBlock = 256 * 16;
 
-constexpr int kBinPtsPerBlock = 256 * 8;
-constexpr int kCellsPerBlock = 256 * 4;
-
-__global__ void __launch_bounds__(256) k_bin_many(const BinJob* __restrict__ jobs, int njobs, int phase,
-                                                  double qscale) {
-    const BinJob& jb = jobs[bin_job_of(jobs, njobs, blockIdx.x)];
+template <int D>
+__global__ void __launch_bounds__(256) k_bin_many(const BinJob* __restrict__ jobs, int njobs, double qscale) {
+    const BinJob& jb = jobs[job_of_warp(njobs, blockIdx.x, [&](int k) { return jobs[k].blk0; })];
     const long long b = (long long)blockIdx.x - jb.blk0;
-    const GridDesc& g = jb.g;
-    const int d = g.d;
-    if (phase == 0) {
-        long long stride[MAXD];
-        {
-            long long s = 1;
-            for (int k = d - 1; k >= 0; --k) {
-                stride[k] = s;
-                s *= g.M[k];
-            }
-        }
-        const int ncorner = 1 << d;
-        Recip inv{};   // the same correctly rounded reciprocals as launch_bin_linear's
-        for (int k = 0; k < d; ++k) inv.v[k] = __drcp_rn(g.delta[k]);
-        unsigned long long nout = 0;
-        const long long i0 = b * kBinPtsPerBlock;
-        const long long i1 = i0 + kBinPtsPerBlock < jb.n ? i0 + kBinPtsPerBlock : jb.n;
-        for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-            double x[MAXD], f[MAXD];
-            long long l[MAXD], base;
-            for (int k = 0; k < d; ++k) x[k] = jb.X[i * d + k];
-            if (!locate(x, g, inv, l, f, &base)) {
-                ++nout;
-                continue;
-            }
-            float ff[MAXD], gg[MAXD];
-            for (int k = 0; k < d; ++k) {
-                ff[k] = (float)f[k];
-                gg[k] = 1.f - ff[k];
-            }
-            const float qs = (float)qscale;
-            for (int c = 0; c < ncorner; ++c) {
-                long long idx = base;
-                for (int k = 0; k < d; ++k) idx += ((c >> k) & 1) * stride[k];
-                atomicAdd(jb.fix + idx, corner_fixed(d, c, ff, gg, qs));
-            }
-        }
-        if (nout) atomicAdd(jb.outside, nout);
-    } else if (phase == 1) {
-        const double unit = 1.0 / qscale;
-        const long long c0 = b * kCellsPerBlock;
-        const long long c1 = c0 + kCellsPerBlock < jb.ncells ? c0 + kCellsPerBlock : jb.ncells;
-        for (long long c = c0 + threadIdx.x; c < c1; c += blockDim.x) jb.counts[c] = (float)((double)jb.fix[c] * unit);
-    } else {
-        // covariance in one pass, shifted by the grid's centre (as
-        // k_moments_shifted): block b of mblk takes the points i = b, b + mblk,
-        // ... in steps of blockDim
-        const int nv = d + d * d;
-        double acc[MAXD + MAXD * MAXD];
-        for (int v = 0; v < nv; ++v) acc[v] = 0.0;
-        for (long long i = b * blockDim.x + threadIdx.x; i < jb.n; i += (long long)jb.mblk * blockDim.x) {
-            double x[MAXD];
-            for (int k = 0; k < d; ++k) x[k] = jb.X[i * d + k] - jb.shift[k];
-            for (int k = 0; k < d; ++k) acc[k] += x[k];
-            for (int a = 0; a < d; ++a)
-                for (int c = 0; c < d; ++c) acc[d + a * d + c] += x[a] * x[c];
-        }
-        __shared__ double red[8][MAXD + MAXD * MAXD];
-        for (int v = 0; v < nv; ++v) {
-            double t = acc[v];
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][v] = t;
-        }
-        __syncthreads();
-        if (threadIdx.x < nv) {
-            double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
-            jb.part[b * nv + threadIdx.x] = t;
-        }
+    bin_pass<D, 0, unsigned long long>(jb.X, jb.n, b * blockDim.x, (long long)jb.mblk * blockDim.x, jb.ax, jb.shift,
+                                       jb.fix, jb.outside, qscale, jb.part + b * (D + D * D));
+}
+
+__global__ void __launch_bounds__(256) k_fix_many(const BinJob* __restrict__ jobs, int njobs, float unit) {
+    const BinJob& jb = jobs[job_of_warp(njobs, blockIdx.x, [&](int k) { return jobs[k].blk1; })];
+    const long long c0 = ((long long)blockIdx.x - jb.blk1) * kCellsPerBlock;
+    const long long c1 = c0 + kCellsPerBlock < jb.ncells ? c0 + kCellsPerBlock : jb.ncells;
+#pragma unroll
+    for (int r = 0; r < kCellsPerBlock / 1024; ++r) {
+        const long long c = c0 + 4LL * (r * 256 + threadIdx.x);
+        if (c < c1) fix_cells(jb.fix, jb.counts, c, c1, unit);
     }
 }
 
-cudaError_t launch_bin_many(BinJob* jobs_h, BinJob* jobs_d, int n, int phase, double qscale, cudaStream_t st) {
+cudaError_t launch_bin_many(BinJob* jobs_h, BinJob* jobs_d, int n, int d, double qscale, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    long long blocks = 0;
+    long long b0 = 0, b1 = 0;
     for (int k = 0; k < n; ++k) {
         BinJob& jb = jobs_h[k];
-        jb.blk0 = blocks;
-        if (phase == 0)
-            blocks += (jb.n + kBinPtsPerBlock - 1) / kBinPtsPerBlock;
-        else if (phase == 1)
-            blocks += (jb.ncells + kCellsPerBlock - 1) / kCellsPerBlock;
-        else
-            blocks += jb.mblk;
+        jb.blk0 = b0;
+        jb.blk1 = b1;
+        b0 += jb.mblk;
+        b1 += (jb.ncells + kCellsPerBlock - 1) / kCellsPerBlock;
     }
-    if (blocks <= 0) return cudaSuccess;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    if (b0 <= 0 || b1 <= 0 || b0 > 0x7fffffffLL || b1 > 0x7fffffffLL) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemcpyAsync(jobs_d, jobs_h, sizeof(BinJob) * n, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
-    k_bin_many<<<(unsigned)blocks, 256, 0, st>>>(jobs_d, n, phase, qscale);
+    switch (d) {
+        case 1: k_bin_many<1><<<(unsigned)b0, 256, 0, st>>>(jobs_d, n, qscale); break;
+        case 2: k_bin_many<2><<<(unsigned)b0, 256, 0, st>>>(jobs_d, n, qscale); break;
+        case 3: k_bin_many<3><<<(unsigned)b0, 256, 0, st>>>(jobs_d, n, qscale); break;
+        case 4: k_bin_many<4><<<(unsigned)b0, 256, 0, st>>>(jobs_d, n, qscale); break;
+        default: return cudaErrorInvalidValue;
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_fix_many<<<(unsigned)b1, 256, 0, st>>>(jobs_d, n, (float)(1.0 / qscale));
     return cudaGetLastError();
+}
+
+template <int D>
+static cudaError_t prepare_bin_d() {
+    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_bin<D, 0, unsigned long long>, at, kBinSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_bin<D, 1, double>, at, kBinSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_bin<D, 2, int>, at, kBinSmem);
+    return e;
 }
 
 cudaError_t prepare_binning() {
-    cudaError_t e = cudaFuncSetAttribute(k_bin_linear<unsigned long long>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_bin_linear<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    cudaError_t e = prepare_bin_d<1>();
+    if (e == cudaSuccess) e = prepare_bin_d<2>();
+    if (e == cudaSuccess) e = prepare_bin_d<3>();
+    if (e == cudaSuccess) e = prepare_bin_d<4>();
+    return e;
 }
 
-template cudaError_t launch_bin_linear<unsigned long long>(const double*, long long, const GridDesc&,
-                                                           unsigned long long*, long long, unsigned long long*, double,
-                                                           int, cudaStream_t);
-template cudaError_t launch_bin_linear<double>(const double*, long long, const GridDesc&, double*, long long,
-                                               unsigned long long*, double, int, cudaStream_t);
 template cudaError_t launch_int_to_real<float>(const int*, float*, long long, cudaStream_t);
 template cudaError_t launch_int_to_real<double>(const int*, double*, long long, cudaStream_t);
 

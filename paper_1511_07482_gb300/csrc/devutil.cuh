@@ -86,6 +86,24 @@ struct dcplx {
     dflt x, y;
 };
 
+// The job whose block range holds block b, from the jobs' first blocks
+// (ascending, first(0) = 0): every warp searches for itself, 32 places at a
+// time (two rounds for 1024 jobs instead of ten dependent loads).
+template <typename F>
+__device__ __forceinline__ int job_of_warp(int n, long long b, F&& first) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, len = n;
+    while (len > 1) {
+        const int step = (len + 31) >> 5;
+        const int at = lane * step;
+        const bool before = at < len && first(lo + at) <= b;
+        const int k = __popc(__ballot_sync(0xffffffffu, before)) - 1;
+        lo += k * step;
+        len = min(step, len - k * step);
+    }
+    return lo;
+}
+
 // per-thread accumulator of the spectral sums: DFloat in FP32 mode, double in FP64 mode
 template <typename real>
 struct SumAcc;

@@ -388,49 +388,59 @@ struct GridDesc {
     long long M[MAXD];
 };
 
-// acc = double (FP64 atomics) or unsigned long long (fixed point: each
-// weight is added as round(w * qscale))
-template <typename acc>
-cudaError_t launch_bin_linear(const double* X, long long n, const GridDesc& g, acc* counts, long long ncells,
-                              unsigned long long* outside, double qscale, int nsm, cudaStream_t st);
-// dst[i] = (float)(src[i] * unit)
-cudaError_t launch_fix_to_f32(const unsigned long long* src, float* dst, long long n, double unit, cudaStream_t st);
-cudaError_t launch_bin_simple(const double* X, long long n, const GridDesc& g, int* counts, long long ncells,
-                              unsigned long long* outside, int nsm, cudaStream_t st);
-template <typename real>
-cudaError_t launch_int_to_real(const int* src, real* dst, long long n, cudaStream_t st);
-cudaError_t launch_f32_to_f64(const float* src, double* dst, long long n, cudaStream_t st);
-// Batched binning of many datasets (FP32 linear binning in fixed point):
-// one launch per phase over a job table, each CTA within one job.
-//   phase 0: bin the points into the job's fixed-point accumulators
-//            (fix, zeroed by the caller) and count the outside points;
-//   phase 1: convert the accumulators to FP32 counts;
-//   phase 2: the job's mblk block partials of the coordinate sums (mean
-//            pass) or, phase 3, of the centred products (mean given).
-struct BinJob {
-    const double* X;
-    long long n, ncells;
-    GridDesc g;
-    unsigned long long* fix;
-    float* counts;
-    unsigned long long* outside;
-    double* part;          // phase 2: mblk x (d + d^2) sums of x - shift and (x - shift)(x - shift)^T
-    double shift[MAXD];    // phase 2: the grid's centre
-    int mblk;
-    long long blk0;        // set by the launcher
+// What a binning pass needs of a grid (bin_axes): the bounds as
+// order-preserving integers, the last base cell M - 2, cell strides.
+struct BinAxes {
+    double lo[MAXD], inv[MAXD], delta[MAXD];
+    long long klo[MAXD], khi[MAXD];
+    int top[MAXD];
+    unsigned int stride[MAXD];
 };
-cudaError_t launch_bin_many(BinJob* jobs_h, BinJob* jobs_d, int n, int phase, double qscale, cudaStream_t st);
-// one-time kernel attributes of the binning launches (before any graph capture)
-cudaError_t prepare_binning();
-
-// blocks of the moment launches (at most two per SM)
-int moments_blocks(long long n, int nsm);
-// one pass: per block b, out[b (d + d^2) + k] = sum of x_k - s_k and
-// out[b (d + d^2) + d + a d + c] = sum of (x_a - s_a)(x_c - s_c)
+void bin_axes(const GridDesc& g, BinAxes& ax);
 struct Shift {
     double s[MAXD];
 };
-cudaError_t launch_moments_shifted(const double* X, long long n, int d, const Shift& sh, double* out, int nsm,
-                                   cudaStream_t st);
+// One pass over the sample: its counts (zeroed by the caller), and for each
+// of the bin_blocks(n, nsm) blocks b at part + b (d + d^2) the sums of
+// x_k - s_k and (x_a - s_a)(x_c - s_c) of the block's points.
+//   fixed:  linear binning, each weight added as round(w * qscale)
+//   f64:    linear binning, FP64 atomics
+//   simple: whole points to their nearest node
+int bin_blocks(long long n, int nsm);
+cudaError_t launch_bin_fixed(const double* X, long long n, const GridDesc& g, const Shift& sh,
+                             unsigned long long* counts, long long ncells, unsigned long long* outside, double qscale,
+                             double* part, int nsm, cudaStream_t st);
+cudaError_t launch_bin_f64(const double* X, long long n, const GridDesc& g, const Shift& sh, double* counts,
+                           long long ncells, unsigned long long* outside, double* part, int nsm, cudaStream_t st);
+cudaError_t launch_bin_simple(const double* X, long long n, const GridDesc& g, const Shift& sh, int* counts,
+                              long long ncells, unsigned long long* outside, double* part, int nsm, cudaStream_t st);
+// dst[i] = (float)src[i] * unit (a power of two); also *outside_copy = *outside.
+// src and dst 16-byte aligned.
+cudaError_t launch_fix_to_f32(const unsigned long long* src, float* dst, long long n, double unit,
+                              const unsigned long long* outside, unsigned long long* outside_copy, int nsm,
+                              cudaStream_t st);
+template <typename real>
+cudaError_t launch_int_to_real(const int* src, real* dst, long long n, cudaStream_t st);
+cudaError_t launch_f32_to_f64(const float* src, double* dst, long long n, cudaStream_t st);
+// Batched binning of many datasets (FP32 linear binning in fixed point): two
+// launches over a job table, each CTA within one job.  The first bins the
+// points into the job's fixed-point accumulators (fix, zeroed by the caller),
+// counts the outside points and writes the job's mblk block partials of the
+// moments; the second converts the accumulators to FP32 counts.
+struct BinJob {
+    const double* X;
+    long long n, ncells;
+    BinAxes ax;
+    unsigned long long* fix;   // 16-byte aligned, as counts
+    float* counts;
+    unsigned long long* outside;
+    double* part;              // mblk x (d + d^2) sums of x - shift and (x - shift)(x - shift)^T
+    double shift[MAXD];        // the grid's centre
+    int mblk;
+    long long blk0, blk1;      // first block in each launch, set by the launcher
+};
+cudaError_t launch_bin_many(BinJob* jobs_h, BinJob* jobs_d, int n, int d, double qscale, cudaStream_t st);
+// one-time kernel attributes of the binning launches (before any graph capture)
+cudaError_t prepare_binning();
 
 }  // namespace kdefft
