@@ -618,10 +618,6 @@ struct kdefft_ctx_s {
     HostBuf h_binres;         // pinned outside count and moment partials of a binning
     cudaEvent_t acjobs_ev = nullptr;
     bool acjobs_free = true;
-    DevBuf specjobs;          // job table of the FP32-pair count-spectrum passes
-    HostBuf h_specjobs;       // its pinned staging copy, free once specjobs_ev has passed
-    cudaEvent_t specjobs_ev = nullptr;
-    bool specjobs_free = true;
     DevBuf binjobs;           // job tables of the batched binning
     DevBuf kdebuf;            // stencil table / outputs of the grid estimate and the mixture term
     std::map<std::string, KStat> kstat;
@@ -1954,28 +1950,6 @@ static int ensure_spectra(kdefft_ctx c, const std::vector<std::pair<kdefft_ds, s
 
 // Evaluate every grid of rs (value = Eq. 25 for that lag kernel).
 // ============================================================ lag-domain engine
-static long long pmin_smooth(long long m) { return next_smooth(m); }
-
-// a_j = sum_i c_i c_{i+j} on the half box A (j_0 in [0, A_0], |j_k| <= A_k),
-// layout [j_{d-1}]..[j_0], from the FP64 count spectrum at P_k >= M_k + A_k
-// (no aliasing on the box) by separable pruned inverse DFTs in FP64; the
-// last pass also writes the FP32 copy.  A box grows (by half of itself at
-// least) when a request needs more.  Every dataset of `req` is brought up to
-// date with one batched spectrum launch sequence and stream-ordered passes
-// through context buffers (no synchronisation).
-// lines per CTA of an autocorrelation pass of length P over `lines` lines:
-// as many as fit 96 KB of shared memory (two resident CTAs per SM), but no
-// more than leave two CTAs per SM busy; at least one
-static int acorr_lines(int P, long long lines, int nsm) {
-    int nl = 1;
-    while (nl < 64 && acorr_smem_bytes(P, nl + 1) <= (size_t)96 * 1024) ++nl;
-    const long long spread = std::max<long long>(1, lines / (2LL * nsm));
-    return (int)std::min<long long>(nl, spread);
-}
-
-// Cache key of a count spectrum held as FP32 pairs (the autocorrelation input
-// of FP32 datasets): element size 8 as for FP64, told apart by this tag.
-static constexpr size_t kPairTag = 9;
 // Largest radix of the FP32-pair transforms.  A pair butterfly is a long
 // chain of dependent FP32 operations, so small radices (more threads busy
 // per stage, shorter chains) win: measured for the count spectrum and
@@ -1983,130 +1957,6 @@ static constexpr size_t kPairTag = 9;
 // to 5, 55 µs up to 8, 84 µs up to 16 (the FP64 passes: 81 µs); 128^3 at
 // P = 180 (n = 1e6): 405, 406, 494 µs (FP64: 921 µs).
 static constexpr int kPairRadix = 5;
-
-// |F(c_zp)|^2 at padded P for FP32 datasets, in FP32-pair arithmetic: d
-// forward passes of k_spec_df per dataset, one launch per pass level for
-// every dataset of a dimension.  The first level transforms the last axis
-// of the FP32 counts (half spectrum), the middle levels the interior axes,
-// the last level axis 0 and writes |X|^2 in the spectrum layout
-// [w_{d-1}]..[w_1][w_0] that the autocorrelation passes read.  Intermediate
-// lines go through the context's two pass buffers (stream-ordered reuse).
-// The launches of a batch of FP32-pair count-spectrum passes, whose job table
-// is already on its way to the device: issued by the caller (in one graph
-// with the autocorrelation passes that read the spectra).
-struct SpecLaunches {
-    SpecJob* jd = nullptr;
-    size_t table_bytes = 0;   // the job table, in h_specjobs until the caller's copy
-    struct L {
-        size_t slot;
-        int n;
-        long long blocks;
-        size_t sm;
-    };
-    std::vector<L> lv;
-    double by = 0.0, fl = 0.0;
-};
-
-static int ensure_spectra_df(kdefft_ctx c, const std::vector<std::pair<kdefft_ds, std::array<int, 4>>>& need,
-                             SpecLaunches& sl) {
-    struct Sj {
-        kdefft_ds ds;
-        std::array<int, 4> P;
-        std::vector<int> key;
-        std::shared_ptr<DevBuf> buf;
-        long long E[MAXD];   // frequencies kept per axis: P_k, the half spectrum on the last axis
-        size_t off, most;
-    };
-    std::vector<Sj> todo;
-    std::set<std::pair<kdefft_ds, std::vector<int>>> queued;
-    for (const auto& np : need) {
-        kdefft_ds ds = np.first;
-        std::vector<int> key = spectrum_key(ds, np.second.data(), kPairTag);
-        if (ds->spectra.count(key) || queued.count({ds, key})) continue;
-        queued.insert({ds, key});
-        Sj j{ds, np.second, key, std::make_shared<DevBuf>(&c->cache), {0, 0, 0, 0}, 0, 0};
-        KCHK(j.buf->ensure(sizeof(double) * spec_elems(ds->d, np.second.data())));
-        todo.push_back(std::move(j));
-    }
-    if (todo.empty()) return KDEFFT_OK;
-    size_t pool = 0;
-    for (Sj& j : todo) {
-        const int d = j.ds->d;
-        for (int k = 0; k < d; ++k) {
-            j.E[k] = (k == d - 1) ? j.P[k] / 2 + 1 : j.P[k];
-            twiddle_offset(c, j.P[k]);
-        }
-        // the largest intermediate: after the pass on axis k (k >= 1), the
-        // untransformed axes m < k hold M_m values and the others E_m
-        j.most = 0;
-        for (int k = d - 1; k >= 1; --k) {
-            long long e = 1;
-            for (int m = 0; m < d; ++m) e *= (m < k) ? j.ds->M[m] : j.E[m];
-            j.most = std::max(j.most, (size_t)e);
-        }
-        j.off = pool;
-        pool += (j.most + 1) & ~(size_t)1;
-    }
-    KCHK(sync_twiddles(c));
-    KCHK(c->acbuf[0].ensure(sizeof(double2) * std::max<size_t>(pool, 1)));
-    KCHK(c->acbuf[1].ensure(sizeof(double2) * std::max<size_t>(pool, 1)));
-    double2* pools[2] = {(double2*)c->acbuf[0].p, (double2*)c->acbuf[1].p};
-    std::vector<SpecJob> all;
-    std::vector<SpecLaunches::L>& lv = sl.lv;
-    double& fl = sl.fl;
-    double& by = sl.by;
-    for (int dim = 1; dim <= MAXD; ++dim) {
-        std::vector<size_t> sel;
-        for (size_t u = 0; u < todo.size(); ++u)
-            if (todo[u].ds->d == dim) sel.push_back(u);
-        if (sel.empty()) continue;
-        for (int lev = 0; lev < dim; ++lev) {
-            const int k = dim - 1 - lev;   // the axis of this level
-            const size_t slot = all.size();
-            all.resize(slot + sel.size());
-            for (size_t v = 0; v < sel.size(); ++v) {
-                const Sj& j = todo[sel[v]];
-                kdefft_ds ds = j.ds;
-                SpecJob& a = all[slot + v];
-                std::memset(&a, 0, sizeof(a));
-                a.d = dim;
-                a.in_f = (lev == 0) ? (const float*)ds->counts.p : nullptr;
-                a.in_c = (lev == 0) ? nullptr : (const void*)(pools[(lev - 1) & 1] + j.off);
-                long long O = 1, I = 1;
-                for (int m = 0; m < k; ++m) O *= ds->M[m];
-                for (int m = k + 1; m < dim; ++m) I *= j.E[m];
-                a.O = O;
-                a.I = I;
-                a.X = (int)ds->M[k];
-                a.Y = (int)j.E[k];
-                if (k == 0) {
-                    a.out_s = j.buf->p;
-                    for (int m = 1; m < dim; ++m) a.ext[m] = (int)j.E[m];
-                } else {
-                    a.out_c = (void*)(pools[lev & 1] + j.off);
-                }
-                a.ap.tw_off = twiddle_offset(c, j.P[k]);
-                if (!radix_plan(j.P[k], a.ap, kPairRadix)) return fail(KDEFFT_ERR_UNSUPPORTED, "no radix plan for P");
-                a.nl = acorr_lines(j.P[k], O * I, c->nsm);
-                fl += 5.0 * j.P[k] * std::log2((double)j.P[k]) * (double)(O * I);
-                by += (lev == 0 ? 4.0 : 16.0) * (double)(O * I) * a.X + (k == 0 ? 8.0 : 16.0) * (double)(O * I) * a.Y;
-            }
-            SpecLaunches::L L{slot, (int)sel.size(), 0, 0};
-            KCU(spec_plan(all.data() + slot, L.n, &L.blocks, &L.sm));
-            lv.push_back(L);
-        }
-    }
-    KCHK(c->specjobs.ensure(sizeof(SpecJob) * all.size()));
-    if (!c->specjobs_free) KCU(cudaEventSynchronize(c->specjobs_ev));
-    KCHK(c->h_specjobs.ensure(sizeof(SpecJob) * all.size()));
-    std::memcpy(c->h_specjobs.p, all.data(), sizeof(SpecJob) * all.size());
-    sl.jd = (SpecJob*)c->specjobs.p;
-    sl.table_bytes = sizeof(SpecJob) * all.size();
-    // the spectra are registered now; the caller copies the table up and
-    // issues the passes before any launch that reads them
-    for (Sj& j : todo) j.ds->spectra[j.key] = j.buf;
-    return KDEFFT_OK;
-}
 
 // Work that follows the autocorrelation passes on the stream (the device
 // search): its launch signature and its copies and launches.
@@ -2117,226 +1967,227 @@ struct StreamTail {
     std::function<int()> issue;
 };
 
-// Grow the count autocorrelation of each dataset to the half box it needs
-// (the FP32-pair or FP64 count spectrum first).  With a tail, the tail's work
-// joins the same launch sequence (one graph replay for all of it); it runs on
-// its own when there is nothing to grow.
+// Grow the count autocorrelation of each dataset to the half box it needs:
+// a_j = sum_i c_i c_{i+j} on the half box A (j_0 in [0, A_0], |j_k| <= A_k),
+// layout [j_{d-1}]..[j_0], through the count spectrum at the smallest smooth
+// P_k >= M_k + A_k (no aliasing on the box) by passes along one axis at a time
+// (k_line); the last pass writes FP64 and FP32.  FP32 datasets: FP32 pairs
+// (about 44 bits, on the FP32 pipes) from the FP32 counts, last axis first,
+// axis 0 forward and back in one pass, then the other axes back.  FP64
+// datasets: the inverse passes from the FP64 count spectrum.  A box grows (by
+// half of itself at least) when a request needs more.  Every dataset of `req`
+// goes through one launch per pass level and dimension, on the stream through
+// the context's two pass buffers (no synchronisation).  With a tail, the
+// tail's work joins the same launch sequence (one graph replay for all of
+// it); it runs on its own when there is nothing to grow.
 static int ensure_autocorr_many(kdefft_ctx c, const std::vector<std::pair<kdefft_ds, std::array<int, 4>>>& req,
                                 StreamTail* tail = nullptr) {
     HostTimer ht(c, "host:acorr");
     struct Job {
         kdefft_ds ds;
         int A[4], P[4];
+        long long E[4];    // frequencies kept per axis: P_k, the half spectrum on the last axis
+        const double* S;   // FP64 datasets: the count spectrum
+        size_t off;        // offset in the pass buffers (complex elements)
+        double ptot;
     };
     std::vector<Job> jobs;
-    std::vector<std::pair<kdefft_ds, std::array<int, 4>>> specs, specs_df;
+    std::vector<std::pair<kdefft_ds, std::array<int, 4>>> specs;
     for (const auto& rq : req) {
         kdefft_ds ds = rq.first;
         const int d = ds->d;
         bool covered = ds->acA[0] >= 0;
         for (int k = 0; k < d; ++k) covered = covered && ds->acA[k] >= rq.second[k];
         if (covered) continue;
-        Job jb{ds, {0, 0, 0, 0}, {1, 1, 1, 1}};
+        Job jb{ds, {0, 0, 0, 0}, {1, 1, 1, 1}, {1, 1, 1, 1}, nullptr, 0, 1.0};
         for (int k = 0; k < d; ++k) {
             const int grow = ds->acA[k] >= 0 ? ds->acA[k] + ds->acA[k] / 2 : 0;
             jb.A[k] = (int)std::min<long long>(ds->M[k] - 1, std::max(rq.second[k], grow));
-            jb.P[k] = (int)pmin_smooth(ds->M[k] + jb.A[k]);
+            jb.P[k] = (int)next_smooth(ds->M[k] + jb.A[k]);
             if (jb.P[k] > MAXP) return KDEFFT_ERR_UNSUPPORTED;
+            jb.E[k] = (k == d - 1) ? jb.P[k] / 2 + 1 : jb.P[k];
+            jb.ptot *= jb.P[k];
         }
         jobs.push_back(jb);
-        (ds->opts.precision == KDEFFT_FP64 ? specs : specs_df).push_back({ds, {jb.P[0], jb.P[1], jb.P[2], jb.P[3]}});
+        if (ds->opts.precision == KDEFFT_FP64) specs.push_back({ds, {jb.P[0], jb.P[1], jb.P[2], jb.P[3]}});
     }
-    // FP64 datasets: the FP64 transforms; FP32 datasets: FP32 pairs (about 44
-    // bits, on the FP32 pipes), far beyond their FP32 counts' own rounding
     if (!specs.empty()) KCHK(ensure_spectra<double>(c, specs));
-    SpecLaunches sl;
-    if (!specs_df.empty()) KCHK(ensure_spectra_df(c, specs_df, sl));
     for (const Job& jb : jobs)
         for (int k = 0; k < jb.ds->d; ++k) twiddle_offset(c, jb.P[k]);
     KCHK(sync_twiddles(c));
-    const double2* tw = (const double2*)c->tw64.p;
-    // Per dataset, the sizes of its passes; pass buffers at offsets in the
-    // two context pools; then every pass level is one launch over all
-    // datasets of that dimension (level k transforms axis k: [w_{d-1} ..
-    // w_{k+1}][w_k][j_{k-1} .. j_0] -> [..][j_k][..]; the last level is the
-    // half-spectrum axis, written as real FP64 and FP32).
-    struct Plan {
-        const double* S;
-        long long O0;      // rows of the innermost pass
-        size_t most;       // complex elements of the largest intermediate
-        size_t off;        // offset in the pools
-        double ptot;
-        int Q;
-    };
-    std::vector<Plan> plan(jobs.size());
     size_t pool = 0;
-    double fl = 0.0, by = 0.0;
-    for (size_t u = 0; u < jobs.size(); ++u) {
-        const Job& jb = jobs[u];
+    for (Job& jb : jobs) {
         kdefft_ds ds = jb.ds;
         const int d = ds->d;
-        const int* A = jb.A;
-        const int* P = jb.P;
         const bool pairs = ds->opts.precision != KDEFFT_FP64;
-        auto sit = ds->spectra.find(spectrum_key(ds, P, pairs ? kPairTag : sizeof(double)));
-        if (sit == ds->spectra.end()) return fail(KDEFFT_ERR_CUDA, "count spectrum missing");
-        Plan& pl = plan[u];
-        pl.S = (const double*)sit->second->p;
-        pl.Q = P[d - 1] / 2 + 1;
-        pl.ptot = 1.0;
-        long long nbox = 1;
-        for (int k = 0; k < d; ++k) {
-            nbox *= (k == 0) ? (A[0] + 1) : (2 * A[k] + 1);
-            pl.ptot *= P[k];
+        if (!pairs) {
+            auto sit = ds->spectra.find(spectrum_key(ds, jb.P, sizeof(double)));
+            if (sit == ds->spectra.end()) return fail(KDEFFT_ERR_CUDA, "count spectrum missing");
+            jb.S = (const double*)sit->second->p;
         }
+        long long nbox = 1;
+        for (int k = 0; k < d; ++k) nbox *= (k == 0) ? (jb.A[0] + 1) : (2 * jb.A[k] + 1);
         KCHK(ds->ac64.ensure(sizeof(double) * nbox));
         KCHK(ds->ac32.ensure(sizeof(float) * nbox));
-        pl.O0 = pl.Q;
-        for (int k = 1; k <= d - 2; ++k) pl.O0 *= P[k];
-        pl.most = 0;
-        {
-            // a length-P complex transform per line: 5 P log2 P flops
-            long long o = pl.O0, ii = 1;
-            for (int k = 0; k < d - 1; ++k) {
-                const int J = (k == 0) ? A[0] + 1 : 2 * A[k] + 1;
-                pl.most = std::max(pl.most, (size_t)(o * J * ii));
-                fl += 5.0 * P[k] * std::log2((double)P[k]) * (double)(o * ii);
-                ii *= J;
-                if (k + 1 <= d - 2) o /= P[k + 1];
+        // the largest intermediate: forward, axes m < k hold M_m values and
+        // the others E_m; back, axes m <= k hold lags and the others E_m
+        long long most = 1;
+        if (pairs)
+            for (int k = d - 1; k >= 1; --k) {
+                long long e = 1;
+                for (int m = 0; m < d; ++m) e *= (m < k) ? ds->M[m] : jb.E[m];
+                most = std::max(most, e);
             }
-            fl += 5.0 * P[d - 1] * std::log2((double)P[d - 1]) * (double)ii;
+        for (int k = 0; k < d - 1; ++k) {
+            long long e = 1;
+            for (int m = 0; m < d; ++m) e *= (m > k) ? jb.E[m] : (m == 0 ? jb.A[0] + 1 : 2 * jb.A[m] + 1);
+            most = std::max(most, e);
         }
-        pl.off = pool;
-        pool += (pl.most + 1) & ~(size_t)1;
-        double b = 8.0 * pl.Q;
-        for (int k = 0; k < d - 1; ++k) b *= P[k];
-        by += b;
+        jb.off = pool;
+        pool += (size_t)((most + 1) & ~1LL);
     }
     if (!jobs.empty()) {
         KCHK(c->acbuf[0].ensure(sizeof(double2) * std::max<size_t>(pool, 1)));
         KCHK(c->acbuf[1].ensure(sizeof(double2) * std::max<size_t>(pool, 1)));
-        // one table slice per launch (at most MAXD launches per dataset); all
-        // slices go up in one copy from pinned memory, so that the host does
-        // not wait for the stream (a pageable copy would)
-        KCHK(c->acjobs.ensure(sizeof(AcorrJob) * jobs.size() * MAXD));
-        AcorrJob* jd = (AcorrJob*)c->acjobs.p;
-        double2* pool0 = (double2*)c->acbuf[0].p;
-        double2* pool1 = (double2*)c->acbuf[1].p;
-        std::vector<AcorrJob> all;
+        double2* pools[2] = {(double2*)c->acbuf[0].p, (double2*)c->acbuf[1].p};
+        // one table slice per launch; all slices go up in one copy from pinned
+        // memory, so that the host does not wait for the stream (a pageable
+        // copy would)
+        std::vector<LineJob> all;
         struct Launch {
+            int kind;
             size_t slot;
             int n;
             long long blocks;
             size_t sm;
-            bool pairs;   // FP32-pair passes (FP32 datasets)
+            int threads;
+            bool pairs;
+            double by, fl;
         };
         std::vector<Launch> lv;
         for (int pr = 0; pr < 2; ++pr)
-        for (int dim = 1; dim <= MAXD; ++dim) {
-            std::vector<size_t> sel;
-            for (size_t u = 0; u < jobs.size(); ++u)
-                if (jobs[u].ds->d == dim && (jobs[u].ds->opts.precision != KDEFFT_FP64) == (pr == 1)) sel.push_back(u);
-            if (sel.empty()) continue;
-            // level k of every selected dataset
-            std::vector<long long> O(sel.size()), I(sel.size(), 1);
-            for (size_t v = 0; v < sel.size(); ++v) O[v] = plan[sel[v]].O0;
-            for (int k = 0; k < dim; ++k) {
-                const bool last = (k == dim - 1);
-                const size_t slot = all.size();
-                all.resize(slot + sel.size());
-                for (size_t v = 0; v < sel.size(); ++v) {
-                    const Job& jb = jobs[sel[v]];
-                    const Plan& pl = plan[sel[v]];
-                    AcorrJob& a = all[slot + v];
-                    std::memset(&a, 0, sizeof(a));
-                    // ping-pong: level k reads pool (k+1)&1, writes pool k&1
-                    double2* rd = ((k & 1) ? pool0 : pool1) + pl.off;
-                    double2* wr = ((k & 1) ? pool1 : pool0) + pl.off;
-                    a.in_r = (k == 0) ? pl.S : nullptr;
-                    a.in_c = (k == 0) ? nullptr : rd;
-                    a.O = last ? 1 : O[v];
-                    a.I = I[v];
-                    a.W = last ? pl.Q : jb.P[k];
-                    a.J = (k == 0) ? jb.A[0] + 1 : 2 * jb.A[k] + 1;
-                    a.jlo = (k == 0) ? 0 : -jb.A[k];
-                    a.ap.tw_off = twiddle_offset(c, jb.P[k]);
-                    if (!radix_plan(jb.P[k], a.ap, pr == 1 ? kPairRadix : 16))
-                        return fail(KDEFFT_ERR_UNSUPPORTED, "no radix plan for P");
-                    a.nl = acorr_lines(jb.P[k], a.O * a.I, c->nsm);
-                    a.half = last ? 1 : 0;
-                    a.scale = last ? 1.0 / pl.ptot : 1.0;
-                    if (last) {
-                        a.out_r = (double*)jb.ds->ac64.p;
-                        a.out_r32 = (float*)jb.ds->ac32.p;
-                    } else {
-                        a.out_c = wr;
+            for (int dim = 1; dim <= MAXD; ++dim) {
+                const bool pairs = pr == 1;
+                std::vector<size_t> sel;
+                for (size_t u = 0; u < jobs.size(); ++u)
+                    if (jobs[u].ds->d == dim && (jobs[u].ds->opts.precision != KDEFFT_FP64) == pairs) sel.push_back(u);
+                if (sel.empty()) continue;
+                // pairs: forward along axes dim - 1 .. 1, axis 0, back along
+                // 1 .. dim - 1; FP64: back along 0 .. dim - 1.  Step s reads
+                // pass buffer (s + 1) & 1 and writes s & 1.
+                const int steps = pairs ? 2 * dim - 1 : dim;
+                for (int s = 0; s < steps; ++s) {
+                    const int back = pairs ? s - (dim - 1) : s;   // axis of an inverse pass (0: Axis0), below 0 forward
+                    const int k = back >= 0 ? back : dim - 1 - s;
+                    const bool last = s == steps - 1;
+                    const int kind = back < 0             ? (s == 0 ? kLineRealRows : kLineForward)
+                                     : (pairs && back == 0) ? kLineAxis0
+                                     : last               ? kLineLast
+                                     : back == 0          ? kLineSpecRows
+                                                          : kLineInverse;
+                    Launch L{kind, all.size(), (int)sel.size(), 0, 0, 0, pairs, 0.0, 0.0};
+                    all.resize(L.slot + sel.size());
+                    long long lines = 0;
+                    for (size_t v = 0; v < sel.size(); ++v) {
+                        const Job& jb = jobs[sel[v]];
+                        kdefft_ds ds = jb.ds;
+                        LineJob& a = all[L.slot + v];
+                        std::memset(&a, 0, sizeof(a));
+                        a.d = dim;
+                        a.in = pools[(s + 1) & 1] + jb.off;
+                        if (back < 0) {
+                            a.O = a.I = 1;
+                            for (int m = 0; m < k; ++m) a.O *= ds->M[m];
+                            for (int m = k + 1; m < dim; ++m) a.I *= jb.E[m];
+                            a.X = (int)ds->M[k];
+                            a.Y = (int)jb.E[k];
+                        } else {
+                            a.O = a.I = 1;
+                            if (kind == kLineAxis0)
+                                for (int m = 1; m < dim; ++m) a.I *= jb.E[m];
+                            else {
+                                for (int m = k + 1; m < dim; ++m) a.O *= jb.E[m];
+                                for (int m = 0; m < k; ++m) a.I *= (m == 0) ? jb.A[0] + 1 : 2 * jb.A[m] + 1;
+                            }
+                            a.X = kind == kLineAxis0 ? (int)ds->M[0] : (int)jb.E[k];
+                            a.Y = (k == 0) ? jb.A[0] + 1 : 2 * jb.A[k] + 1;
+                            a.ylo = (k == 0) ? 0 : -jb.A[k];
+                            for (int m = 1; m < dim; ++m) a.ext[m] = (int)jb.E[m];
+                        }
+                        if (pairs && s == 0) a.in_f = (const float*)ds->counts.p;
+                        if (!pairs && s == 0) {
+                            a.in = jb.S;
+                            a.in_real = dim == 1;
+                        }
+                        if (last) {
+                            a.out_r = (double*)ds->ac64.p;
+                            a.out_r32 = (float*)ds->ac32.p;
+                            a.scale = 1.0 / jb.ptot;
+                        } else {
+                            a.out = pools[s & 1] + jb.off;
+                        }
+                        a.ap.tw_off = twiddle_offset(c, jb.P[k]);
+                        if (!radix_plan(jb.P[k], a.ap, pairs ? kPairRadix : 16))
+                            return fail(KDEFFT_ERR_UNSUPPORTED, "no radix plan for P");
+                        lines += a.O * a.I;
+                        // 5 P log2 P flops per complex transform
+                        const double ntr = (double)(a.O * a.I) * (kind == kLineAxis0  ? 1.5
+                                                                  : kind == kLineForward || kind == kLineInverse ? 1.0
+                                                                                                                 : 0.5);
+                        L.fl += 5.0 * jb.P[k] * std::log2((double)jb.P[k]) * ntr;
+                        L.by += (double)(a.O * a.I) *
+                                ((kind == kLineRealRows ? 4.0 : kind == kLineSpecRows ? 8.0 : 16.0) * a.X +
+                                 (last ? 12.0 : 16.0) * a.Y);
                     }
-                }
-                Launch L{slot, (int)sel.size(), 0, 0, pr == 1};
-                KCU(acorr_plan(all.data() + slot, L.n, &L.blocks, &L.sm));
-                lv.push_back(L);
-                for (size_t v = 0; v < sel.size(); ++v) {
-                    const Job& jb = jobs[sel[v]];
-                    const int J = (k == 0) ? jb.A[0] + 1 : 2 * jb.A[k] + 1;
-                    I[v] *= J;
-                    if (k + 1 <= dim - 2) O[v] /= jb.P[k + 1];
+                    for (size_t v = 0; v < sel.size(); ++v)
+                        all[L.slot + v].nl = line_lines(kind, all[L.slot + v].ap.P, lines, c->nsm);
+                    KCU(line_plan(all.data() + L.slot, L.n, kind, &L.blocks, &L.sm, &L.threads));
+                    lv.push_back(L);
                 }
             }
-        }
         for (const Job& jb : jobs)
             for (int k = 0; k < 4; ++k) jb.ds->acA[k] = (k < jb.ds->d) ? jb.A[k] : 0;
         if (!c->acjobs_free) KCU(cudaEventSynchronize(c->acjobs_ev));
-        const size_t acb = sizeof(AcorrJob) * all.size();
+        const size_t acb = sizeof(LineJob) * all.size();
+        KCHK(c->acjobs.ensure(acb));
         KCHK(c->h_acjobs.ensure(acb));
+        LineJob* jd = (LineJob*)c->acjobs.p;
         std::memcpy(c->h_acjobs.p, all.data(), acb);
-        // the table copies, the count-spectrum passes (FP32 datasets), the
-        // autocorrelation passes and the tail in one launch sequence,
-        // replayed as a CUDA graph when its tables, sizes and launch shapes
-        // repeat (the copies read the pinned tables when the graph runs)
-        std::vector<long long> sig = {7, (long long)(uintptr_t)sl.jd, (long long)(uintptr_t)jd,
-                                      (long long)(uintptr_t)c->h_specjobs.p, (long long)sl.table_bytes,
-                                      (long long)(uintptr_t)c->h_acjobs.p, (long long)acb,
-                                      (long long)(uintptr_t)c->twdf.p, (long long)(uintptr_t)tw,
-                                      (long long)sl.lv.size()};
-        for (const auto& L : sl.lv) sig.insert(sig.end(), {(long long)L.slot, L.n, L.blocks, (long long)L.sm});
+        // the table copy, the passes and the tail in one launch sequence,
+        // replayed as a CUDA graph when its table, sizes and launch shapes
+        // repeat (the copy reads the pinned table when the graph runs)
+        std::vector<long long> sig = {7, (long long)(uintptr_t)jd, (long long)(uintptr_t)c->h_acjobs.p, (long long)acb,
+                                      (long long)(uintptr_t)c->twdf.p, (long long)(uintptr_t)c->tw64.p,
+                                      (long long)lv.size()};
         for (const Launch& L : lv)
-            sig.insert(sig.end(), {(long long)L.slot, L.n, L.blocks, (long long)L.sm, L.pairs ? 1 : 0});
+            sig.insert(sig.end(), {L.kind, (long long)L.slot, L.n, L.blocks, (long long)L.sm, L.threads, L.pairs ? 1 : 0});
         if (tail) KCHK(tail->prepare(sig));
         auto issue = [&]() -> int {
-            if (sl.table_bytes)
-                KCU(cudaMemcpyAsync(sl.jd, c->h_specjobs.p, sl.table_bytes, cudaMemcpyHostToDevice, c->stream));
             KCU(cudaMemcpyAsync(jd, c->h_acjobs.p, acb, cudaMemcpyHostToDevice, c->stream));
-            if (!sl.lv.empty()) {
-                cudaEvent_t es = prof_start(c);
+            for (size_t u = 0; u < lv.size();) {   // forward passes and axis 0, then the way back
+                const auto ahead = [](const Launch& L) { return L.kind <= kLineAxis0; };
+                const bool fwd = ahead(lv[u]);
+                cudaEvent_t ev = prof_start(c);
+                double by = 0.0, fl = 0.0;
                 c->launches--;   // counted per launch below
-                for (const auto& L : sl.lv) {
+                for (; u < lv.size() && ahead(lv[u]) == fwd; ++u) {
+                    const Launch& L = lv[u];
                     c->launches++;
-                    KCU(launch_spec_df(sl.jd + L.slot, L.n, L.blocks, L.sm, c->twdf.p, c->stream));
+                    KCU(launch_line(L.kind, L.pairs, jd + L.slot, L.n, L.blocks, L.sm, L.threads,
+                                    L.pairs ? c->twdf.p : c->tw64.p, c->stream));
+                    by += L.by;
+                    fl += L.fl;
                 }
-                prof_stop(c, es, "spec_df", sl.by, sl.fl);
+                prof_stop(c, ev, fwd ? "spec_df" : "acorr", by, fl);
             }
-            cudaEvent_t ev = prof_start(c);
-            c->launches--;   // counted per launch below
-            for (const Launch& L : lv) {
-                c->launches++;
-                if (L.pairs)
-                    KCU(launch_acorr_df(jd + L.slot, L.n, L.blocks, L.sm, c->twdf.p, c->stream));
-                else
-                    KCU(launch_acorr(jd + L.slot, L.n, L.blocks, L.sm, tw, c->stream));
-            }
-            prof_stop(c, ev, "acorr", by, fl);
             if (tail) KCHK(tail->issue());
             return KDEFFT_OK;
         };
         KCHK(run_graph(c, sig, issue));
-        // the pinned tables are free again once this work has run
-        if (sl.table_bytes) {
-            KCU(cudaEventRecord(c->specjobs_ev, c->stream));
-            c->specjobs_free = false;
-        }
+        // the pinned table is free again once this work has run
         KCU(cudaEventRecord(c->acjobs_ev, c->stream));
         c->acjobs_free = false;
-        c->h2d += (int64_t)(sl.table_bytes + acb);
+        c->h2d += (int64_t)acb;
         tail = nullptr;
     }
     if (tail) {
@@ -3161,15 +3012,13 @@ int kdefft_create(kdefft_ctx* out, int device, void* stream) {
     }
     c->nsm = prop.multiProcessorCount;
     for (DevBuf* b : {&c->tw32, &c->tw64, &c->twdf, &c->scratch, &c->partial, &c->items, &c->tiles, &c->out,
-                      &c->sel_buf, &c->binfix, &c->acbuf[0], &c->acbuf[1], &c->acjobs, &c->binjobs, &c->kdebuf,
-                      &c->specjobs})
+                      &c->sel_buf, &c->binfix, &c->acbuf[0], &c->acbuf[1], &c->acjobs, &c->binjobs, &c->kdebuf})
         b->gen = &c->buf_gen;
     c->h_items.gen = &c->buf_gen;
     c->h_out.gen = &c->buf_gen;
     c->h_binres.gen = &c->buf_gen;
     if (cudaEventCreateWithFlags(&c->staging_ev, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->acjobs_ev, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->specjobs_ev, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&c->acjobs_ev, cudaEventDisableTiming) != cudaSuccess) {
         delete c;
         return fail(KDEFFT_ERR_CUDA, "event creation failed");
     }
@@ -3367,9 +3216,7 @@ int kdefft_destroy(kdefft_ctx c) {
     if (c->join_ev) cudaEventDestroy(c->join_ev);
     if (c->staging_ev) cudaEventDestroy(c->staging_ev);
     if (c->acjobs_ev) cudaEventDestroy(c->acjobs_ev);
-    if (c->specjobs_ev) cudaEventDestroy(c->specjobs_ev);
     c->h_acjobs.release();
-    c->h_specjobs.release();
     c->h_sel.release();
     c->h_binres.release();
     if (c->errflag) cudaFree(c->errflag);

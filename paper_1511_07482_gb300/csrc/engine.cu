@@ -314,7 +314,14 @@ __device__ __forceinline__ C* smem_fft(C* a, C* b, int nl, const AxisPlan& ap, c
     C* dst = b;
     for (int s = 0; s < ap.nst; ++s) {
         const int R = ap.radix[s];
-        if constexpr (sizeof(C) == 16) {
+        if constexpr (std::is_same<C, dcplx>::value) {   // radices to 5 (their plans ask for no more)
+            switch (R) {
+                case 2: stockham_pass<C, 2>(src, dst, nl, ap.P, Ns, tw); break;
+                case 3: stockham_pass<C, 3>(src, dst, nl, ap.P, Ns, tw); break;
+                case 4: stockham_pass<C, 4>(src, dst, nl, ap.P, Ns, tw); break;
+                default: stockham_pass<C, 5>(src, dst, nl, ap.P, Ns, tw); break;
+            }
+        } else if constexpr (sizeof(C) == 16) {
             switch (R) {
                 case 2: stockham_pass<C, 2>(src, dst, nl, ap.P, Ns, tw); break;
                 case 3: stockham_pass<C, 3>(src, dst, nl, ap.P, Ns, tw); break;
@@ -645,152 +652,61 @@ __global__ void __launch_bounds__(256) k_final(const Item<real>* __restrict__ it
 }
 
 // ------------------------------------------------------------ autocorrelation passes
-// One pass of the count autocorrelation a = F^-1(|C|^2) (FP64) along one
-// axis, for many datasets in one launch.  A line holds the W spectrum values
-// along the axis (weights h_w: 2 on the interior of a half-spectrum axis,
-// else 1), zero-extended to the padded size P; its inverse DFT of length P
-// runs in shared memory and the J lags jlo .. jlo + J - 1 are kept.  The
-// inverse comes from the forward transform:
+// The count autocorrelation a = F^-1(|F(c)|^2) by passes along one axis at a
+// time, each line's transform of length P in shared memory (LineJob: what the
+// passes read and write).  The inverse comes from the forward transform:
 //   sum_w x_w e^{+2 pi i w j / P} = conj(sum_w conj(x_w) e^{-2 pi i w j / P}).
-// Line l = o I + i of a pass reads (o, w, i) at (o W + w) I + i and writes
-// lag jj to (o J + jj) I + i; the real spectrum of the first pass has I = 1.
-template <typename J>
-__device__ __forceinline__ int job_of(const J* __restrict__ jobs, int n, long long b) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (jobs[mid].blk0 <= b)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
+//
+// Bound by the FP32 pipes (pairs) or the FP64 pipe, so the passes transform as
+// little as they can: two real lines share one complex transform wherever the
+// input or the result is real (the first and the last pass, and the inverse
+// along axis 0), and along axis 0 the forward transform, |X|^2 and the inverse
+// are one pass, without the spectrum's way through memory.  Lines find their
+// places in memory once per line (a table in shared memory), not per value.
+// Against one complex transform per line in every pass, the spectrum in memory
+// and a 64-bit division per value (events around a data set's passes): 128^3
+// at P = 144 to 160 173 us (285), 48^4 420 us (737), 256^2 42 us (44: a line
+// per block, bound by the chain of stages); 512 data sets of 64^2 to 256^2 659
+// us (3378, most of it one line a block of 256 threads).  Issue slots 50 to 60
+// % busy, FP32 pipes 45 %, barriers and loads the rest.
+struct LineDiv {   // n / D for n < 2^20 (D <= 4096)
+    uint32_t m, D;
+    __device__ __forceinline__ explicit LineDiv(int d) : m(magic_of((uint32_t)max(d, 2))), D((uint32_t)d) {}
+    __device__ __forceinline__ int div(int n) const { return D == 1u ? n : (int)qdiv((uint32_t)n, m); }
+};
+__device__ __forceinline__ dflt half_of(dflt a) { return dflt(0.5f * a.h, 0.5f * a.l); }
+__device__ __forceinline__ double half_of(double a) { return 0.5 * a; }
+__device__ __forceinline__ dflt to_real(float v, dflt) { return dflt(v, 0.f); }
 
-// C: double2 (FP64) or dcplx (FP32 pairs, the same layout and size)
+// The transforms of real lines 0 and 1 at frequency w from that of x_0 + i x_1
+// (z at w, m at P - w).
 template <typename C>
-__global__ void __launch_bounds__(256) k_acorr_fft(const AcorrJob* __restrict__ jobs, int njobs,
-                                                   const C* __restrict__ twpool) {
-    using R = decltype(C{}.x);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const AcorrJob& jb = jobs[job_of(jobs, njobs, blockIdx.x)];
-    const int P = jb.ap.P, W = jb.W, J = jb.J, cap = jb.nl;
-    const long long I = jb.I;
-    const R* in_r = reinterpret_cast<const R*>(jb.in_r);
-    const C* in_c = reinterpret_cast<const C*>(jb.in_c);
-    C* out_c = reinterpret_cast<C*>(jb.out_c);
-    C* bufa = reinterpret_cast<C*>(smem_raw);
-    C* bufb = bufa + padded_cap(cap * P);
-    C* tw = bufb + padded_cap(cap * P);
-    const long long l0 = ((long long)blockIdx.x - jb.blk0) * cap;
-    const int nl = (int)min((long long)cap, jb.O * I - l0);
-    load_twiddles(tw, twpool, jb.ap);
-    auto hw = [&](int w) { return (jb.half && w != 0 && 2 * w != P) ? R(2.0) : R(1.0); };
-    if (I == 1) {   // consecutive lines are rows: w fastest
-        for (int t = threadIdx.x; t < nl * P; t += blockDim.x) {
-            const int c = t / P, w = t - c * P;
-            C x{R(0.0), R(0.0)};
-            if (w < W) {
-                const long long at = (l0 + c) * W + w;
-                const R h = hw(w);
-                x = in_r ? C{h * in_r[at], R(0.0)} : C{h * in_c[at].x, -(h * in_c[at].y)};
-            }
-            bufa[pad(t)] = x;
-        }
-    } else {        // consecutive lines are consecutive i: line fastest
-        for (int t = threadIdx.x; t < nl * P; t += blockDim.x) {
-            const int w = t / nl, c = t - w * nl;
-            C x{R(0.0), R(0.0)};
-            if (w < W) {
-                const long long l = l0 + c, o = l / I, i = l - o * I;
-                const C v = in_c[(o * W + w) * I + i];
-                const R h = hw(w);
-                x = C{h * v.x, -(h * v.y)};
-            }
-            bufa[pad(c * P + w)] = x;
-        }
-    }
-    const C* Y = smem_fft(bufa, bufb, nl, jb.ap, tw);
-    for (int t = threadIdx.x; t < nl * J; t += blockDim.x) {
-        int c, jj;
-        if (I == 1) {
-            c = t / J;
-            jj = t - c * J;
-        } else {
-            jj = t / nl;
-            c = t - jj * nl;
-        }
-        int j = (jb.jlo + jj) % P;
-        if (j < 0) j += P;
-        const C y = Y[pad(c * P + j)];
-        const long long l = l0 + c, o = l / I, i = l - o * I;
-        const long long at = (o * J + jj) * I + i;
-        if (jb.out_r) {
-            const double v = to_double(y.x) * jb.scale;
-            jb.out_r[at] = v;
-            if (jb.out_r32) jb.out_r32[at] = (float)v;
-        } else {
-            out_c[at] = C{y.x, -y.y};
-        }
-    }
+__device__ __forceinline__ C split_pair(int which, C z, C m) {
+    return which == 0 ? C{half_of(z.x + m.x), half_of(z.y - m.y)} : C{half_of(z.y + m.y), half_of(m.x - z.x)};
 }
 
-// Forward passes of the count spectrum in FP32 pairs (SpecJob).
-__global__ void __launch_bounds__(256) k_spec_df(const SpecJob* __restrict__ jobs, int njobs,
-                                                 const dcplx* __restrict__ twpool) {
-    using C = dcplx;
-    using R = dflt;
+template <typename C, int KIND>
+__global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, int njobs,
+                                              const C* __restrict__ twpool) {
+    using R = decltype(C{}.x);
+    constexpr bool packed = KIND == kLineRealRows || KIND == kLineLast || KIND == kLineSpecRows;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SpecJob& jb = jobs[job_of(jobs, njobs, blockIdx.x)];
-    const int P = jb.ap.P, X = jb.X, Yn = jb.Y, cap = jb.nl;
-    const long long I = jb.I;
-    const C* in_c = reinterpret_cast<const C*>(jb.in_c);
+    __shared__ long long src[kMaxLines], dst[kMaxLines];
+    const LineJob& jb = jobs[job_of_warp(njobs, blockIdx.x, [&](int k) { return jobs[k].blk0; })];
+    const int P = jb.ap.P, X = jb.X, Y = jb.Y, cap = jb.nl;
+    const int capf = packed ? (cap + 1) / 2 : cap;   // complex lines
     C* bufa = reinterpret_cast<C*>(smem_raw);
-    C* bufb = bufa + padded_cap(cap * P);
-    C* tw = bufb + padded_cap(cap * P);
+    C* bufb = bufa + padded_cap(capf * P);
+    C* tw = bufb + padded_cap(capf * P);
     const long long l0 = ((long long)blockIdx.x - jb.blk0) * cap;
-    const int nl = (int)min((long long)cap, jb.O * I - l0);
-    load_twiddles(tw, twpool, jb.ap);
-    if (I == 1) {   // rows: x fastest
-        for (int t = threadIdx.x; t < nl * P; t += blockDim.x) {
-            const int c = t / P, x = t - c * P;
-            C v{R(0.0), R(0.0)};
-            if (x < X) {
-                const long long at = (l0 + c) * X + x;
-                v = jb.in_f ? C{R(jb.in_f[at], 0.f), R(0.0)} : in_c[at];
-            }
-            bufa[pad(t)] = v;
-        }
-    } else {        // line fastest
-        for (int t = threadIdx.x; t < nl * P; t += blockDim.x) {
-            const int x = t / nl, c = t - x * nl;
-            C v{R(0.0), R(0.0)};
-            if (x < X) {
-                const long long l = l0 + c, o = l / I, i = l - o * I;
-                const long long at = (o * X + x) * I + i;
-                v = jb.in_f ? C{R(jb.in_f[at], 0.f), R(0.0)} : in_c[at];
-            }
-            bufa[pad(c * P + x)] = v;
-        }
-    }
-    const C* Yb = smem_fft(bufa, bufb, nl, jb.ap, tw);
-    C* out_c = reinterpret_cast<C*>(jb.out_c);
-    R* out_s = reinterpret_cast<R*>(jb.out_s);
-    for (int t = threadIdx.x; t < nl * Yn; t += blockDim.x) {
-        int c, y;
-        if (I == 1) {
-            c = t / Yn;
-            y = t - c * Yn;
-        } else {
-            y = t / nl;
-            c = t - y * nl;
-        }
-        const C v = Yb[pad(c * P + y)];
-        const long long l = l0 + c, o = l / I, i = l - o * I;
-        if (out_c) {
-            out_c[(o * Yn + y) * I + i] = v;
-        } else {
-            // |X|^2 at the inner index reordered with w_{d-1} slowest
+    const int nl = (int)min((long long)cap, jb.O * jb.I - l0);
+    const int nf = packed ? (nl + 1) / 2 : nl;
+    const long long I = jb.I;
+    if (threadIdx.x < nl) {
+        const long long l = l0 + threadIdx.x, o = l / I, i = l - o * I;
+        src[threadIdx.x] = o * X * I + i;
+        long long at = o * Y * I + i;
+        if constexpr (KIND == kLineAxis0) {   // rows of lags, w_{d-1} slowest
             long long r = i, q = 0;
             int wv[MAXD];
             for (int m = jb.d - 1; m >= 1; --m) {
@@ -798,65 +714,188 @@ __global__ void __launch_bounds__(256) k_spec_df(const SpecJob* __restrict__ job
                 r /= jb.ext[m];
             }
             for (int m = jb.d - 1; m >= 1; --m) q = q * jb.ext[m] + wv[m];
-            out_s[q * P + y] = v.x * v.x + v.y * v.y;
+            at = q * Y;
+        }
+        dst[threadIdx.x] = at;
+    }
+    load_twiddles(tw, twpool, jb.ap);
+    __syncthreads();
+    const LineDiv dP(P), dY(Y), dn(nl), df(nf);
+    const C zero{R(0.0), R(0.0)};
+    if constexpr (KIND == kLineRealRows || KIND == kLineSpecRows) {   // two real rows a line, values fastest
+        for (int t = threadIdx.x; t < nf * P; t += blockDim.x) {
+            const int c = dP.div(t), x = t - c * P;
+            C v = zero;
+            if (x < X) {
+                if constexpr (KIND == kLineRealRows) {
+                    v.x = to_real(jb.in_f[src[2 * c] + x], R());
+                    if (2 * c + 1 < nl) v.y = to_real(jb.in_f[src[2 * c + 1] + x], R());
+                } else {
+                    const R* in = reinterpret_cast<const R*>(jb.in);
+                    v.x = in[src[2 * c] + x];
+                    if (2 * c + 1 < nl) v.y = in[src[2 * c + 1] + x];
+                }
+            }
+            bufa[pad(t)] = v;
+        }
+    } else if constexpr (KIND == kLineLast) {
+        // half spectra of two real results: Z = X_0 + i X_1 on the whole line
+        // (X at P - w is conj(X) at w), conjugated for the inverse
+        const int half = P / 2;
+        for (int t = threadIdx.x; t < nf * (half + 1); t += blockDim.x) {
+            const int w = df.div(t), c = t - w * nf;
+            C a = zero, b = zero;
+            if (w < X) {
+                if (jb.in_real) {   // d = 1: the real spectrum itself
+                    a.x = reinterpret_cast<const R*>(jb.in)[src[2 * c] + w];
+                } else {
+                    const C* in = reinterpret_cast<const C*>(jb.in);
+                    a = in[src[2 * c] + w * I];
+                    if (2 * c + 1 < nl) b = in[src[2 * c + 1] + w * I];
+                }
+            }
+            if (w == 0 || 2 * w == P) {   // real, but for rounding
+                bufa[pad(c * P + w)] = C{a.x, -b.x};
+            } else {
+                bufa[pad(c * P + w)] = C{a.x - b.y, -(a.y + b.x)};
+                bufa[pad(c * P + P - w)] = C{a.x + b.y, a.y - b.x};
+            }
+        }
+    } else {   // complex lines, line fastest
+        for (int t = threadIdx.x; t < nl * P; t += blockDim.x) {
+            const int x = dn.div(t), c = t - x * nl;
+            C v = zero;
+            if (x < X) {
+                const long long at = src[c] + x * I;
+                if constexpr (KIND == kLineAxis0) {
+                    if (jb.in_f)   // d = 1: the counts themselves
+                        v.x = to_real(jb.in_f[at], R());
+                    else
+                        v = reinterpret_cast<const C*>(jb.in)[at];
+                } else {
+                    v = reinterpret_cast<const C*>(jb.in)[at];
+                    if constexpr (KIND == kLineInverse) v.y = -v.y;
+                }
+            }
+            bufa[pad(c * P + x)] = v;
+        }
+    }
+    C* Z = smem_fft(bufa, bufb, nf, jb.ap, tw);
+    if constexpr (KIND == kLineAxis0) {
+        // |X|^2 of two lines share a complex line of the inverse
+        C* other = Z == bufa ? bufb : bufa;
+        const int nh = (nl + 1) / 2;
+        for (int t = threadIdx.x; t < nh * P; t += blockDim.x) {
+            const int c = dP.div(t), w = t - c * P;
+            const C a = Z[pad(2 * c * P + w)];
+            C v{a.x * a.x + a.y * a.y, R(0.0)};
+            if (2 * c + 1 < nl) {
+                const C b = Z[pad((2 * c + 1) * P + w)];
+                v.y = b.x * b.x + b.y * b.y;
+            }
+            other[pad(t)] = v;
+        }
+        Z = smem_fft(other, Z, nh, jb.ap, tw);
+    }
+    C* out = reinterpret_cast<C*>(jb.out);
+    if constexpr (KIND == kLineRealRows || KIND == kLineSpecRows || KIND == kLineAxis0) {   // values fastest
+        for (int t = threadIdx.x; t < nl * Y; t += blockDim.x) {
+            const int c = dY.div(t), y = t - c * Y;
+            const int zb = (c >> 1) * P;
+            C v = split_pair(c & 1, Z[pad(zb + y)], Z[pad(zb + (y ? P - y : 0))]);
+            if constexpr (KIND != kLineRealRows) v.y = -v.y;
+            if (KIND == kLineAxis0 && jb.out_r) {   // d = 1
+                const double r = to_double(v.x) * jb.scale;
+                jb.out_r[dst[c] + y] = r;
+                jb.out_r32[dst[c] + y] = (float)r;
+            } else {
+                out[dst[c] + y] = v;
+            }
+        }
+    } else {   // line fastest
+        for (int t = threadIdx.x; t < nl * Y; t += blockDim.x) {
+            const int y = dn.div(t), c = t - y * nl;
+            const long long at = dst[c] + y * I;
+            if constexpr (KIND == kLineForward) {
+                out[at] = Z[pad(c * P + y)];
+            } else {
+                int j = jb.ylo + y;   // a lag, |j| < P
+                if (j < 0) j += P;
+                if constexpr (KIND == kLineInverse) {
+                    const C v = Z[pad(c * P + j)];
+                    out[at] = C{v.x, -v.y};
+                } else {
+                    const C v = Z[pad((c >> 1) * P + j)];
+                    const double r = to_double((c & 1) ? -v.y : v.x) * jb.scale;
+                    jb.out_r[at] = r;
+                    jb.out_r32[at] = (float)r;
+                }
+            }
         }
     }
 }
 
-cudaError_t acorr_plan(AcorrJob* jobs_h, int n, long long* blocks_out, size_t* sm_out) {
+int line_lines(int kind, int P, long long lines, int nsm) {
+    // Complex lines per CTA: as many as fill kLineSmem (four CTAs an SM, for
+    // lines of a few hundred values), but no more than leave two CTAs an SM
+    // busy over all lines of the launch; at least one.
+    const bool packed = kind == kLineRealRows || kind == kLineLast || kind == kLineSpecRows;
+    constexpr size_t kLineSmem = 56 * 1024;
+    int f = 1;
+    while (f < kMaxLines / 2 && line_smem_bytes(P, f + 1) <= kLineSmem) ++f;
+    const long long spread = std::max<long long>(1, (packed ? (lines + 1) / 2 : lines) / (2LL * nsm));
+    f = (int)std::min<long long>(f, spread);
+    return packed ? 2 * f : f;
+}
+
+cudaError_t line_plan(LineJob* jobs_h, int n, int kind, long long* blocks_out, size_t* sm_out, int* threads_out) {
+    const bool packed = kind == kLineRealRows || kind == kLineLast || kind == kLineSpecRows;
     long long blocks = 0;
     size_t sm = 0;
+    int work = 0;
     for (int k = 0; k < n; ++k) {
-        AcorrJob& jb = jobs_h[k];
-        if (jb.nl < 1 || jb.ap.P < 2 || jb.W > jb.ap.P || (!jb.in_r && !jb.in_c) || (jb.in_r && jb.I != 1))
+        LineJob& jb = jobs_h[k];
+        const bool rows = kind == kLineRealRows || kind == kLineSpecRows;
+        if (jb.nl < 1 || jb.nl > kMaxLines || jb.ap.P < 2 || jb.X > jb.ap.P || jb.Y > jb.ap.P || (!jb.in && !jb.in_f) ||
+            (!jb.out && !jb.out_r) || (rows && jb.I != 1) || (kind == kLineAxis0 && jb.O != 1) || jb.d < 1 ||
+            jb.d > MAXD || (jb.in_real && jb.O * jb.I != 1))
             return cudaErrorInvalidValue;
         jb.blk0 = blocks;
         blocks += (jb.O * jb.I + jb.nl - 1) / jb.nl;
-        sm = std::max(sm, acorr_smem_bytes(jb.ap.P, jb.nl));
+        const int f = packed ? (jb.nl + 1) / 2 : jb.nl;
+        sm = std::max(sm, line_smem_bytes(jb.ap.P, f));
+        work = std::max(work, f * jb.ap.P / 4);
     }
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     *blocks_out = blocks;
     *sm_out = sm;
+    *threads_out = std::min(256, std::max(64, (work + 31) / 32 * 32));   // about a butterfly a thread
     return cudaSuccess;
 }
 
-cudaError_t spec_plan(SpecJob* jobs_h, int n, long long* blocks_out, size_t* sm_out) {
-    long long blocks = 0;
-    size_t sm = 0;
-    for (int k = 0; k < n; ++k) {
-        SpecJob& jb = jobs_h[k];
-        if (jb.nl < 1 || jb.ap.P < 2 || jb.X > jb.ap.P || jb.Y > jb.ap.P || (!jb.in_f && !jb.in_c) ||
-            (!jb.out_c && !jb.out_s) || (jb.out_s && jb.O != 1) || jb.d < 1 || jb.d > MAXD)
-            return cudaErrorInvalidValue;
-        jb.blk0 = blocks;
-        blocks += (jb.O * jb.I + jb.nl - 1) / jb.nl;
-        sm = std::max(sm, acorr_smem_bytes(jb.ap.P, jb.nl));
+template <typename C>
+static cudaError_t line_go(int kind, const LineJob* jobs, int n, unsigned blocks, size_t sm, int threads,
+                           const void* tw, cudaStream_t st) {
+    const C* twp = (const C*)tw;
+    if constexpr (std::is_same<C, dcplx>::value) {
+        if (kind == kLineRealRows) k_line<C, kLineRealRows><<<blocks, threads, sm, st>>>(jobs, n, twp);
+        if (kind == kLineForward) k_line<C, kLineForward><<<blocks, threads, sm, st>>>(jobs, n, twp);
+        if (kind == kLineAxis0) k_line<C, kLineAxis0><<<blocks, threads, sm, st>>>(jobs, n, twp);
+    } else {
+        if (kind == kLineSpecRows) k_line<C, kLineSpecRows><<<blocks, threads, sm, st>>>(jobs, n, twp);
     }
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    *blocks_out = blocks;
-    *sm_out = sm;
-    return cudaSuccess;
-}
-
-cudaError_t launch_acorr(const AcorrJob* jobs_d, int n, long long blocks, size_t sm, const double2* twpool,
-                         cudaStream_t st) {
-    if (n <= 0 || blocks <= 0) return cudaSuccess;
-    k_acorr_fft<double2><<<(unsigned)blocks, 256, sm, st>>>(jobs_d, n, twpool);
+    if (kind == kLineInverse) k_line<C, kLineInverse><<<blocks, threads, sm, st>>>(jobs, n, twp);
+    if (kind == kLineLast) k_line<C, kLineLast><<<blocks, threads, sm, st>>>(jobs, n, twp);
     return cudaGetLastError();
 }
 
-cudaError_t launch_acorr_df(const AcorrJob* jobs_d, int n, long long blocks, size_t sm, const void* twpool,
-                            cudaStream_t st) {
+cudaError_t launch_line(int kind, bool pairs, const LineJob* jobs_d, int n, long long blocks, size_t sm, int threads,
+                        const void* twpool, cudaStream_t st) {
     if (n <= 0 || blocks <= 0) return cudaSuccess;
-    k_acorr_fft<dcplx><<<(unsigned)blocks, 256, sm, st>>>(jobs_d, n, (const dcplx*)twpool);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_spec_df(const SpecJob* jobs_d, int n, long long blocks, size_t sm, const void* twpool,
-                           cudaStream_t st) {
-    if (n <= 0 || blocks <= 0) return cudaSuccess;
-    k_spec_df<<<(unsigned)blocks, 256, sm, st>>>(jobs_d, n, (const dcplx*)twpool);
-    return cudaGetLastError();
+    const bool known = pairs ? kind != kLineSpecRows : (kind == kLineSpecRows || kind == kLineInverse || kind == kLineLast);
+    if (!known) return cudaErrorInvalidValue;
+    return pairs ? line_go<dcplx>(kind, jobs_d, n, (unsigned)blocks, sm, threads, twpool, st)
+                 : line_go<double2>(kind, jobs_d, n, (unsigned)blocks, sm, threads, twpool, st);
 }
 
 // ------------------------------------------------------------ reduce
@@ -2237,8 +2276,11 @@ cudaError_t prepare_kernels() {
     const void* dyn[] = {(const void*)k_stage_a<float>,    (const void*)k_stage_a<double>,
                          (const void*)k_mid<float>,        (const void*)k_mid<double>,
                          (const void*)k_final<float>,      (const void*)k_final<double>,
-                         (const void*)k_acorr_fft<double2>, (const void*)k_acorr_fft<dcplx>,
-                         (const void*)k_spec_df,           (const void*)k_select2d_lag<1>,
+                         (const void*)k_line<dcplx, kLineRealRows>, (const void*)k_line<dcplx, kLineForward>,
+                         (const void*)k_line<dcplx, kLineAxis0>,    (const void*)k_line<dcplx, kLineInverse>,
+                         (const void*)k_line<dcplx, kLineLast>,     (const void*)k_line<double2, kLineSpecRows>,
+                         (const void*)k_line<double2, kLineInverse>, (const void*)k_line<double2, kLineLast>,
+                         (const void*)k_select2d_lag<1>,
                          (const void*)k_select2d_lag<2>,   (const void*)k_select2d_lag<4>,
                          (const void*)k_select2d,          (const void*)k_fused2d<float, 2>,
                          (const void*)k_fused2d<float, 4>, (const void*)k_fused2d<double, 2>};

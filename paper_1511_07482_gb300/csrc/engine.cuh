@@ -283,69 +283,54 @@ struct LagSum {
     double scale;
 };
 cudaError_t launch_lag_sum(const LagSum* sums, int nitems, const double* partial, double* out, cudaStream_t st);
-// One separable pass of the inverse DFT that turns the FP64 count spectrum
-// into the autocorrelation, for one dataset: out[o][jj][i] = sum_{w < W} h(w)
-// in[o][w][i] e^{+2 pi i w (jlo + jj) / P}, h(w) = 1, or for the
-// half-spectrum axis (half != 0) 1 at w = 0 and w = P/2 and 2 elsewhere.  in:
-// real (in_r) or complex (in_c); out: complex (out_c), or the real part times
-// `scale` (out_r, and rounded to FP32 into out_r32 when given).  Twiddles
-// exp(-2 pi i t / P), t < P, at twpool + tw_off.  blk0: the job's first
-// block in a launch over many jobs (set by the launcher).
-struct AcorrJob {
-    const double* in_r;          // real input (the count spectrum; first pass, I = 1), or
-    const double2* in_c;         // complex input of a later pass
-    double2* out_c;              // complex output of a pass before the last, or
-    double* out_r;               // real part of the last pass (times scale), with
-    float* out_r32;              // its FP32 copy
-    long long O, I;              // lines O I; element (o, w, i) at (o W + w) I + i
-    int W, J, jlo, half;         // W values per line (<= P); lags jlo .. jlo + J - 1; half: weights 2 inside
-    int nl;                      // lines per CTA
+// One pass of the count autocorrelation along one axis, for one dataset: O I
+// lines, each a transform of length P of X input values (zero-extended), of
+// which Y results are kept.  Element (o, x, i) of the input lies at
+// (o X + x) I + i, result y at (o Y + y) I + i.  Complex values are complex
+// FP32 pairs (dcplx, FP32 datasets) or double2 (FP64 datasets), real ones the
+// pair or the double.
+//   RealRows  rows of FP32 counts (in_f, I = 1) -> frequencies 0 .. Y - 1 of
+//             the half spectrum
+//   Forward   complex lines -> frequencies 0 .. Y - 1
+//   Axis0     complex lines along axis 0 (O = 1; d = 1: the counts, in_f):
+//             forward, |X|^2, inverse; lags 0 .. Y - 1 to a row at q Y, q the
+//             inner index (w_1 .. w_{d-1}, extents ext[1..d-1], w_{d-1}
+//             fastest) reordered with w_{d-1} slowest; d = 1: the result
+//             itself (out_r, out_r32)
+//   SpecRows  rows of a real spectrum (I = 1) -> inverse, lags 0 .. Y - 1
+//   Inverse   complex lines -> inverse, lags ylo .. ylo + Y - 1
+//   Last      half spectra (frequencies 0 .. X - 1 = P / 2; in_real: one real
+//             line) -> the real inverse times scale, lags ylo .. ylo + Y - 1,
+//             as FP64 (out_r) and FP32 (out_r32)
+enum { kLineRealRows, kLineForward, kLineAxis0, kLineSpecRows, kLineInverse, kLineLast };
+constexpr int kMaxLines = 64;    // lines of a CTA
+struct LineJob {
+    const float* in_f;
+    const void* in;
+    void* out;
+    double* out_r;
+    float* out_r32;
+    long long O, I;
+    int X, Y, ylo, nl;           // nl: lines per CTA (line_lines)
+    int d, in_real;
+    int ext[MAXD];
     AxisPlan ap;                 // the length-P transform (radix stages, twiddle offset)
     double scale;
-    long long blk0;
+    long long blk0;              // the job's first block in a launch over many jobs (line_plan)
 };
-// shared memory of an autocorrelation pass: two line buffers and P twiddles
-__host__ __device__ constexpr size_t acorr_smem_bytes(int P, int nl) {
-    return sizeof(double2) * ((size_t)2 * (size_t)(nl * P + ((nl * P) >> 4) + 1) + (size_t)P);
+// shared memory of a pass: two line buffers and P twiddles
+__host__ __device__ constexpr size_t line_smem_bytes(int P, int lines) {
+    return sizeof(double2) * ((size_t)2 * (size_t)(lines * P + ((lines * P) >> 4) + 1) + (size_t)P);
 }
-// All jobs' passes of one level in one launch (one CTA per nl lines).
-// acorr_plan (host) checks the table, writes each job's blk0 and returns the
-// CTA count and shared memory of the launch; launch_acorr runs the table
-// once it is on the device.
-cudaError_t acorr_plan(AcorrJob* jobs_h, int n, long long* blocks, size_t* sm);
-cudaError_t launch_acorr(const AcorrJob* jobs_d, int n, long long blocks, size_t sm, const double2* twpool,
-                         cudaStream_t st);
-// The same passes in FP32-pair arithmetic (FP32 datasets): the pointers of
-// the jobs then hold FP32 pairs of the same sizes (in_r: the spectrum as
-// pairs; in_c / out_c: complex pairs); out_r / out_r32 stay FP64 / FP32.
-// twpool: the twiddles as complex FP32 pairs.
-cudaError_t launch_acorr_df(const AcorrJob* jobs_d, int n, long long blocks, size_t sm, const void* twpool,
-                            cudaStream_t st);
-
-// One forward pass of the count spectrum |F(c_zp)|^2 in FP32-pair arithmetic
-// (FP32 datasets), for one dataset: lines O I, element (o, x, i) at
-// (o X + x) I + i for x < X (the grid's M_k values along the axis, zero-
-// extended to P), its forward DFT of length P, the first Y frequencies kept.
-// The first pass reads the FP32 counts (in_f, rows: I = 1) and keeps the
-// half spectrum; the others read complex pairs (in_c).  A pass before the
-// last writes (o, y, i) at (o Y + y) I + i (out_c); the last (axis 0, O = 1)
-// writes |X_y|^2 as an FP32 pair to out_s at q P + y, q the inner index
-// (w_1 .. w_{d-1}, extents ext[1..d-1], w_{d-1} fastest) reordered with
-// w_{d-1} slowest: the layout the autocorrelation passes read.
-struct SpecJob {
-    const float* in_f;
-    const void* in_c;
-    void* out_c;
-    void* out_s;
-    long long O, I;
-    int X, Y, nl, d;
-    int ext[MAXD];
-    AxisPlan ap;
-    long long blk0;
-};
-cudaError_t spec_plan(SpecJob* jobs_h, int n, long long* blocks, size_t* sm);
-cudaError_t launch_spec_df(const SpecJob* jobs_d, int n, long long blocks, size_t sm, const void* twpool,
-                           cudaStream_t st);
+// lines per CTA for a launch over `lines` lines of length P in all
+int line_lines(int kind, int P, long long lines, int nsm);
+// All jobs' passes of one level in one launch.  line_plan (host) checks the
+// table, writes each job's blk0 and returns the launch's CTAs, shared memory
+// and threads; launch_line runs the table once it is on the device.  twpool:
+// the twiddles as complex FP32 pairs (pairs) or double2.
+cudaError_t line_plan(LineJob* jobs_h, int n, int kind, long long* blocks, size_t* sm, int* threads);
+cudaError_t launch_line(int kind, bool pairs, const LineJob* jobs_d, int n, long long blocks, size_t sm, int threads,
+                        const void* twpool, cudaStream_t st);
 
 // ---- kernel density estimate on the grid and mixture cross term (kde.cu)
 struct KdeDesc {
