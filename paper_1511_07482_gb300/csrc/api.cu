@@ -589,8 +589,8 @@ struct kdefft_ctx_s {
     // all of them
     struct PendingRead {
         ReqSet* rs;
-        std::vector<std::pair<int, int>> pairs;   // grid pairs in the order of their results
-        size_t off;                               // first double in h_out
+        std::vector<int> grids;   // in the order of their results
+        size_t off;               // first double in h_out
     };
     std::vector<PendingRead> pend_reads;
     size_t hout_used = 0;       // doubles of h_out holding pending results
@@ -933,6 +933,11 @@ struct GridReq {
     int P[4];
     TermVec terms;
     bool fp64 = false;     // evaluate in FP64 even on an FP32 dataset
+    // 0: a weighted sum of the covariances' Gaussians; r > 0: of one partial of
+    // order r, the grids of an order following one another in graded order
+    // (place: the partial's place among them); -1: anything else
+    signed char order = -1;
+    short place = 0;
     double value = 0.0;    // result: n^-2 sum_w |C|^2 K / prod P  (= Eq. 25)
 };
 
@@ -1064,30 +1069,33 @@ static int add_lscv_at(ReqSet& rs, kdefft_ds ds, const Mat& H, bool grad, int si
     const Mat& basis = (ds->opts.L_basis == KDEFFT_L_WIDEST) ? sp.sig[0] : H;
     KCHK(plan_for(ds, basis, L, P));
     int gi = g0;
-    auto put = [&](TermVec t) {
+    auto put = [&](TermVec t, int order, int place) {
         GridReq& g = rs.grids[gi++];
         g.ds = ds;
         g.spec = si;
         std::memcpy(g.L, L, sizeof(L));
         std::memcpy(g.P, P, sizeof(P));
         g.terms = std::move(t);
+        g.order = (signed char)order;
+        g.place = (short)place;
     };
     const double n = (double)ds->n;
     if (!ds->opts.exact_loo) {
-        put({Term{0, {0, 0, 0, 0}, 1.0}, Term{1, {0, 0, 0, 0}, -2.0}});
+        put({Term{0, {0, 0, 0, 0}, 1.0}, Term{1, {0, 0, 0, 0}, -2.0}}, 0, 0);
     } else {
-        put({Term{0, {0, 0, 0, 0}, 1.0}});
-        put({Term{1, {0, 0, 0, 0}, 1.0}});
+        put({Term{0, {0, 0, 0, 0}, 1.0}}, 0, 0);
+        put({Term{1, {0, 0, 0, 0}, 1.0}}, 0, 0);
     }
     if (grad) {
         const double f = ds->opts.exact_loo ? n / (n - 1.0) : 1.0;
+        int place = 0;
         for (int a = 0; a < d; ++a)
             for (int b = a; b < d; ++b) {
                 const double s = (a == b) ? 1.0 : 2.0;
                 Term t0{0, {0}, s}, t1{1, {0}, -s * f};
                 alpha2(d, a, b, t0.alpha);
                 alpha2(d, a, b, t1.alpha);
-                put({t0, t1});
+                put({t0, t1}, 2, place++);
             }
     }
     return KDEFFT_OK;
@@ -1147,13 +1155,15 @@ static int add_scv(ReqSet& rs, kdefft_ds ds, const Mat& H, const Mat& G, bool gr
     const Mat& basis = (ds->opts.L_basis == KDEFFT_L_PAPER) ? H : sp.sig[0];
     KCHK(plan_for(ds, basis, L, P));
     first = (int)rs.grids.size();
-    auto push = [&](TermVec t) {
+    auto push = [&](TermVec t, int order, int place) {
         GridReq g;
         g.ds = ds;
         g.spec = si;
         std::memcpy(g.L, L, sizeof(L));
         std::memcpy(g.P, P, sizeof(P));
         g.terms = std::move(t);
+        g.order = (signed char)order;
+        g.place = (short)place;
         rs.grids.push_back(std::move(g));
     };
     // value: the two H-dependent Gaussians as separate grids (one packed pair);
@@ -1161,20 +1171,21 @@ static int add_scv(ReqSet& rs, kdefft_ds ds, const Mat& H, const Mat& G, bool gr
     // because the full SCV kernel integrates to zero and its transform near
     // w = 0 would cancel in FP32
     if (split64) {
-        push({Term{0, {0}, 1.0}});
-        push({Term{1, {0}, 1.0}});
+        push({Term{0, {0}, 1.0}}, 0, 0);
+        push({Term{1, {0}, 1.0}}, 0, 0);
         rs.grids[first].fp64 = rs.grids[first + 1].fp64 = true;
     } else {
-        push({Term{0, {0}, 1.0}, Term{1, {0}, -2.0}, Term{2, {0}, 1.0}});
+        push({Term{0, {0}, 1.0}, Term{1, {0}, -2.0}, Term{2, {0}, 1.0}}, 0, 0);
     }
     if (grad) {
+        int place = 0;
         for (int a = 0; a < d; ++a)
             for (int b = a; b < d; ++b) {
                 const double s = (a == b) ? 1.0 : 2.0;
                 Term t0{0, {0}, s}, t1{1, {0}, -s};
                 alpha2(d, a, b, t0.alpha);
                 alpha2(d, a, b, t1.alpha);
-                push({t0, t1});
+                push({t0, t1}, 2, place++);
             }
     }
     return KDEFFT_OK;
@@ -1211,8 +1222,14 @@ static int add_psi_at(ReqSet& rs, kdefft_ds ds, const Mat& H, const std::vector<
         std::memcpy(g.L, L, sizeof(L));
         std::memcpy(g.P, P, sizeof(P));
         Term t{0, {0}, 1.0};
-        for (int k = 0; k < MAXD; ++k) t.alpha[k] = (k < d) ? m.a[k] : 0;
+        int order = 0;
+        for (int k = 0; k < MAXD; ++k) {
+            t.alpha[k] = (k < d) ? m.a[k] : 0;
+            order += t.alpha[k];
+        }
         g.terms.assign(1, t);
+        g.order = (signed char)order;
+        g.place = (short)(gi - 1 - g0);
     }
     return KDEFFT_OK;
 }
@@ -1326,6 +1343,7 @@ static int add_eta_m(ReqSet& rs, kdefft_ds ds, const Mat& Sg, int m, int& first)
     std::memcpy(g.L, L, sizeof(L));
     std::memcpy(g.P, P, sizeof(P));
     laplacian_power_terms(ds->d, m, 0, 1.0, g.terms);
+    if (m == 0) g.order = 0;
     rs.grids.push_back(std::move(g));
     return KDEFFT_OK;
 }
@@ -1567,10 +1585,7 @@ static int flush_reads(kdefft_ctx c) {
     }
     const double* o = (const double*)c->h_out.p;
     for (const auto& pr : c->pend_reads)
-        for (size_t i = 0; i < pr.pairs.size(); ++i) {
-            pr.rs->grids[pr.pairs[i].first].value = o[pr.off + 2 * i];
-            if (pr.pairs[i].second >= 0) pr.rs->grids[pr.pairs[i].second].value = o[pr.off + 2 * i + 1];
-        }
+        for (size_t i = 0; i < pr.grids.size(); ++i) pr.rs->grids[pr.grids[i]].value = o[pr.off + i];
     c->pend_reads.clear();
     c->hout_used = 0;
     return KDEFFT_OK;
@@ -2198,34 +2213,77 @@ static int ensure_autocorr_many(kdefft_ctx c, const std::vector<std::pair<kdefft
     return KDEFFT_OK;
 }
 
-// highest derivative order among the terms of a grid pair
-static int pair_order(const ReqSet& rs, const std::pair<int, int>& pr, int d) {
+// highest derivative order among the terms of the grids ids[0 .. n)
+static int group_order(const ReqSet& rs, const int* ids, int n, int d) {
     int R = 0;
-    for (int gi : {pr.first, pr.second}) {
-        if (gi < 0) continue;
-        for (const Term& t : rs.grids[gi].terms) {
+    for (int i = 0; i < n; ++i)
+        for (const Term& t : rs.grids[ids[i]].terms) {
             int o = 0;
             for (int k = 0; k < d; ++k) o += t.alpha[k];
             R = std::max(R, o);
         }
-    }
     return R;
 }
 
+// Points of a FP32 lag tile (per launch, 1024 / 2048 / 4096 points): one
+// bandwidth 10.7 / 12.5 / 16.1 us, plug-in in 4-D 32 / 41 / 58 us, 256 LSCV
+// bandwidths 17 / 15 / 17 us; large batches pay for the smaller tiles (psi_4 of
+// 256 bandwidths on 128^3 78 / 66 / 62 us, 512 data sets x 16 148 / 134 / 135
+// us), a few percent of calls that take 0.6 and 6.6 ms.
+static constexpr long long kLagTile = 1024;
+
+// A lag work item to be: n consecutive grids of one dataset, covariances and
+// plan, from ids[first] of a run's grid list.  Form: nv Gaussians and all
+// partials of order R (nv >= 0), or dense, two kernels up to order R (nv < 0).
+struct LagGroup {
+    int first, n, R, nv;
+    int sums() const {   // kernels that its launch sums (the dense form and merged ones: maybe one more than n)
+        return nv < 0 || (R == 0 && nv == 2) ? 2 : n;
+    }
+};
+
 // the lag-domain engine computes exactly the FFT route's value when the
 // padding has no aliasing (P_k >= M_k + L_k on every axis)
-template <typename real>
-static bool lag_eligible(kdefft_ctx c, const ReqSet& rs, const std::pair<int, int>& pr) {
+static bool lag_covers(kdefft_ctx c, const GridReq& g) {
     if (!c->lag) return false;
-    const GridReq& g = rs.grids[pr.first];
     const int d = g.ds->d;
     long long pts = g.L[0] + 1;   // half-box points: the lag kernel indexes them in 32 bits
     for (int k = 0; k < d; ++k) {
         if (g.P[k] < g.ds->M[k] + g.L[k]) return false;
         if (k > 0) pts *= 2 * g.L[k] + 1;
     }
-    if (pts > (1LL << 32)) return false;
-    return lag_table_size(d, pair_order(rs, pr, d), sizeof(real) == 8) > 0;
+    return pts <= (1LL << 32);
+}
+
+// Lag groups of the grids ids[a .. b), which share dataset, covariances and
+// plan: one group where they are Gaussians followed by a whole order of
+// partials (values and gradients, psi_r), else pairs; pairs that no lag kernel
+// covers go to `rest`.
+static void lag_groups(const ReqSet& rs, const std::vector<int>& ids, int a, int b, bool dbl,
+                       std::vector<LagGroup>& out, std::vector<std::pair<int, int>>& rest) {
+    const GridReq& g = rs.grids[ids[a]];
+    const int d = g.ds->d;
+    int nv = 0;
+    while (a + nv < b && rs.grids[ids[a + nv]].order == 0) ++nv;
+    const int R = a + nv < b ? rs.grids[ids[a + nv]].order : 0;
+    bool whole = R >= 0;
+    int members = 1;   // partials of order R
+    for (int i = 1; i < d; ++i) members = members * (R + i) / i;
+    whole = whole && b - a == nv + (R > 0 ? members : 0);
+    for (int i = a + nv; whole && i < b; ++i)
+        whole = rs.grids[ids[i]].order == R && rs.grids[ids[i]].place == i - a - nv;
+    if (whole && lag_single_form(d, R, nv, rs.specs[g.spec].nsig)) {
+        out.push_back({a, b - a, R, nv});
+        return;
+    }
+    for (int i = a; i < b; i += 2) {
+        const int n = std::min(2, b - i);
+        const int Rp = group_order(rs, &ids[i], n, d);
+        if (lag_table_size(d, Rp, dbl) > 0)
+            out.push_back({i, n, (Rp + 1) & ~1, -1});
+        else
+            rest.push_back({ids[i], n > 1 ? ids[i + 1] : -1});
+    }
 }
 
 // Granlund and Montgomery's unsigned division by an invariant integer
@@ -2242,21 +2300,22 @@ static void invariant_div(uint32_t v, unsigned int& m, int& sh) {
 }
 
 // The lag-domain work of one precision in a run, built on the host: the
-// items (LagItem<real>), their tiles and dense weights, the derivative-order
-// classes (R, first tile, tiles; one launch each) and the grid pairs in item
-// order.  run_lag builds it; issue_lag uploads and launches the batches of
-// both precisions of a run together.
+// items (LagItem<real>), their tiles and weights, the forms (R, nv, first
+// tile, tiles; one launch each) and the grids in the order of the results.
+// run_lag builds it; issue_lag uploads and launches the batches of both
+// precisions of a run together.
 struct LagBatch {
     bool dbl = false;
     int d = 0;
     int nitems = 0;
+    size_t nslots = 0;                   // partial sums
     std::vector<LagItem<float>> it32;    // the items (it64 for FP64)
     std::vector<LagItem<double>> it64;
-    std::vector<float> w32;              // the dense weights (w64 for FP64)
+    std::vector<float> w32;              // the weights (w64 for FP64)
     std::vector<double> w64;
     std::vector<LagTile> tiles;
-    std::vector<std::array<int, 3>> classes;
-    std::vector<std::pair<int, int>> pairs;
+    std::vector<std::array<int, 4>> classes;
+    std::vector<int> grids;
     double fl = 0.0, by = 0.0;   // algorithmic flops and bytes of the batch
     template <typename real>
     std::vector<LagItem<real>>& items() {
@@ -2272,20 +2331,21 @@ struct LagBatch {
     size_t w_size() const { return dbl ? sizeof(double) * w64.size() : sizeof(float) * w32.size(); }
 };
 
-// Build the lag-domain batch for the grid pairs (the count autocorrelation
+// Build the lag-domain batch for the groups (the count autocorrelation
 // box they need is grown first).  (Building a large set in chunks, each
 // issued while the next is built, was measured slower: each chunk's launch
 // leaves the GPU partly idle at its tail.)
 
 template <typename real>
-static int run_lag(kdefft_ctx c, ReqSet& rs, std::vector<std::pair<int, int>> pairs, std::vector<LagBatch>& out) {
-    if (pairs.empty()) return KDEFFT_OK;
+static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::vector<LagGroup> groups,
+                   std::vector<LagBatch>& out) {
+    if (groups.empty()) return KDEFFT_OK;
     const bool dbl = sizeof(real) == 8;
-    const int d = rs.grids[pairs[0].first].ds->d;
+    const int d = rs.grids[ids[0]].ds->d;
     {
         std::map<kdefft_ds, std::array<int, 4>> need;
-        for (const auto& pr : pairs) {
-            const GridReq& g = rs.grids[pr.first];
+        for (const LagGroup& gr : groups) {
+            const GridReq& g = rs.grids[ids[gr.first]];
             auto& a = need[g.ds];
             for (int k = 0; k < d; ++k) a[k] = std::max(a[k], g.L[k]);
         }
@@ -2293,112 +2353,111 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, std::vector<std::pair<int, int>> pa
         KCHK(ensure_autocorr_many(c, rq));
     }
     HostTimer hbuild(c, "host:lag_build");
-    // order classes, contiguous
-    std::vector<int> Re(pairs.size());
-    for (size_t i = 0; i < pairs.size(); ++i) Re[i] = (pair_order(rs, pairs[i], d) + 1) & ~1;
-    std::vector<size_t> ord(pairs.size());
+    // single Gaussians join the pairs of Gaussians, if there are any, in one launch
+    bool two = false;
+    for (const LagGroup& gr : groups) two = two || (gr.R == 0 && gr.nv == 2);
+    for (LagGroup& gr : groups)
+        if (two && gr.R == 0 && gr.nv == 1) gr.nv = 2;
+    // forms, contiguous
+    std::vector<size_t> ord(groups.size());
     for (size_t i = 0; i < ord.size(); ++i) ord[i] = i;
-    std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) { return Re[a] < Re[b]; });
+    std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) {
+        return groups[a].R != groups[b].R ? groups[a].R < groups[b].R : groups[a].nv < groups[b].nv;
+    });
     HermiteIndex& hx = hindex();
     // fixed tiles, so that an item's sum depends on the item alone, not on
-    // the batch it came in: 4096 points in FP32 (smaller tiles halved the
-    // throughput of batches: per-tile work is then too small for a CTA), 256
-    // in FP64 (the points are slow on the FP64 pipe: more CTAs in flight, one
-    // point per thread)
-    const long long T = dbl ? 32 * kLagSlices : 4096;
+    // the batch it came in: kLagTile points in FP32, 256 in FP64 (the points
+    // are slow on the FP64 pipe: more CTAs in flight, one point per thread)
+    const long long T = dbl ? 32 * kLagSlices : kLagTile;
     const size_t ni = ord.size();
     LagBatch bt;
     bt.dbl = dbl;
     bt.d = d;
     std::vector<LagItem<real>>& items = bt.items<real>();
     std::vector<real>& wpool = bt.wpool<real>();
-    // layout (serial): each item's tiles and weights at fixed offsets, the
-    // order classes, the algorithmic work
-    std::vector<long long> tile0(ni + 1), woff(ni + 1), npts(ni);
-    tile0[0] = 0;
-    woff[0] = 0;
+    // layout (serial): each item's tiles, partials, weights and results at
+    // fixed offsets, the forms, the algorithmic work
+    std::vector<long long> tile0(ni + 1), woff(ni + 1), part0(ni + 1), npts(ni);
+    std::vector<int> out0(ni + 1);
+    tile0[0] = woff[0] = part0[0] = 0;
+    out0[0] = 0;
     for (size_t q = 0; q < ni; ++q) {
-        const size_t u = ord[q];
-        const GridReq& g = rs.grids[pairs[u].first];
+        const LagGroup& gr = groups[ord[q]];
+        const GridReq& g = rs.grids[ids[gr.first]];
         const int nsig = rs.specs[g.spec].nsig;
         long long pts = g.L[0] + 1;
         for (int k = 1; k < d; ++k) pts *= 2 * g.L[k] + 1;
         npts[q] = pts;
-        const int N = lag_table_size(d, Re[u], dbl);
-        tile0[q + 1] = tile0[q] + (pts + T - 1) / T;
-        woff[q + 1] = woff[q] + 2LL * nsig * N;
-        if (bt.classes.empty() || bt.classes.back()[0] != Re[u]) bt.classes.push_back({Re[u], (int)tile0[q], 0});
-        bt.classes.back()[2] += (int)(tile0[q + 1] - tile0[q]);
-        bt.fl += (double)pts * nsig * (2.0 * d * d + 8.0 * N);
+        int N = 1;   // Hermite values
+        for (int i = 1; i <= d; ++i) N = N * (gr.R + i) / i;
+        const long long nt = (pts + T - 1) / T;
+        tile0[q + 1] = tile0[q] + nt;
+        part0[q + 1] = part0[q] + nt * (dbl ? kLagSlices : 1) * gr.sums();
+        woff[q + 1] = woff[q] + (long long)nsig * (gr.nv < 0 ? 2 * N : gr.sums());
+        out0[q + 1] = out0[q] + gr.n;
+        if (bt.classes.empty() || bt.classes.back()[0] != gr.R || bt.classes.back()[1] != gr.nv)
+            bt.classes.push_back({gr.R, gr.nv, (int)tile0[q], 0});
+        bt.classes.back()[3] += (int)nt;
+        bt.fl += (double)pts * (nsig * (2.0 * d * d + 3.0 * N) + 12.0 * gr.n);
         bt.by += (double)pts * sizeof(real);
-        bt.pairs.push_back(pairs[u]);
+        bt.grids.insert(bt.grids.end(), ids.begin() + gr.first, ids.begin() + gr.first + gr.n);
     }
     if (tile0[ni] > 0x7fffffffLL || woff[ni] > 0x7fffffffLL)
         return fail(KDEFFT_ERR_UNSUPPORTED, "lag batch too large");
+    bt.nslots = (size_t)part0[ni];
     items.resize(ni);
     bt.tiles.resize((size_t)tile0[ni]);
     wpool.assign((size_t)woff[ni], real(0));
-    // inverse covariances and normalisations once per kernel spec (the pairs
-    // of one bandwidth share them), then the items: both over index ranges
-    // that may run on several host threads (each writes its own entries;
-    // the result does not depend on the split)
-    struct SpecInv {
-        double lam[MAXSIG][MAXD * MAXD];
-        double nrm[MAXSIG];
-    };
-    std::vector<char> used(rs.specs.size(), 0);
-    for (size_t q = 0; q < ni; ++q) used[rs.grids[pairs[ord[q]].first].spec] = 1;
-    std::vector<SpecInv> sinv(rs.specs.size());
+    // the items, with the inverse covariances and normalisations of their
+    // kernel spec, over index ranges that may run on several host threads
+    // (each writes its own entries; the result does not depend on the split)
     std::atomic<int> err{KDEFFT_OK};
-    host_parallel_for(rs.specs.size(), 2048, [&](size_t s0, size_t s1) {
-        for (size_t si = s0; si < s1; ++si) {
-            if (!used[si]) continue;
-            const KSpec& sp = rs.specs[si];
-            for (int s = 0; s < sp.nsig; ++s) {
-                Mat inv;
-                double det;
-                if (!spd_inv_det(sp.sig[s], inv, det)) {
-                    err = KDEFFT_ERR_NOT_SPD;
-                    return;
-                }
-                for (int a = 0; a < d; ++a)
-                    for (int b = 0; b < d; ++b) sinv[si].lam[s][a * MAXD + b] = inv(a, b);
-                sinv[si].nrm[s] = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
-            }
-        }
-    });
-    if (err != KDEFFT_OK) return fail(KDEFFT_ERR_NOT_SPD, "a kernel covariance is not positive definite");
-    host_parallel_for(ni, 2048, [&](size_t q0, size_t q1) {
+    host_parallel_for(ni, 1024, [&](size_t q0, size_t q1) {
+        int last = -1;   // dense pairs of a spec follow one another
         for (size_t q = q0; q < q1; ++q) {
-            const size_t u = ord[q];
-            const auto& pr = pairs[u];
-            const GridReq& g = rs.grids[pr.first];
+            const LagGroup& gr = groups[ord[q]];
+            const GridReq& g = rs.grids[ids[gr.first]];
             const KSpec& sp = rs.specs[g.spec];
             kdefft_ds ds = g.ds;
             LagItem<real>& it = items[q];
             std::memset(&it, 0, sizeof(it));
             it.d = d;
             it.nsig = sp.nsig;
-            it.R = Re[u];
+            it.R = gr.R;
             for (int k = 0; k < d; ++k) {
                 it.L[k] = g.L[k];
                 it.A[k] = ds->acA[k];
                 it.delta[k] = (real)ds->delta[k];
                 invariant_div((uint32_t)(k == 0 ? g.L[0] + 1 : 2 * g.L[k] + 1), it.qm[k], it.qs[k]);
             }
-            const SpecInv& si = sinv[g.spec];
-            for (int s = 0; s < sp.nsig; ++s) {
-                for (int a = 0; a < d; ++a)
-                    for (int b = 0; b < d; ++b) it.lam[s][a * MAXD + b] = (real)si.lam[s][a * MAXD + b];
-                it.nrm[s] = (real)si.nrm[s];
+            if (g.spec == last) {
+                std::memcpy(it.lam, items[q - 1].lam, sizeof(it.lam));
+                std::memcpy(it.nrm, items[q - 1].nrm, sizeof(it.nrm));
+            } else {
+                for (int s = 0; s < sp.nsig; ++s) {
+                    Mat inv;
+                    double det;
+                    if (!spd_inv_det(sp.sig[s], inv, det)) {
+                        err = KDEFFT_ERR_NOT_SPD;
+                        return;
+                    }
+                    for (int a = 0; a < d; ++a)
+                        for (int b = 0; b < d; ++b) it.lam[s][a * MAXD + b] = (real)inv(a, b);
+                    it.nrm[s] = (real)(std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det));
+                }
+                last = g.spec;
             }
             it.acorr = dbl ? (const real*)ds->ac64.p : (const real*)ds->ac32.p;
-            const int N = lag_table_size(d, it.R, dbl);
             it.w_off = (int)woff[q];
-            const int gi[2] = {pr.first, pr.second};
-            for (int h = 0; h < 2; ++h) {
-                if (gi[h] < 0) continue;
-                for (const Term& t : rs.grids[gi[h]].terms) {
+            int N = 1;
+            for (int i = 1; i <= d; ++i) N = N * (gr.R + i) / i;
+            for (int h = 0; h < gr.n; ++h)
+                for (const Term& t : rs.grids[ids[gr.first + h]].terms) {
+                    it.sigs |= 1 << t.sig;
+                    if (gr.nv >= 0) {   // even orders: no sign
+                        wpool[it.w_off + h * sp.nsig + t.sig] += (real)t.w;
+                        continue;
+                    }
                     int o = 0;
                     for (int k = 0; k < d; ++k) o += t.alpha[k];
                     const int hidx = hx.idx(d, t.alpha);
@@ -2408,40 +2467,39 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, std::vector<std::pair<int, int>> pa
                     }
                     wpool[it.w_off + (h * sp.nsig + t.sig) * N + hidx] += (real)(((o & 1) ? -1.0 : 1.0) * t.w);
                 }
-            }
             const double nn = (double)ds->n;
             it.scale = 1.0 / (nn * nn);
             it.tile0 = (int)tile0[q];
             it.ntile = (int)(tile0[q + 1] - tile0[q]);
+            it.part0 = part0[q];
+            it.nout = gr.n;
+            it.out0 = out0[q];
             const long long pts = npts[q];
             long long f = 0;
             for (long long tq = tile0[q]; tq < tile0[q + 1]; ++tq, f += T)
                 bt.tiles[tq] = LagTile{(int)q, (int)std::min(T, pts - f), f};
         }
     });
+    if (err == KDEFFT_ERR_NOT_SPD) return fail(KDEFFT_ERR_NOT_SPD, "a kernel covariance is not positive definite");
     if (err != KDEFFT_OK) return fail(KDEFFT_ERR_UNSUPPORTED, "derivative order too high");
     bt.nitems = (int)items.size();
     out.push_back(std::move(bt));
     return KDEFFT_OK;
 }
 
-// Upload the lag batches of a run in one copy and launch them (one tiled
-// launch per batch and derivative-order class, then one fixed-order sum of
-// every item's tile partials), then one copy of all values back; the values
-// are read by flush_reads.
+// Upload the lag batches of a run in one copy (their items, tiles, weights and
+// zeroed counters) and launch them, one launch per batch and form; each item's
+// last block writes its results to pinned host memory, from where flush_reads
+// takes them.
 static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
     if (bts.empty()) return KDEFFT_OK;
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     struct Lay {
-        size_t oI, oT, oW;
-        int item0;
-        long long tile0;   // first partial pair of the batch
+        size_t oI, oT, oW, oD;
+        size_t out0, slot0;   // the batch's first result and first partial sum
     };
     std::vector<Lay> lay(bts.size());
-    size_t bytes = 0;
-    int nit = 0;
-    long long ntl = 0;   // partial pairs of the run
-    std::vector<LagSum> sums;
+    size_t bytes = 0, need = 0, slots = 0;
     for (size_t b = 0; b < bts.size(); ++b) {
         const LagBatch& bt = bts[b];
         lay[b].oI = bytes;
@@ -2450,34 +2508,18 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
         bytes += al(sizeof(LagTile) * bt.tiles.size());
         lay[b].oW = bytes;
         bytes += al(std::max<size_t>(bt.w_size(), 16));
-        lay[b].item0 = nit;
-        lay[b].tile0 = ntl;
-        const int ps = bt.dbl ? kLagSlices : 1;   // partial pairs per tile
-        for (int i = 0; i < bt.nitems; ++i) {
-            // the item's tile range and scale, wherever its precision keeps them
-            int t0i, nti;
-            double sc;
-            if (bt.dbl) {
-                const LagItem<double>& q = bt.it64[i];
-                t0i = q.tile0, nti = q.ntile, sc = q.scale;
-            } else {
-                const LagItem<float>& q = bt.it32[i];
-                t0i = q.tile0, nti = q.ntile, sc = q.scale;
-            }
-            sums.push_back(LagSum{ntl + (long long)t0i * ps, nti, ps, sc});
-        }
-        nit += bt.nitems;
-        ntl += (long long)bt.tiles.size() * ps;
+        lay[b].oD = bytes;
+        bytes += al(sizeof(unsigned int) * bt.nitems);
+        lay[b].out0 = need;
+        lay[b].slot0 = slots;
+        need += bt.grids.size();
+        slots += bt.nslots;
     }
-    const size_t oS = bytes;
-    bytes += al(sizeof(LagSum) * sums.size());
     KCHK(staging_wait(c));
     KCHK(c->h_items.ensure(bytes));
     KCHK(c->items.ensure(bytes));
-    KCHK(c->partial.ensure(sizeof(double) * 2 * (size_t)ntl));
-    KCHK(c->out.ensure(sizeof(double) * 2 * (size_t)nit));
+    KCHK(c->partial.ensure(sizeof(double) * slots));
     // results go behind those of earlier lag launches still on their way
-    const size_t need = 2 * (size_t)nit;
     if (c->h_out.cap < sizeof(double) * (c->hout_used + need)) {
         // (the results still on their way point into h_out: read them first;
         // grow by at least 4x, so that the next chunks of a large run fit)
@@ -2489,23 +2531,23 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
     unsigned char* h = (unsigned char*)c->h_items.p;
     unsigned char* dbase = (unsigned char*)c->items.p;
     double* part = (double*)c->partial.p;
-    double* dout = (double*)c->out.p;
-    std::memcpy(h + oS, sums.data(), sizeof(LagSum) * sums.size());
+    double* hout = (double*)c->h_out.p + off;
     std::vector<long long> sig = {3, (long long)(uintptr_t)dbase, (long long)(uintptr_t)h, (long long)bytes,
-                                  (long long)(uintptr_t)part, (long long)(uintptr_t)dout, (long long)oS, nit,
-                                  (long long)(uintptr_t)c->h_out.p, (long long)off};
+                                  (long long)(uintptr_t)part, (long long)(uintptr_t)hout};
     for (size_t b = 0; b < bts.size(); ++b) {
         const LagBatch& bt = bts[b];
         std::memcpy(h + lay[b].oI, bt.item_bytes(), bt.item_size());
         std::memcpy(h + lay[b].oT, bt.tiles.data(), sizeof(LagTile) * bt.tiles.size());
         if (bt.w_size()) std::memcpy(h + lay[b].oW, bt.w_bytes(), bt.w_size());
+        std::memset(h + lay[b].oD, 0, sizeof(unsigned int) * bt.nitems);
         sig.insert(sig.end(), {bt.dbl ? 8 : 4, bt.d, bt.nitems, (long long)bt.tiles.size(), (long long)lay[b].oI,
-                               (long long)lay[b].oT, (long long)lay[b].oW, lay[b].item0, lay[b].tile0});
-        for (const auto& cl : bt.classes) sig.insert(sig.end(), {cl[0], cl[1], cl[2]});
+                               (long long)lay[b].oT, (long long)lay[b].oW, (long long)lay[b].oD,
+                               (long long)lay[b].out0, (long long)lay[b].slot0});
+        for (const auto& cl : bt.classes) sig.insert(sig.end(), {cl[0], cl[1], cl[2], cl[3]});
     }
     // a run with batches of both precisions launches its FP64 batch on the
-    // side stream, beside the FP32 one (the two touch disjoint partials;
-    // k_lag_sum joins them); not while profiling, whose events time the
+    // side stream, beside the FP32 one (the two touch disjoint partials,
+    // counters and results); not while profiling, whose events time the
     // launches one after another on the main stream
     bool has32 = false, has64 = false;
     for (const LagBatch& bt : bts) (bt.dbl ? has64 : has32) = true;
@@ -2515,8 +2557,8 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
         if (!c->fork_ev) KCU(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
         if (!c->join_ev) KCU(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
     }
-    // the upload from pinned staging, the launches and the copy back replay
-    // as one graph (the copy reads the staging buffer when the graph runs)
+    // the upload from pinned staging and the launches replay as one graph (the
+    // copy reads the staging buffer when the graph runs)
     auto issue = [&]() -> int {
         KCU(cudaMemcpyAsync(dbase, h, bytes, cudaMemcpyHostToDevice, c->stream));
         // the staging buffer is free again once this copy is done (inside a
@@ -2537,42 +2579,35 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
             const cudaStream_t ls = (fork && bt.dbl) ? c->side : c->stream;
             for (const auto& cl : bt.classes) {
                 cudaEvent_t ev = prof_start(c);
-                if (bt.dbl) {
-                    // fewer tiles than SMs: a warp slice per CTA, so that the
-                    // FP64 points spread over kLagSlices times as many SMs
-                    const bool sl = cl[2] < c->nsm;
-                    const LagJob<double> j{(const LagItem<double>*)(dbase + lay[b].oI), (const LagTile*)(dbase + lay[b].oT),
-                                           cl[1], cl[2], sl ? cl[2] * kLagSlices : std::min(cl[2], c->nsm * 8),
-                                           sl ? 32 : 256, (const double*)(dbase + lay[b].oW),
-                                           part + 2 * (size_t)lay[b].tile0};
-                    KCU(launch_lag<double>(bt.d, cl[0], j, ls));
-                } else {
-                    const LagJob<float> j{(const LagItem<float>*)(dbase + lay[b].oI), (const LagTile*)(dbase + lay[b].oT),
-                                          cl[1], cl[2], std::min(cl[2], c->nsm * 8), 256,
-                                          (const float*)(dbase + lay[b].oW), part + 2 * (size_t)lay[b].tile0};
-                    KCU(launch_lag<float>(bt.d, cl[0], j, ls));
-                }
-                prof_stop(c, ev, bt.dbl ? "lag_f64" : "lag_f32", bt.by * cl[2] / nt, bt.fl * cl[2] / nt);
+                auto go = [&](auto zero) -> cudaError_t {
+                    using real = decltype(zero);
+                    // FP64, fewer tiles than SMs: a warp slice per CTA, so that
+                    // the points spread over kLagSlices times as many SMs (with
+                    // more tiles the extra CTAs cost more than they balance: 36 ->
+                    // 40 us for 16 SCV bandwidths on 256^2, 31 -> 46 us in 3-D)
+                    const bool sl = sizeof(real) == 8 && cl[3] < c->nsm;
+                    const LagJob<real> j{(const LagItem<real>*)(dbase + lay[b].oI), (const LagTile*)(dbase + lay[b].oT),
+                                         cl[2], cl[3], sl ? cl[3] * kLagSlices : std::min(cl[3], c->nsm * 8),
+                                         sl ? 32 : 256, (const real*)(dbase + lay[b].oW), part + lay[b].slot0,
+                                         (unsigned int*)(dbase + lay[b].oD), hout + lay[b].out0};
+                    return launch_lag<real>(bt.d, cl[0], cl[1], j, ls);
+                };
+                KCU(bt.dbl ? go(0.0) : go(0.f));
+                prof_stop(c, ev, bt.dbl ? "lag_f64" : "lag_f32", bt.by * cl[3] / nt, bt.fl * cl[3] / nt);
             }
         }
         if (fork) {
             KCU(cudaEventRecord(c->join_ev, c->side));
             KCU(cudaStreamWaitEvent(c->stream, c->join_ev, 0));
         }
-        cudaEvent_t es = prof_start(c);
-        KCU(launch_lag_sum((const LagSum*)(dbase + oS), nit, part, dout, c->stream));
-        prof_stop(c, es, "lag_sum", 16.0 * ntl, 2.0 * ntl);
-        KCU(cudaMemcpyAsync((double*)c->h_out.p + off, dout, sizeof(double) * need, cudaMemcpyDeviceToHost, c->stream));
         return KDEFFT_OK;
     };
     KCHK(run_graph(c, sig, issue));
     c->staging_free = false;
     c->h2d += (int64_t)bytes;
     c->d2h += (int64_t)(sizeof(double) * need);
-    for (size_t b = 0; b < bts.size(); ++b) {
-        kdefft_ctx_s::PendingRead pr{&rs, std::move(bts[b].pairs), off + 2 * (size_t)lay[b].item0};
-        c->pend_reads.push_back(std::move(pr));
-    }
+    for (size_t b = 0; b < bts.size(); ++b)
+        c->pend_reads.push_back({&rs, std::move(bts[b].grids), off + lay[b].out0});
     c->hout_used += need;
     bts.clear();
     prof_flush(c);
@@ -2675,37 +2710,39 @@ static int run_requests(kdefft_ctx c, ReqSet& rs, const std::vector<int>& sel, s
     if (sel.empty()) return KDEFFT_OK;
     const int d = rs.grids[sel[0]].ds->d;
     HermiteIndex& hx = hindex();
-    // pair consecutive selected grids that share dataset, covariances and plan
+    // consecutive selected grids that share dataset, covariances and plan: in
+    // groups through the lag-domain engine where it covers them, in pairs
+    // through the FFT route otherwise
     std::vector<std::pair<int, int>> pairs;
+    std::vector<LagGroup> groups;
     for (size_t u = 0; u < sel.size();) {
         const GridReq& a = rs.grids[sel[u]];
-        if (u + 1 < sel.size()) {
-            const GridReq& b = rs.grids[sel[u + 1]];
-            if (b.ds == a.ds && b.spec == a.spec && std::memcmp(a.L, b.L, sizeof(a.L)) == 0 &&
-                std::memcmp(a.P, b.P, sizeof(a.P)) == 0) {
-                pairs.push_back({sel[u], sel[u + 1]});
-                u += 2;
-                continue;
-            }
+        size_t v = u + 1;
+        while (v < sel.size()) {
+            const GridReq& b = rs.grids[sel[v]];
+            if (b.ds != a.ds || b.spec != a.spec || std::memcmp(a.L, b.L, sizeof(a.L)) != 0 ||
+                std::memcmp(a.P, b.P, sizeof(a.P)) != 0)
+                break;
+            ++v;
         }
-        pairs.push_back({sel[u], -1});
-        u += 1;
+        if (lag_covers(c, a))
+            lag_groups(rs, sel, (int)u, (int)v, sizeof(real) == 8, groups, pairs);
+        else
+            for (size_t i = u; i < v; i += 2) pairs.push_back({sel[i], i + 1 < v ? sel[i + 1] : -1});
+        u = v;
     }
     const int cap = cap_elems(sizeof(real) == 8);
-    // lag-domain engine for the pairs it covers; the FFT route for the rest
-    {
-        std::vector<std::pair<int, int>> lagp, fftp;
-        for (const auto& pr : pairs) (lag_eligible<real>(c, rs, pr) ? lagp : fftp).push_back(pr);
-        if (!lagp.empty()) {
-            const int lr = run_lag<real>(c, rs, lagp, lagq);
-            if (lr == KDEFFT_ERR_UNSUPPORTED)
-                fftp.insert(fftp.end(), lagp.begin(), lagp.end());   // autocorrelation box beyond MAXP
-            else
-                KCHK(lr);
+    if (!groups.empty()) {
+        const int lr = run_lag<real>(c, rs, sel, groups, lagq);
+        if (lr == KDEFFT_ERR_UNSUPPORTED) {   // autocorrelation box beyond MAXP
+            for (const LagGroup& gr : groups)
+                for (int i = gr.first; i < gr.first + gr.n; i += 2)
+                    pairs.push_back({sel[i], i + 1 < gr.first + gr.n ? sel[i + 1] : -1});
+        } else {
+            KCHK(lr);
         }
-        pairs.swap(fftp);
-        if (pairs.empty()) return KDEFFT_OK;
     }
+    if (pairs.empty()) return KDEFFT_OK;
     // count spectra first, all missing ones in one launch sequence
     {
         HostTimer hs(c, "host:spectra");
@@ -3767,6 +3804,7 @@ static int scv_requests(ReqSet& rs, kdefft_ds ds, const double* H, int nH, const
             std::memcpy(g.L, g0.L, sizeof(g.L));
             std::memcpy(g.P, g0.P, sizeof(g.P));
             g.terms = {Term{0, {0}, 1.0}};
+            g.order = 0;
             g.fp64 = true;
             missing[keys[h]] = (int)rs.grids.size();
             rs.grids.push_back(std::move(g));

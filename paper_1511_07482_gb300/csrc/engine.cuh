@@ -228,8 +228,8 @@ cudaError_t prepare_kernels();
 // The autocorrelation array holds the half box of a larger box A, layout
 // [j_{d-1}]..[j_1][j_0] (j_0 innermost, j_k + A_k for k >= 1).
 template <typename real>
-struct LagItem {
-    int d, nsig, R, pad_;
+struct LagItem {                      // a group of kernels that share covariances and support
+    int d, nsig, R, sigs;             // sigs: bit s set where covariance s has a weight
     int L[MAXD];                      // support of this item's kernels
     int A[MAXD];                      // box of the autocorrelation array
     // division of a flat half-box index by the extents L_0 + 1, 2 L_k + 1
@@ -240,9 +240,11 @@ struct LagItem {
     real lam[MAXSIG][MAXD * MAXD];    // Sigma^{-1}, row stride MAXD
     real nrm[MAXSIG];                 // (2 pi)^{-d/2} |Sigma|^{-1/2}
     real delta[MAXD];
+    int w_off;                        // weights at wpool + w_off: [kernel][nsig], or dense [2][nsig][N(d, R)]
     const real* acorr;
-    int w_off;                        // dense weights [2][nsig][N(d, R)] at wpool + w_off
-    int tile0, ntile;                 // this item's tiles (their partial sums)
+    long long part0;                  // its partials at partial + part0: [slot][kernel]
+    int tile0, ntile;                 // this item's tiles (FP64: kLagSlices slots each, else one)
+    int nout, out0;                   // its kernels, and the first of their results
     double scale;                     // n^-2
 };
 struct LagTile {
@@ -250,18 +252,19 @@ struct LagTile {
     int n;                            // points of the item's half box in this tile
     long long first;                  // first flat index (j_0 fastest)
 };
-// Number of Hermite entries C(d + R, d) of the compile-time tables, or 0 when
-// no lag kernel is instantiated for (d, R, real) (the caller uses the FFT path).
+// Number of Hermite entries C(d + R, d) of the dense kernels' tables, or 0 when
+// none is instantiated for (d, R, real) (the caller uses the FFT path).
 int lag_table_size(int d, int R, bool dbl);
+// Is there a kernel for a group of nv Gaussians and (R > 0) all partials of
+// order R, each a weighted sum over nsig covariances?
+bool lag_single_form(int d, int R, int nv, int nsig);
 // One launch of the lag kernel over tiles [t0, t0 + ntiles) of a batch (one
-// derivative-order class): items, tiles and weights of the batch, partial
-// (2 per tile of the batch).
-// FP64 lag tiles hold 32 * kLagSlices points, one per thread, in kLagSlices
-// warp slices; each slice writes its own partial pair (kLagSlices per tile),
-// which k_lag_sum combines in a fixed order.  So a launch may run one slice
-// per 32-thread CTA (few tiles: the slow FP64 points spread over the SMs) or
-// a whole tile per 256-thread CTA, with the same bits.  FP32 tiles write one
-// partial pair each.
+// form): items, tiles and weights of the batch.  FP64 lag tiles hold
+// 32 * kLagSlices points, one per thread, in kLagSlices warp slices, so a
+// launch may run one slice per 32-thread CTA (few tiles: the slow FP64 points
+// spread over the SMs) or a whole tile per 256-thread CTA, with the same bits.
+// done: a counter per item, zero; out: the results (device memory, or host
+// memory that the device can write).
 constexpr int kLagSlices = 8;
 template <typename real>
 struct LagJob {
@@ -270,19 +273,13 @@ struct LagJob {
     int t0, ntiles, grid;
     int block;                        // 256; FP64 also 32, 64 or 128 (slices per CTA = block / 32)
     const real* wpool;
-    double* partial;                  // per tile of the batch: 1 pair (FP32) or kLagSlices pairs (FP64)
+    double* partial;
+    unsigned int* done;
+    double* out;
 };
+// nv < 0: the dense form (two kernels of any partials up to order R)
 template <typename real>
-cudaError_t launch_lag(int d, int R, const LagJob<real>& j, cudaStream_t st);
-// An item's tile partials (tile0 indexes the run's whole partial buffer, in
-// pairs) and its scale n^-2: the per-item sums of a run, whatever the
-// batch's precision.
-struct LagSum {
-    long long tile0;                  // first partial pair of the item's first tile
-    int ntile, nslice;                // tiles; partial pairs per tile (1 or kLagSlices)
-    double scale;
-};
-cudaError_t launch_lag_sum(const LagSum* sums, int nitems, const double* partial, double* out, cudaStream_t st);
+cudaError_t launch_lag(int d, int R, int nv, const LagJob<real>& j, cudaStream_t st);
 // One pass of the count autocorrelation along one axis, for one dataset: O I
 // lines, each a transform of length P of X input values (zero-extended), of
 // which Y results are kept.  Element (o, x, i) of the input lies at
