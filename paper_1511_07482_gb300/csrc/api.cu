@@ -615,6 +615,7 @@ struct kdefft_ctx_s {
     DevBuf acjobs;            // job table of the batched autocorrelation passes
     HostBuf h_acjobs;         // its pinned staging copy, free once acjobs_ev has passed
     HostBuf h_sel;            // pinned start / end table of the lag-domain device search
+    HostBuf h_mix;            // pinned components and results of the mixture term
     HostBuf h_binres;         // pinned outside count and moment partials of a binning
     cudaEvent_t acjobs_ev = nullptr;
     bool acjobs_free = true;
@@ -3256,6 +3257,7 @@ int kdefft_destroy(kdefft_ctx c) {
     c->h_acjobs.release();
     c->h_sel.release();
     c->h_binres.release();
+    c->h_mix.release();
     if (c->errflag) cudaFree(c->errflag);
     delete c;
     return KDEFFT_OK;
@@ -4076,40 +4078,56 @@ int kdefft_ise_mixture(kdefft_ds ds, const double* H, int nH, int K, const doubl
         KCHK(sym_check(H + (size_t)h * d * d, d, Hs[h], "H"));
         KCHK(add_eta_m(rs, ds, scaled(2.0, Hs[h]), 0, first[h]));
     }
-    KCHK(run(c, rs));
-    // int f_hat f = n^-1 sum_g c_g sum_m w_m phi_{H + S_m}(x_g - mu_m)
-    const KdeDesc g = kde_desc(ds, nullptr);
-    const int nb = std::max(1, std::min(c->nsm * 4, (int)((ds->ncells + 255) / 256)));
-    const size_t bc = (sizeof(MixComp) * K + 255) & ~(size_t)255;
-    KCHK(c->kdebuf.ensure(bc + sizeof(double) * nb));
-    MixComp* dcomp = (MixComp*)c->kdebuf.p;
-    double* dpart = (double*)((unsigned char*)c->kdebuf.p + bc);
-    std::vector<double> v(nH), part(nb);
-    for (int h = 0; h < nH; ++h) {
-        std::vector<MixComp> comps(K);
-        for (int m = 0; m < K; ++m) {
-            std::memset(&comps[m], 0, sizeof(MixComp));
-            const Mat Sc = lin(1.0, Hs[h], 1.0, Sm[m]);
-            Mat inv;
-            double det;
-            spd_inv_det(Sc, inv, det);
-            for (int k = 0; k < d; ++k) comps[m].mu[k] = mu[(size_t)m * d + k];
-            for (int a = 0; a < d; ++a)
-                for (int b = 0; b < d; ++b) comps[m].lam[a * MAXD + b] = inv(a, b);
-            comps[m].nrm = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
-            comps[m].w = w[m];
-        }
-        KCU(cudaMemcpyAsync(dcomp, comps.data(), sizeof(MixComp) * K, cudaMemcpyHostToDevice, c->stream));
+    // int f_hat f = n^-1 sum_g c_g sum_m w_m phi_{H + S_m}(x_g - mu_m): a launch
+    // for all bandwidths (whose component tables stay below 32 MB), ahead of
+    // the lag launches, whose wait covers both
+    const int chunk = (int)std::max<long long>(1, std::min<long long>(nH, (32LL << 20) / ((long long)sizeof(MixComp) * K)));
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t oD = al(sizeof(MixComp) * K * chunk), up = oD + al(sizeof(unsigned int) * chunk);
+    MixJob mj;
+    std::memset(&mj, 0, sizeof(mj));
+    mj.counts = (const float*)ds->counts.p;
+    mj.g = kde_desc(ds, nullptr);
+    mj.ncomp = K;
+    mj.nb = (int)std::max<long long>(1, std::min<long long>((ds->ncells + 255) / 256, (8LL * c->nsm + nH - 1) / nH));
+    KCHK(c->kdebuf.ensure(up + sizeof(double) * (size_t)mj.nb * chunk));
+    KCHK(c->h_mix.ensure(up + sizeof(double) * chunk));
+    unsigned char* hb = (unsigned char*)c->h_mix.p;
+    unsigned char* db = (unsigned char*)c->kdebuf.p;
+    mj.comps = (const MixComp*)db;
+    mj.done = (unsigned int*)(db + oD);
+    mj.partial = (double*)(db + up);
+    mj.out = (double*)(hb + up);
+    std::vector<double> v(nH);
+    for (int h0 = 0; h0 < nH; h0 += chunk) {
+        const int nh = std::min(chunk, nH - h0);
+        std::memset(hb, 0, up);
+        for (int h = 0; h < nh; ++h)
+            for (int m = 0; m < K; ++m) {
+                MixComp& mc = ((MixComp*)hb)[(size_t)h * K + m];
+                const Mat Sc = lin(1.0, Hs[h0 + h], 1.0, Sm[m]);
+                Mat inv;
+                double det;
+                spd_inv_det(Sc, inv, det);
+                for (int k = 0; k < d; ++k) mc.mu[k] = mu[(size_t)m * d + k];
+                for (int a = 0; a < d; ++a)
+                    for (int b = 0; b < d; ++b) mc.lam[a * MAXD + b] = inv(a, b);
+                mc.nrm = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
+                mc.w = w[m];
+            }
+        KCU(cudaMemcpyAsync(db, hb, up, cudaMemcpyHostToDevice, c->stream));
+        c->h2d += (int64_t)up;
         cudaEvent_t ev = prof_start(c);
-        KCU(launch_mix_dot((const float*)ds->counts.p, g, dcomp, K, dpart, nb, c->stream));
-        prof_stop(c, ev, "mix_dot", 4.0 * (double)ds->ncells, 12.0 * (double)ds->ncells * K);
-        KCU(cudaMemcpyAsync(part.data(), dpart, sizeof(double) * nb, cudaMemcpyDeviceToHost, c->stream));
-        KCU(cudaStreamSynchronize(c->stream));
-        double cross = 0.0;
-        for (int b = 0; b < nb; ++b) cross += part[b];
-        cross /= (double)ds->n;
-        v[h] = rs.grids[first[h]].value - 2.0 * cross + ff;
+        KCU(launch_mix_dot(mj, nh, c->stream));
+        prof_stop(c, ev, "mix_dot", 4.0 * (double)ds->ncells * nh, 12.0 * (double)ds->ncells * K * nh);
+        int rr = KDEFFT_OK;
+        if (h0 + nh == nH) rr = run(c, rs);
+        KCU(cudaStreamSynchronize(c->stream));   // the pinned table and results, whatever run did
+        KCHK(rr);
+        c->d2h += (int64_t)(sizeof(double) * nh);
+        for (int h = 0; h < nh; ++h) v[h0 + h] = mj.out[h] / (double)ds->n;
     }
+    for (int h = 0; h < nH; ++h) v[h] = rs.grids[first[h]].value - 2.0 * v[h] + ff;
     prof_flush(c);
     return write_out(c, out, v.data(), v.size());
 }

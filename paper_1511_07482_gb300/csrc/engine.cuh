@@ -354,9 +354,20 @@ cudaError_t launch_kde_table(const KdeDesc& g, const KdeKernel& kn, float* tab, 
 // last axis fastest); counts FP32
 cudaError_t launch_kde_grid(const float* counts, const KdeDesc& g, const float* ktab, double* out, int nsm,
                             cudaStream_t st);
-// partial[b] (b < nblocks) = block b's share of sum_g c_g sum_m (comps[m] at x_g)
-cudaError_t launch_mix_dot(const float* counts, const KdeDesc& g, const MixComp* comps, int ncomp, double* partial,
-                           int nblocks, cudaStream_t st);
+// out[h] = sum_g c_g sum_m (comps[h ncomp + m] at x_g) for nH mixtures of ncomp
+// components, nb blocks each (partial: nH nb values; done: nH zeros; out: device
+// memory, or host memory that the device can write)
+constexpr int kMixMax = 64;
+struct MixJob {
+    const float* counts;
+    KdeDesc g;
+    const MixComp* comps;
+    int ncomp, nb;
+    double* partial;
+    unsigned int* done;
+    double* out;
+};
+cudaError_t launch_mix_dot(const MixJob& j, int nH, cudaStream_t st);
 
 // Binning (binning.cu).  Grid node k along axis a is lo[a] + k delta[a],
 // k < M[a].  Counts accumulate into `counts` (zeroed by the caller);

@@ -9,8 +9,8 @@
 //             FP64.  The direct sum keeps the relative accuracy of small
 //             values (and exact zeros beyond the support), which a transform
 //             does not.
-//   mix_dot   sum_g c_g sum_m w_m phi_{S_m}(x_g - mu_m) (FP64), one FP64
-//             partial per block, summed in block order by the host.
+//   mix_dot   sum_g c_g sum_m w_m phi_{S_m}(x_g - mu_m) (FP64) for a batch of
+//             mixtures.
 #include "devutil.cuh"
 #include "engine.cuh"
 
@@ -331,46 +331,90 @@ cudaError_t launch_kde_grid(const float* counts, const KdeDesc& g, const float* 
     return kde_go<2, 8, 4, 4>(counts, g, ktab, out, st);
 }
 
-__global__ void __launch_bounds__(256) k_mix_dot(const float* __restrict__ counts, KdeDesc g,
-                                                 const MixComp* __restrict__ comps, int ncomp,
-                                                 double* __restrict__ partial) {
-    const int d = g.d;
+// sum_g c_g sum_m w_m phi_{S_m}(x_g - mu_m) for many mixtures (one per
+// bandwidth), nb blocks each: block b of mixture h takes the cells b, b + nb,
+// ... in steps of a block.  Bound by the FP64 pipe (an exponential and a
+// quadratic form per component and cell with counts, about 35 operations), so
+// all mixtures are one launch that fills the SMs; the mixture's last block adds
+// its nb partials in block order.
+// 32 bandwidths, three components, a 101^2 grid: 55 us (512 us in 32 launches,
+// with an upload, a copy back and a host wait each: the call 953 -> 98 us).
+template <int D>
+__global__ void __launch_bounds__(256) k_mix_dot(const __grid_constant__ MixJob jb) {
+    __shared__ double mu[kMixMax][D], lam[kMixMax][D * D], amp[kMixMax];
+    __shared__ double red[8];
+    __shared__ int lastone;
+    const KdeDesc& g = jb.g;
+    const int h = blockIdx.x / jb.nb, b = blockIdx.x % jb.nb, K = jb.ncomp;
+    const MixComp* comps = jb.comps + (long long)h * K;
+    for (int m = threadIdx.x; m < K; m += blockDim.x) {
+        for (int k = 0; k < D; ++k) mu[m][k] = comps[m].mu[k];
+        for (int k = 0; k < D * D; ++k) lam[m][k] = comps[m].lam[(k / D) * MAXD + k % D];
+        amp[m] = comps[m].w * comps[m].nrm;
+    }
+    __syncthreads();
     double acc = 0.0;
-    for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < g.ncells;
-         cell += (long long)gridDim.x * blockDim.x) {
-        const float cv = counts[cell];
+    for (long long cell = (long long)b * blockDim.x + threadIdx.x; cell < g.ncells; cell += (long long)jb.nb * blockDim.x) {
+        const float cv = jb.counts[cell];
         if (cv == 0.f) continue;
-        double x[MAXD] = {0.0, 0.0, 0.0, 0.0};
+        double x[D];
         {
             long long r = cell;
-            for (int k = d - 1; k >= 0; --k) {
+#pragma unroll
+            for (int k = D - 1; k >= 0; --k) {
                 const int i = (int)(r % g.M[k]);
                 r /= g.M[k];
                 x[k] = g.lo[k] + g.delta[k] * (double)i;
             }
         }
         double f = 0.0;
-        for (int m = 0; m < ncomp; ++m) {
-            const MixComp& c = comps[m];
-            double z[MAXD], q = 0.0;
-            for (int k = 0; k < d; ++k) z[k] = x[k] - c.mu[k];
-            for (int a = 0; a < d; ++a) {
+        for (int m = 0; m < K; ++m) {
+            double z[D], q = 0.0;
+#pragma unroll
+            for (int k = 0; k < D; ++k) z[k] = x[k] - mu[m][k];
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
                 double t = 0.0;
-                for (int b = 0; b < d; ++b) t += c.lam[a * MAXD + b] * z[b];
-                q += z[a] * t;
+#pragma unroll
+                for (int k = 0; k < D; ++k) t += lam[m][i * D + k] * z[k];
+                q += z[i] * t;
             }
-            f += c.w * c.nrm * exp(-0.5 * q);
+            f += amp[m] * exp(-0.5 * q);
         }
         acc += (double)cv * f;
     }
-    double out2[2];
-    block_reduce2<double>(acc, 0.0, out2);
-    if (threadIdx.x == 0) partial[blockIdx.x] = out2[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        jb.partial[(long long)h * jb.nb + b] = t;
+        __threadfence();
+        lastone = atomicAdd(jb.done + h, 1u) == (unsigned)jb.nb - 1u;
+    }
+    __syncthreads();
+    if (!lastone || threadIdx.x >= 32) return;
+    __threadfence();
+    double t = 0.0;   // lane l takes the partials l, l + 32, .., then a fixed tree
+    for (int k = threadIdx.x; k < jb.nb; k += 32) t += __ldcg(jb.partial + (long long)h * jb.nb + k);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) jb.out[h] = t;
 }
 
-cudaError_t launch_mix_dot(const float* counts, const KdeDesc& g, const MixComp* comps, int ncomp, double* partial,
-                           int nblocks, cudaStream_t st) {
-    k_mix_dot<<<nblocks, 256, 0, st>>>(counts, g, comps, ncomp, partial);
+cudaError_t launch_mix_dot(const MixJob& j, int nH, cudaStream_t st) {
+    if (nH <= 0) return cudaSuccess;
+    const long long blocks = (long long)j.nb * nH;
+    if (j.ncomp < 1 || j.ncomp > kMixMax || j.nb < 1 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    switch (j.g.d) {
+        case 1: k_mix_dot<1><<<(unsigned)blocks, 256, 0, st>>>(j); break;
+        case 2: k_mix_dot<2><<<(unsigned)blocks, 256, 0, st>>>(j); break;
+        case 3: k_mix_dot<3><<<(unsigned)blocks, 256, 0, st>>>(j); break;
+        case 4: k_mix_dot<4><<<(unsigned)blocks, 256, 0, st>>>(j); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 
