@@ -294,12 +294,17 @@ __device__ __forceinline__ void lag_tiles(const LagJob<real>& jb) {
     }
 }
 
+template <typename real, int D, int R, int NV>
+__global__ void __launch_bounds__(256) k_lag(const __grid_constant__ LagJob<real> jb) {
+    lag_tiles<real, D, R, NV>(jb);
+}
+
 // FP32 groups with d <= 2 are held to 64 registers, four CTAs an SM (512 data
 // sets x 16 bandwidths 122 us, against 148 with the compiler's 75); with d = 3
 // the same cap (or three CTAs) is slower than the compiler's 126 (psi_4 91 and
 // 82 us against 78, SCV gradients 18 and 15 against 12).
 template <typename real, int D, int R, int NV>
-__global__ void __launch_bounds__(256, (sizeof(real) == 4 && D <= 2 && NV >= 0) ? 4 : 1) k_lag(const __grid_constant__ LagJob<real> jb) {
+__global__ void __launch_bounds__(256, 4) k_lag_occ4(const __grid_constant__ LagJob<real> jb) {
     lag_tiles<real, D, R, NV>(jb);
 }
 
@@ -318,7 +323,10 @@ static int lag_rmax(int d, bool dbl) {
 
 template <typename real, int D, int R, int NV>
 static cudaError_t lag_go(const LagJob<real>& j, cudaStream_t st) {
-    k_lag<real, D, R, NV><<<j.grid, j.block, 0, st>>>(j);
+    if constexpr (sizeof(real) == 4 && D <= 2 && NV >= 0)
+        k_lag_occ4<real, D, R, NV><<<j.grid, j.block, 0, st>>>(j);
+    else
+        k_lag<real, D, R, NV><<<j.grid, j.block, 0, st>>>(j);
     return cudaGetLastError();
 }
 
