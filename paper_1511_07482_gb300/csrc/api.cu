@@ -374,6 +374,13 @@ static double lambda_max(const Mat& S) {
 // ============================================================ Hermite recurrence tables
 static const int kRmax[5] = {0, 8, 8, 8, 6};
 
+// (2 pi)^{-d/2}
+static double two_pi_pow(int d) {
+    static const double t[5] = {1.0, std::pow(2.0 * M_PI, -0.5), std::pow(2.0 * M_PI, -1.0),
+                                std::pow(2.0 * M_PI, -1.5), std::pow(2.0 * M_PI, -2.0)};
+    return t[d];
+}
+
 struct MultiIndex {
     int a[MAXD];
 };
@@ -1323,7 +1330,7 @@ static double dphi_at0(const Mat& Sigma, const int* alpha) {
     std::vector<int> a(alpha, alpha + d);
     int tot = 0;
     for (int v : a) tot += v;
-    const double phi0 = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
+    const double phi0 = two_pi_pow(d) / std::sqrt(det);
     return ((tot & 1) ? -1.0 : 1.0) * he(a) * phi0;
 }
 
@@ -2245,13 +2252,12 @@ struct LagGroup {
 
 // the lag-domain engine computes exactly the FFT route's value when the
 // padding has no aliasing (P_k >= M_k + L_k on every axis)
-static bool lag_covers(kdefft_ctx c, const GridReq& g) {
+static bool lag_covers(kdefft_ctx c, kdefft_ds ds, const int* L, const int* P) {
     if (!c->lag) return false;
-    const int d = g.ds->d;
-    long long pts = g.L[0] + 1;   // half-box points: the lag kernel indexes them in 32 bits
-    for (int k = 0; k < d; ++k) {
-        if (g.P[k] < g.ds->M[k] + g.L[k]) return false;
-        if (k > 0) pts *= 2 * g.L[k] + 1;
+    long long pts = L[0] + 1;   // half-box points: the lag kernel indexes them in 32 bits
+    for (int k = 0; k < ds->d; ++k) {
+        if (P[k] < ds->M[k] + L[k]) return false;
+        if (k > 0) pts *= 2 * L[k] + 1;
     }
     return pts <= (1LL << 32);
 }
@@ -2298,6 +2304,39 @@ static void invariant_div(uint32_t v, unsigned int& m, int& sh) {
     while ((1ULL << l) < v) ++l;
     m = (unsigned int)(((((1ULL << l) - v) << 32) / v) + 1);
     sh = std::min(l, 1) | (std::max(l - 1, 0) << 8);
+}
+
+// A lag item's dataset, support and scale (its autocorrelation box is final) ...
+template <typename real>
+static void lag_item_frame(LagItem<real>& it, kdefft_ds ds, const int* L, int nsig, int R) {
+    std::memset(&it, 0, sizeof(it));
+    const int d = ds->d;
+    it.d = d;
+    it.nsig = nsig;
+    it.R = R;
+    for (int k = 0; k < d; ++k) {
+        it.L[k] = L[k];
+        it.A[k] = ds->acA[k];
+        it.delta[k] = (real)ds->delta[k];
+        invariant_div((uint32_t)(k == 0 ? L[0] + 1 : 2 * L[k] + 1), it.qm[k], it.qs[k]);
+    }
+    it.acorr = sizeof(real) == 8 ? (const real*)ds->ac64.p : (const real*)ds->ac32.p;
+    const double nn = (double)ds->n;
+    it.scale = 1.0 / (nn * nn);
+}
+// ... and its covariances; false where one is not positive definite
+template <typename real>
+static bool lag_item_sigmas(LagItem<real>& it, const Mat* sig, int nsig) {
+    const int d = it.d;
+    for (int s = 0; s < nsig; ++s) {
+        Mat inv;
+        double det;
+        if (!spd_inv_det(sig[s], inv, det)) return false;
+        for (int a = 0; a < d; ++a)
+            for (int b = 0; b < d; ++b) it.lam[s][a * MAXD + b] = (real)inv(a, b);
+        it.nrm[s] = (real)(two_pi_pow(d) / std::sqrt(det));
+    }
+    return true;
 }
 
 // The lag-domain work of one precision in a run, built on the host: the
@@ -2421,34 +2460,17 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
             const KSpec& sp = rs.specs[g.spec];
             kdefft_ds ds = g.ds;
             LagItem<real>& it = items[q];
-            std::memset(&it, 0, sizeof(it));
-            it.d = d;
-            it.nsig = sp.nsig;
-            it.R = gr.R;
-            for (int k = 0; k < d; ++k) {
-                it.L[k] = g.L[k];
-                it.A[k] = ds->acA[k];
-                it.delta[k] = (real)ds->delta[k];
-                invariant_div((uint32_t)(k == 0 ? g.L[0] + 1 : 2 * g.L[k] + 1), it.qm[k], it.qs[k]);
-            }
+            lag_item_frame(it, ds, g.L, sp.nsig, gr.R);
             if (g.spec == last) {
                 std::memcpy(it.lam, items[q - 1].lam, sizeof(it.lam));
                 std::memcpy(it.nrm, items[q - 1].nrm, sizeof(it.nrm));
             } else {
-                for (int s = 0; s < sp.nsig; ++s) {
-                    Mat inv;
-                    double det;
-                    if (!spd_inv_det(sp.sig[s], inv, det)) {
-                        err = KDEFFT_ERR_NOT_SPD;
-                        return;
-                    }
-                    for (int a = 0; a < d; ++a)
-                        for (int b = 0; b < d; ++b) it.lam[s][a * MAXD + b] = (real)inv(a, b);
-                    it.nrm[s] = (real)(std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det));
+                if (!lag_item_sigmas(it, sp.sig, sp.nsig)) {
+                    err = KDEFFT_ERR_NOT_SPD;
+                    return;
                 }
                 last = g.spec;
             }
-            it.acorr = dbl ? (const real*)ds->ac64.p : (const real*)ds->ac32.p;
             it.w_off = (int)woff[q];
             int N = 1;
             for (int i = 1; i <= d; ++i) N = N * (gr.R + i) / i;
@@ -2468,8 +2490,6 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
                     }
                     wpool[it.w_off + (h * sp.nsig + t.sig) * N + hidx] += (real)(((o & 1) ? -1.0 : 1.0) * t.w);
                 }
-            const double nn = (double)ds->n;
-            it.scale = 1.0 / (nn * nn);
             it.tile0 = (int)tile0[q];
             it.ntile = (int)(tile0[q + 1] - tile0[q]);
             it.part0 = part0[q];
@@ -2486,6 +2506,22 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
     bt.nitems = (int)items.size();
     out.push_back(std::move(bt));
     return KDEFFT_OK;
+}
+
+// The grid of a lag launch over tiles [t0, t0 + n).  FP64, fewer tiles than SMs: a
+// warp slice per CTA, so that the points spread over kLagSlices times as many
+// SMs (with more tiles the extra CTAs cost more than they balance: 36 -> 40 us
+// for 16 SCV bandwidths on 256^2, 31 -> 46 us in 3-D).
+template <typename real>
+static LagJob<real> lag_job(kdefft_ctx c, int t0, int n) {
+    const bool sl = sizeof(real) == 8 && n < c->nsm;
+    LagJob<real> j;
+    std::memset(&j, 0, sizeof(j));
+    j.t0 = t0;
+    j.ntiles = n;
+    j.grid = sl ? n * kLagSlices : std::min(n, c->nsm * 8);
+    j.block = sl ? 32 : 256;
+    return j;
 }
 
 // Upload the lag batches of a run in one copy (their items, tiles, weights and
@@ -2582,15 +2618,13 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
                 cudaEvent_t ev = prof_start(c);
                 auto go = [&](auto zero) -> cudaError_t {
                     using real = decltype(zero);
-                    // FP64, fewer tiles than SMs: a warp slice per CTA, so that
-                    // the points spread over kLagSlices times as many SMs (with
-                    // more tiles the extra CTAs cost more than they balance: 36 ->
-                    // 40 us for 16 SCV bandwidths on 256^2, 31 -> 46 us in 3-D)
-                    const bool sl = sizeof(real) == 8 && cl[3] < c->nsm;
-                    const LagJob<real> j{(const LagItem<real>*)(dbase + lay[b].oI), (const LagTile*)(dbase + lay[b].oT),
-                                         cl[2], cl[3], sl ? cl[3] * kLagSlices : std::min(cl[3], c->nsm * 8),
-                                         sl ? 32 : 256, (const real*)(dbase + lay[b].oW), part + lay[b].slot0,
-                                         (unsigned int*)(dbase + lay[b].oD), hout + lay[b].out0};
+                    LagJob<real> j = lag_job<real>(c, cl[2], cl[3]);
+                    j.items = (const LagItem<real>*)(dbase + lay[b].oI);
+                    j.tiles = (const LagTile*)(dbase + lay[b].oT);
+                    j.wpool = (const real*)(dbase + lay[b].oW);
+                    j.partial = part + lay[b].slot0;
+                    j.done = (unsigned int*)(dbase + lay[b].oD);
+                    j.out = hout + lay[b].out0;
                     return launch_lag<real>(bt.d, cl[0], cl[1], j, ls);
                 };
                 KCU(bt.dbl ? go(0.0) : go(0.f));
@@ -2612,6 +2646,154 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
     c->hout_used += need;
     bts.clear();
     prof_flush(c);
+    return KDEFFT_OK;
+}
+
+// ---- bandwidths straight to lag items --------------------------------------
+// The kernels of a call that evaluates one form at many bandwidths (LSCV with or
+// without gradients, psi_r): nv Gaussians and all partials of order R over nsig
+// covariances, weights w[kernel][nsig], the same for every bandwidth.
+struct DirectForm {
+    int R, nv, nsig;
+    std::vector<double> w;
+    int kernels() const { return (int)w.size() / nsig; }
+};
+
+// Evaluate a form at the bandwidths Hs (dataset owner[many ? h : 0] of Hs[h];
+// cov(H, sig) gives its covariances, basis(H, sig) the matrix of its support):
+// *res points to the kernels' values, bandwidth by bandwidth, until the next
+// call.  The supports come first, so that the autocorrelation passes run while
+// the host writes the items, and these are written where the upload reads
+// them.  KDEFFT_ERR_UNSUPPORTED: a bandwidth that the lag engine does not cover
+// or that is in error; the general path then takes the call (and reports).
+// Against grid requests (230 bytes a kernel, written, paged in and read again):
+// 512 data sets x 16 LSCV bandwidths with their binning 4.9 ms (6.6), psi_4 of
+// 256 bandwidths on 128^3 with its binning 0.46 ms (0.60), 256 LSCV bandwidths
+// 95 us (165).
+template <typename real, typename Cov, typename Basis>
+static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool many, const std::vector<Mat>& Hs,
+                      const DirectForm& f, Cov&& cov, Basis&& basis, const double** res) {
+    const bool dbl = sizeof(real) == 8;
+    const size_t n = Hs.size();
+    const int d = owner[0]->d;
+    if (!c->lag || !lag_single_form(d, f.R, f.nv, f.nsig)) return KDEFFT_ERR_UNSUPPORTED;
+    HostTimer hbuild(c, "host:direct");
+    auto ds_of = [&](size_t h) { return owner[many ? h : 0]; };
+    const long long T = dbl ? 32 * kLagSlices : kLagTile;
+    const int per = dbl ? kLagSlices : 1, nk = f.kernels();
+    std::vector<std::array<int, 4>> L(n);
+    std::vector<int> tile0(n + 1);
+    std::atomic<bool> ok{true};
+    host_parallel_for(n, 2048, [&](size_t h0, size_t h1) {
+        for (size_t h = h0; h < h1 && ok; ++h) {
+            kdefft_ds ds = ds_of(h);
+            Mat chol;
+            int P[4];
+            if (!cholesky(Hs[h], chol) || plan_for(ds, basis(Hs[h]), L[h].data(), P) != KDEFFT_OK ||
+                !lag_covers(c, ds, L[h].data(), P)) {
+                ok = false;
+                return;
+            }
+            long long pts = L[h][0] + 1;
+            for (int k = 1; k < d; ++k) pts *= 2 * L[h][k] + 1;
+            tile0[h + 1] = (int)((pts + T - 1) / T);
+        }
+    });
+    if (!ok) return KDEFFT_ERR_UNSUPPORTED;
+    long long nt = 0;
+    {
+        std::map<kdefft_ds, std::array<int, 4>> need;
+        auto at = need.end();
+        for (size_t h = 0; h < n; ++h) {
+            kdefft_ds ds = ds_of(h);
+            if (at == need.end() || at->first != ds) at = need.emplace(ds, std::array<int, 4>{0, 0, 0, 0}).first;
+            for (int k = 0; k < d; ++k) at->second[k] = std::max(at->second[k], L[h][k]);
+            nt += tile0[h + 1];
+            tile0[h + 1] = (int)std::min<long long>(nt, 0x7fffffffLL);
+        }
+        tile0[0] = 0;
+        if (nt > 0x7fffffffLL || n * (size_t)nk > 0x7fffffffULL) return KDEFFT_ERR_UNSUPPORTED;
+        const int ar =
+            ensure_autocorr_many(c, std::vector<std::pair<kdefft_ds, std::array<int, 4>>>(need.begin(), need.end()));
+        if (ar != KDEFFT_OK) return ar;
+    }
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t oT = al(sizeof(LagItem<real>) * n), oW = oT + al(sizeof(LagTile) * (size_t)nt),
+                 oD = oW + al(sizeof(real) * f.w.size()), bytes = oD + al(sizeof(unsigned int) * n);
+    KCHK(staging_wait(c));
+    KCHK(c->h_items.ensure(bytes));
+    KCHK(c->items.ensure(bytes));
+    KCHK(c->partial.ensure(sizeof(double) * (size_t)nt * per * nk));
+    KCHK(flush_reads(c));
+    KCHK(c->h_out.ensure(sizeof(double) * n * nk));
+    unsigned char* h8 = (unsigned char*)c->h_items.p;
+    unsigned char* d8 = (unsigned char*)c->items.p;
+    LagItem<real>* items = (LagItem<real>*)h8;
+    LagTile* tiles = (LagTile*)(h8 + oT);
+    real* w = (real*)(h8 + oW);
+    int sigs = 0;
+    for (size_t i = 0; i < f.w.size(); ++i) {
+        w[i] = (real)f.w[i];
+        if (f.w[i] != 0.0) sigs |= 1 << (int)(i % f.nsig);
+    }
+    std::memset(h8 + oD, 0, sizeof(unsigned int) * n);
+    host_parallel_for(n, 1024, [&](size_t h0, size_t h1) {
+        for (size_t h = h0; h < h1; ++h) {
+            kdefft_ds ds = ds_of(h);
+            LagItem<real>& it = items[h];
+            lag_item_frame(it, ds, L[h].data(), f.nsig, f.R);
+            Mat sig[MAXSIG];
+            cov(Hs[h], sig);
+            if (!lag_item_sigmas(it, sig, f.nsig)) {
+                ok = false;
+                return;
+            }
+            it.sigs = sigs;
+            it.tile0 = tile0[h];
+            it.ntile = tile0[h + 1] - tile0[h];
+            it.part0 = (long long)tile0[h] * per * nk;
+            it.nout = nk;
+            it.out0 = (int)(h * nk);
+            long long pts = L[h][0] + 1;
+            for (int k = 1; k < d; ++k) pts *= 2 * L[h][k] + 1;
+            long long at = 0;
+            for (int t = tile0[h]; t < tile0[h + 1]; ++t, at += T)
+                tiles[t] = LagTile{(int)h, (int)std::min(T, pts - at), at};
+        }
+    });
+    if (!ok) return KDEFFT_ERR_UNSUPPORTED;
+    int N = 1;   // Hermite values
+    for (int i = 1; i <= d; ++i) N = N * (f.R + i) / i;
+    const double fl = (double)nt * (double)T * (f.nsig * (2.0 * d * d + 3.0 * N) + 12.0 * nk);   // (whole tiles)
+    const double by = (double)nt * (double)T * sizeof(real);
+    double* hout = (double*)c->h_out.p;
+    const std::vector<long long> sig = {10, dbl ? 8 : 4, d, f.R, f.nv, (long long)n, nt, (long long)bytes, (long long)oT,
+                                        (long long)oW, (long long)oD, (long long)(uintptr_t)h8, (long long)(uintptr_t)d8,
+                                        (long long)(uintptr_t)c->partial.p, (long long)(uintptr_t)hout};
+    auto issue = [&]() -> int {
+        KCU(cudaMemcpyAsync(d8, h8, bytes, cudaMemcpyHostToDevice, c->stream));
+        cudaEvent_t ev = prof_start(c);
+        LagJob<real> j = lag_job<real>(c, 0, (int)nt);
+        j.items = (const LagItem<real>*)d8;
+        j.tiles = (const LagTile*)(d8 + oT);
+        j.wpool = (const real*)(d8 + oW);
+        j.partial = (double*)c->partial.p;
+        j.done = (unsigned int*)(d8 + oD);
+        j.out = hout;
+        KCU(launch_lag<real>(d, f.R, f.nv, j, c->stream));
+        prof_stop(c, ev, dbl ? "lag_f64" : "lag_f32", by, fl);
+        return KDEFFT_OK;
+    };
+    const int r = run_graph(c, sig, issue);
+    c->h2d += (int64_t)bytes;
+    c->d2h += (int64_t)(sizeof(double) * n * nk);
+    {
+        HostTimer wt(c, "host:wait");
+        KCU(cudaStreamSynchronize(c->stream));   // the results, and the staging buffer free again
+    }
+    KCHK(r);
+    prof_flush(c);
+    *res = hout;
     return KDEFFT_OK;
 }
 
@@ -2726,7 +2908,7 @@ static int run_requests(kdefft_ctx c, ReqSet& rs, const std::vector<int>& sel, s
                 break;
             ++v;
         }
-        if (lag_covers(c, a))
+        if (lag_covers(c, a.ds, a.L, a.P))
             lag_groups(rs, sel, (int)u, (int)v, sizeof(real) == 8, groups, pairs);
         else
             for (size_t i = u; i < v; i += 2) pairs.push_back({sel[i], i + 1 < v ? sel[i + 1] : -1});
@@ -2789,7 +2971,7 @@ static int run_requests(kdefft_ctx c, ReqSet& rs, const std::vector<int>& sel, s
                         return fail(KDEFFT_ERR_NOT_SPD, "a kernel covariance is not positive definite");
                     for (int a = 0; a < d; ++a)
                         for (int b = 0; b < d; ++b) it.lam[s][a * MAXD + b] = inv(a, b);
-                    it.nrm[s] = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
+                    it.nrm[s] = two_pi_pow(d) / std::sqrt(det);
                 }
                 int R = 0;
                 const int gi[2] = {pr.first, pr.second};
@@ -2859,21 +3041,22 @@ static int run(kdefft_ctx c, ReqSet& rs) {
 }
 
 // ============================================================ objective assembly
-static void assemble_lscv(kdefft_ds ds, const Mat& H, const GridReq* g, double* val, double* grad) {
+// LSCV from the values v of its kernels (lscv_grid_count of them)
+static void assemble_lscv(kdefft_ds ds, const Mat& H, const double* v, double* val, double* grad) {
     const int d = ds->d;
     const double n = (double)ds->n;
     Mat inv;
     double det;
     spd_inv_det(H, inv, det);
-    const double k0 = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
+    const double k0 = two_pi_pow(d) / std::sqrt(det);
     int gi = 0;
     double c0;
     if (!ds->opts.exact_loo) {
-        *val = g[0].value + 2.0 * k0 / n;
+        *val = v[0] + 2.0 * k0 / n;
         gi = 1;
         c0 = 2.0 / n;
     } else {
-        *val = g[0].value - 2.0 * n / (n - 1.0) * g[1].value + 2.0 / (n - 1.0) * k0;
+        *val = v[0] - 2.0 * n / (n - 1.0) * v[1] + 2.0 / (n - 1.0) * k0;
         gi = 2;
         c0 = 2.0 / (n - 1.0);
     }
@@ -2881,8 +3064,8 @@ static void assemble_lscv(kdefft_ds ds, const Mat& H, const GridReq* g, double* 
         for (int a = 0; a < d; ++a)
             for (int b = a; b < d; ++b) {
                 const double tie = (a == b) ? 1.0 : 2.0;
-                const double v = g[gi++].value + c0 * tie * (-0.5 * k0 * inv(a, b));
-                grad[a * d + b] = grad[b * d + a] = v;
+                const double e = v[gi++] + c0 * tie * (-0.5 * k0 * inv(a, b));
+                grad[a * d + b] = grad[b * d + a] = e;
             }
     }
 }
@@ -3671,19 +3854,34 @@ int kdefft_psi(kdefft_ds ds, const double* H, int nH, int r, double* out) {
     ReqSet rs;
     std::vector<int> first(nH);
     const std::vector<MultiIndex> alphas = order_alphas(d, r);
+    const std::vector<int> map = kron_map(d, r, alphas);
+    const size_t len = map.size();
+    std::vector<Mat> Hs((size_t)nH);
+    for (int h = 0; h < nH; ++h) {
+        KCHK(sym_check(H + (size_t)h * d * d, d, Hs[h], "H"));
+        KCHK(spd_or_fail(Hs[h], "H"));
+    }
+    std::vector<double> res(len * nH);
+    {   // straight to lag items: one covariance, every partial of the order
+        const DirectForm f{r, r == 0 ? 1 : 0, 1, std::vector<double>(alphas.size(), 1.0)};
+        const double* v = nullptr;
+        auto cov = [](const Mat& Hm, Mat* sig) { sig[0] = Hm; };
+        auto basis = [](const Mat& Hm) { return Hm; };
+        const int dr = ds->opts.precision == KDEFFT_FP64
+                           ? direct_lag<double>(ds->ctx, {ds}, false, Hs, f, cov, basis, &v)
+                           : direct_lag<float>(ds->ctx, {ds}, false, Hs, f, cov, basis, &v);
+        if (dr == KDEFFT_OK) {
+            for (int h = 0; h < nH; ++h)
+                for (size_t p = 0; p < len; ++p) res[(size_t)h * len + p] = v[(size_t)h * alphas.size() + map[p]];
+            return write_out(ds->ctx, out, res.data(), res.size());
+        }
+        if (dr != KDEFFT_ERR_UNSUPPORTED) return dr;
+    }
     {
         HostTimer hq(ds->ctx, "host:psi_requests");
-        std::vector<Mat> Hs((size_t)nH);
-        for (int h = 0; h < nH; ++h) {
-            KCHK(sym_check(H + (size_t)h * d * d, d, Hs[h], "H"));
-            KCHK(spd_or_fail(Hs[h], "H"));
-        }
         KCHK(add_psi_many(rs, ds, Hs, alphas, first));
     }
     KCHK(run(ds->ctx, rs));
-    const std::vector<int> map = kron_map(d, r, alphas);
-    const size_t len = map.size();
-    std::vector<double> res(len * nH);
     for (int h = 0; h < nH; ++h) kron_expand(map, &rs.grids[first[h]], res.data() + (size_t)h * len);
     return write_out(ds->ctx, out, res.data(), res.size());
 }
@@ -3736,6 +3934,13 @@ static int lscv_requests(ReqSet& rs, kdefft_ds ds, const double* H, int nH, bool
     return add_lscv_many(rs, std::vector<kdefft_ds>((size_t)nH, ds), j.Hs, grad, j.first);
 }
 
+// LSCV from the grids of a request set, the first of them g
+static void assemble_lscv(kdefft_ds ds, const Mat& H, const GridReq* g, double* val, double* grad) {
+    double v[16];
+    for (int i = 0; i < lscv_grid_count(ds, grad != nullptr); ++i) v[i] = g[i].value;
+    assemble_lscv(ds, H, v, val, grad);
+}
+
 static void lscv_assemble(const ReqSet& rs, kdefft_ds ds, const LscvJob& j, std::vector<double>& val,
                           std::vector<double>* grad) {
     const int d = ds->d, nH = (int)j.first.size();
@@ -3745,7 +3950,66 @@ static void lscv_assemble(const ReqSet& rs, kdefft_ds ds, const LscvJob& j, std:
         assemble_lscv(ds, j.Hs[h], &rs.grids[j.first[h]], &val[h], grad ? grad->data() + (size_t)h * d * d : nullptr);
 }
 
+// LSCV of many bandwidths straight to lag items (direct_lag), written to val
+// and grad (may be null); KDEFFT_ERR_UNSUPPORTED leaves the call to the general
+// path.  Datasets of one call share options' weights: leave-one-out weights
+// carry n, so only calls on one dataset take them here.
+static int direct_lscv(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool many, const std::vector<Mat>& Hs,
+                       double* val, double* grad) {
+    kdefft_ds ds0 = owner[0];
+    const int d = ds0->d;
+    const bool loo = ds0->opts.exact_loo != 0;
+    if (many)
+        for (kdefft_ds ds : owner)
+            if (ds->opts.exact_loo) return KDEFFT_ERR_UNSUPPORTED;
+    const double n = (double)ds0->n, fac = loo ? n / (n - 1.0) : 1.0;
+    DirectForm f{grad ? 2 : 0, loo ? 2 : 1, 2, {}};
+    if (loo)
+        f.w = {1.0, 0.0, 0.0, 1.0};
+    else
+        f.w = {1.0, -2.0};
+    if (grad)
+        for (int a = 0; a < d; ++a)
+            for (int b = a; b < d; ++b) {
+                const double s = (a == b) ? 1.0 : 2.0;
+                f.w.push_back(s);
+                f.w.push_back(-s * fac);
+            }
+    auto cov = [](const Mat& H, Mat* sig) {
+        sig[0] = scaled(2.0, H);
+        sig[1] = H;
+    };
+    auto run_as = [&](auto zero, const double** res) {
+        using real = decltype(zero);
+        // the support's matrix (a batch's datasets may differ in L_basis: the general path)
+        const int basis0 = ds0->opts.L_basis;
+        if (many)
+            for (kdefft_ds ds : owner)
+                if (ds->opts.L_basis != basis0) return (int)KDEFFT_ERR_UNSUPPORTED;
+        return direct_lag<real>(c, owner, many, Hs, f, cov,
+                                [&](const Mat& H) { return basis0 == KDEFFT_L_WIDEST ? scaled(2.0, H) : H; }, res);
+    };
+    const double* res = nullptr;
+    const int r = ds0->opts.precision == KDEFFT_FP64 ? run_as(0.0, &res) : run_as(0.f, &res);
+    if (r != KDEFFT_OK) return r;
+    const int nk = f.kernels();
+    host_parallel_for(Hs.size(), 2048, [&](size_t h0, size_t h1) {
+        for (size_t h = h0; h < h1; ++h)
+            assemble_lscv(owner[many ? h : 0], Hs[h], res + h * nk, val + h, grad ? grad + h * d * d : nullptr);
+    });
+    return KDEFFT_OK;
+}
+
 static int eval_lscv(kdefft_ds ds, const double* H, int nH, std::vector<double>& val, std::vector<double>* grad) {
+    const int d = ds->d;
+    {
+        std::vector<Mat> Hs(nH);
+        for (int h = 0; h < nH; ++h) KCHK(sym_check(H + (size_t)h * d * d, d, Hs[h], "H"));
+        val.resize(nH);
+        if (grad) grad->resize((size_t)nH * d * d);
+        const int r = direct_lscv(ds->ctx, {ds}, false, Hs, val.data(), grad ? grad->data() : nullptr);
+        if (r != KDEFFT_ERR_UNSUPPORTED) return r;
+    }
     ReqSet rs;
     LscvJob j;
     KCHK(lscv_requests(rs, ds, H, nH, grad != nullptr, j));
@@ -4011,7 +4275,7 @@ int kdefft_kde_grid(kdefft_ds ds, const double* H, double* out) {
     spd_inv_det(Hm, inv, det);
     KdeKernel kn;
     std::memset(&kn, 0, sizeof(kn));
-    kn.nrm = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
+    kn.nrm = two_pi_pow(d) / std::sqrt(det);
     for (int a = 0; a < d; ++a)
         for (int b = 0; b < d; ++b) kn.lam[a * MAXD + b] = inv(a, b);
     // the kernel writes a device output itself (FP64-aligned memory of this
@@ -4060,7 +4324,7 @@ int kdefft_ise_mixture(kdefft_ds ds, const double* H, int nH, int K, const doubl
         double q = 0.0;
         for (int a = 0; a < d; ++a)
             for (int b = 0; b < d; ++b) q += x[a] * inv(a, b) * x[b];
-        return std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det) * std::exp(-0.5 * q);
+        return two_pi_pow(d) / std::sqrt(det) * std::exp(-0.5 * q);
     };
     // int f^2 = sum_lm w_l w_m phi_{S_l + S_m}(mu_l - mu_m), closed form
     double ff = 0.0;
@@ -4112,7 +4376,7 @@ int kdefft_ise_mixture(kdefft_ds ds, const double* H, int nH, int K, const doubl
                 for (int k = 0; k < d; ++k) mc.mu[k] = mu[(size_t)m * d + k];
                 for (int a = 0; a < d; ++a)
                     for (int b = 0; b < d; ++b) mc.lam[a * MAXD + b] = inv(a, b);
-                mc.nrm = std::pow(2.0 * M_PI, -0.5 * d) / std::sqrt(det);
+                mc.nrm = two_pi_pow(d) / std::sqrt(det);
                 mc.w = w[m];
             }
         KCU(cudaMemcpyAsync(db, hb, up, cudaMemcpyHostToDevice, c->stream));
@@ -4187,10 +4451,18 @@ int kdefft_batch_lscv(kdefft_ctx c, int nds, const kdefft_ds* dss, const int* nH
         }
         off += nH_per_ds[i];
     }
+    const size_t nt = Hs.size();
+    if (nt == 0) return KDEFFT_OK;
+    std::vector<double> v(nt), g(grad ? nt * d * d : 0);
+    const int dr = direct_lscv(c, owner, true, Hs, v.data(), grad ? g.data() : nullptr);
+    if (dr == KDEFFT_OK) {
+        std::memcpy(val, v.data(), sizeof(double) * nt);
+        if (grad) std::memcpy(grad, g.data(), sizeof(double) * g.size());
+        return KDEFFT_OK;
+    }
+    if (dr != KDEFFT_ERR_UNSUPPORTED) return dr;
     KCHK(add_lscv_many(rs, owner, Hs, grad != nullptr, first));
     KCHK(run(c, rs));
-    const size_t nt = Hs.size();
-    std::vector<double> v(nt), g(grad ? nt * d * d : 0);
     host_parallel_for(nt, 2048, [&](size_t h0, size_t h1) {
         for (size_t h = h0; h < h1; ++h)
             assemble_lscv(owner[h], Hs[h], &rs.grids[first[h]], &v[h], grad ? g.data() + h * d * d : nullptr);
