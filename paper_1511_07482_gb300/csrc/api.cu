@@ -865,8 +865,9 @@ static int sync_twiddles(kdefft_ctx c) {
     for (size_t i = 0; i < 2 * n; ++i) {
         const double v = c->tw_host[i];
         f[i] = (float)v;
-        fp[2 * i] = (float)v;                          // FP32 pair: leading part
-        fp[2 * i + 1] = (float)(v - (double)(float)v);  // and its remainder
+        float* pair = &fp[4 * (i / 2) + i % 2];   // FP32 pairs: leading parts of x, y, then the remainders
+        pair[0] = (float)v;
+        pair[2] = (float)(v - (double)(float)v);
     }
     KCU(cudaMemcpy(c->tw64.p, c->tw_host.data(), n * sizeof(double2), cudaMemcpyHostToDevice));
     KCU(cudaMemcpy(c->tw32.p, f.data(), n * sizeof(float2), cudaMemcpyHostToDevice));

@@ -81,10 +81,100 @@ __device__ __forceinline__ dflt operator*(dflt a, dflt b) {
 }
 __device__ __forceinline__ double to_double(dflt a) { return (double)a.h + (double)a.l; }
 __device__ __forceinline__ double to_double(double a) { return a; }
-// complex FP32 pair: the layout and size of double2
-struct dcplx {
-    dflt x, y;
+// Two FP32 values in a 64-bit register pair and the packed operations on
+// them (both halves rounded as the scalar operations round): the FP32 pipes
+// take a packed instruction in two cycles, so arithmetic that fills them
+// leaves every other issue slot to loads and control.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+// a - b: one rounding, as the subtraction's
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack2(-1.f, -1.f), a); }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f32x2 swap2(f32x2 a) {
+    const float2 v = unpack2(a);
+    return pack2(v.y, v.x);
+}
+
+// Complex FP32 pair, of double2's size: h holds the leading parts of (x, y), l
+// the remainders, so that both components take each operation together (the
+// sequences are dflt's, so are the bits).
+struct __align__(16) dcplx {
+    f32x2 h, l;
 };
+__device__ __forceinline__ dcplx cadd(dcplx a, dcplx b) {
+    const f32x2 s = add2(a.h, b.h);
+    const f32x2 bb = sub2(s, a.h);
+    const f32x2 e = add2(add2(sub2(a.h, sub2(s, bb)), sub2(b.h, bb)), add2(a.l, b.l));
+    const f32x2 h = add2(s, e);
+    return dcplx{h, sub2(e, sub2(h, s))};
+}
+__device__ __forceinline__ dcplx csub(dcplx a, dcplx b) {
+    const f32x2 s = sub2(a.h, b.h);
+    const f32x2 bb = sub2(s, a.h);
+    const f32x2 e = add2(sub2(sub2(a.h, sub2(s, bb)), add2(b.h, bb)), sub2(a.l, b.l));
+    const f32x2 h = add2(s, e);
+    return dcplx{h, sub2(e, sub2(h, s))};
+}
+// component-wise product (a.x b.x, a.y b.y)
+__device__ __forceinline__ dcplx pmul(dcplx a, dcplx b) {
+    const f32x2 p = mul2(a.h, b.h);
+    const f32x2 e = fma2(a.h, b.l, fma2(a.l, b.h, fma2(a.h, b.h, neg2(p))));
+    const f32x2 h = add2(p, e);
+    return dcplx{h, sub2(e, sub2(h, p))};
+}
+__device__ __forceinline__ dcplx cmul(dcplx a, dcplx b) {   // a (x of b) + i a (y of b)
+    const float2 bh = unpack2(b.h), bl = unpack2(b.l);
+    return cadd(pmul(a, dcplx{pack2(bh.x, bh.x), pack2(bl.x, bl.x)}),
+                pmul(dcplx{swap2(a.h), swap2(a.l)}, dcplx{pack2(-bh.y, bh.y), pack2(-bl.y, bl.y)}));
+}
+__device__ __forceinline__ dcplx cconj(dcplx a) {
+    return dcplx{a.h ^ 0x8000000000000000ull, a.l ^ 0x8000000000000000ull};
+}
+__device__ __forceinline__ dcplx cmi(dcplx a) { return cconj(dcplx{swap2(a.h), swap2(a.l)}); }   // -i a
+__device__ __forceinline__ dcplx cscale(dflt s, dcplx a) {
+    return pmul(dcplx{pack2(s.h, s.h), pack2(s.l, s.l)}, a);
+}
+__device__ __forceinline__ dcplx chalf(dcplx a) {
+    return dcplx{mul2(a.h, pack2(0.5f, 0.5f)), mul2(a.l, pack2(0.5f, 0.5f))};
+}
+__device__ __forceinline__ dflt re(dcplx a) { return dflt(unpack2(a.h).x, unpack2(a.l).x); }
+__device__ __forceinline__ dflt im(dcplx a) { return dflt(unpack2(a.h).y, unpack2(a.l).y); }
+__device__ __forceinline__ dcplx cmake(dflt x, dflt y) { return dcplx{pack2(x.h, y.h), pack2(x.l, y.l)}; }
+__device__ __forceinline__ dflt cnorm2(dcplx a) {
+    const dcplx q = pmul(a, a);
+    return re(q) + im(q);
+}
+__device__ __forceinline__ bool czero(dcplx a) { return (a.h & 0x7fffffff7fffffffull) == 0; }   // (l is zero where h is)
+// the same names for double2
+__device__ __forceinline__ double2 cconj(double2 a) { return double2{a.x, -a.y}; }
+__device__ __forceinline__ double2 chalf(double2 a) { return double2{0.5 * a.x, 0.5 * a.y}; }
+__device__ __forceinline__ double re(double2 a) { return a.x; }
+__device__ __forceinline__ double im(double2 a) { return a.y; }
+__device__ __forceinline__ double2 cmake(double x, double y) { return double2{x, y}; }
 
 // The job whose block range holds block b, from the jobs' first blocks
 // (ascending, first(0) = 0): every warp searches for itself, 32 places at a

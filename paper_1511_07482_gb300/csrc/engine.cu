@@ -117,6 +117,38 @@ struct Dft<C, 5> {
     }
 };
 
+// complex FP32 pairs: the same transforms on packed components
+template <>
+struct Dft<dcplx, 3> {
+    __device__ __forceinline__ static void run(dcplx* v) {
+        const dcplx t1 = cadd(v[1], v[2]);
+        const dcplx m = csub(v[0], cscale(dflt(0.5), t1));
+        const dcplx r = cscale(dflt(0.8660254037844386), cmi(csub(v[1], v[2])));   // -i sin(2 pi / 3) (v1 - v2)
+        v[0] = cadd(v[0], t1);
+        v[1] = cadd(m, r);
+        v[2] = csub(m, r);
+    }
+};
+template <>
+struct Dft<dcplx, 5> {
+    __device__ __forceinline__ static void run(dcplx* v) {
+        const dflt c1(0.30901699437494745), c2(-0.8090169943749473);   // cos(2 pi / 5), cos(4 pi / 5)
+        const dflt s1(0.9510565162951535), s2(0.5877852522924732);     // sin(2 pi / 5), sin(4 pi / 5)
+        const dcplx a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]);
+        const dcplx a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
+        const dcplx x0 = v[0];
+        const dcplx p1 = cadd(cadd(x0, cscale(c1, a1)), cscale(c2, a2));
+        const dcplx p2 = cadd(cadd(x0, cscale(c2, a1)), cscale(c1, a2));
+        const dcplx q1 = cmi(cadd(cscale(s1, b1), cscale(s2, b2)));   // X1 = p1 - i q1, X2 = p2 - i q2
+        const dcplx q2 = cmi(csub(cscale(s2, b1), cscale(s1, b2)));
+        v[0] = cadd(cadd(x0, a1), a2);
+        v[1] = cadd(p1, q1);
+        v[4] = csub(p1, q1);
+        v[2] = cadd(p2, q2);
+        v[3] = csub(p2, q2);
+    }
+};
+
 template <typename C>
 struct Dft<C, 8> {
     __device__ __forceinline__ static void run(C* v) {
@@ -199,22 +231,6 @@ struct CxTw {
     }
 };
 
-// the same twiddles as FP32 pairs, split at compile time (no FP64
-// conversion at run time when the table is indexed)
-template <int R>
-struct CxTwPair {
-    float ch[R], cl[R], sh[R], sl[R];
-    constexpr CxTwPair() : ch(), cl(), sh(), sl() {
-        for (int m = 0; m < R; ++m) {
-            const CxCis z = cx_cis(m, R);
-            ch[m] = (float)z.c;
-            cl[m] = (float)(z.c - (double)(float)z.c);
-            sh[m] = (float)z.s;
-            sl[m] = (float)(z.s - (double)(float)z.s);
-        }
-    }
-};
-
 template <typename C, int R>
 struct Dft {
     __device__ __forceinline__ static void run(C* v) {
@@ -222,7 +238,6 @@ struct Dft {
         constexpr int A = cx_small_factor(R);
         constexpr int B = R / A;
         constexpr CxTw<R> tw{};
-        constexpr CxTwPair<R> tp{};
         C u[R];
         // A-point DFTs over b-strided subsequences: u[b * A + k1]
 #pragma unroll
@@ -239,13 +254,8 @@ struct Dft {
                 } else {
                     // t * exp(-2 pi i m / R) = t * (cos - i sin)
                     R_ cw, sw;
-                    if constexpr (sizeof(R_) == 8 && !std::is_same<R_, double>::value) {   // FP32 pairs
-                        cw = R_(tp.ch[m], tp.cl[m]);
-                        sw = R_(tp.sh[m], tp.sl[m]);
-                    } else {
-                        cw = R_(tw.c[m]);
-                        sw = R_(tw.s[m]);
-                    }
+                    cw = R_(tw.c[m]);
+                    sw = R_(tw.s[m]);
                     u[b * A + k1] = C{t[k1].x * cw + t[k1].y * sw, t[k1].y * cw - t[k1].x * sw};
                 }
             }
@@ -667,30 +677,28 @@ __global__ void __launch_bounds__(256) k_final(const Item<real>* __restrict__ it
 // places in memory once per line (a table in shared memory), not per value.
 // Against one complex transform per line in every pass, the spectrum in memory
 // and a 64-bit division per value (events around a data set's passes): 128^3
-// at P = 144 to 160 173 us (285), 48^4 420 us (737), 256^2 42 us (44: a line
-// per block, bound by the chain of stages); 512 data sets of 64^2 to 256^2 659
-// us (3378, most of it one line a block of 256 threads).  Issue slots 50 to 60
-// % busy, FP32 pipes 45 %, barriers and loads the rest.
+// at P = 144 to 160 153 us (285), 48^4 349 us (737), 256^2 41 us (44: a line
+// per block, bound by the chain of stages); 512 data sets of 64^2 to 256^2 593
+// us (3378, most of it one line a block of 256 threads).  Packed operations on
+// the two components take 8 % off the scalar ones.  Issue slots 50 to 60 %
+// busy, FP32 pipes 45 %, barriers and loads the rest.
 struct LineDiv {   // n / D for n < 2^20 (D <= 4096)
     uint32_t m, D;
     __device__ __forceinline__ explicit LineDiv(int d) : m(magic_of((uint32_t)max(d, 2))), D((uint32_t)d) {}
     __device__ __forceinline__ int div(int n) const { return D == 1u ? n : (int)qdiv((uint32_t)n, m); }
 };
-__device__ __forceinline__ dflt half_of(dflt a) { return dflt(0.5f * a.h, 0.5f * a.l); }
-__device__ __forceinline__ double half_of(double a) { return 0.5 * a; }
-__device__ __forceinline__ dflt to_real(float v, dflt) { return dflt(v, 0.f); }
 
 // The transforms of real lines 0 and 1 at frequency w from that of x_0 + i x_1
 // (z at w, m at P - w).
 template <typename C>
 __device__ __forceinline__ C split_pair(int which, C z, C m) {
-    return which == 0 ? C{half_of(z.x + m.x), half_of(z.y - m.y)} : C{half_of(z.y + m.y), half_of(m.x - z.x)};
+    return chalf(which == 0 ? cadd(z, cconj(m)) : cmi(csub(z, cconj(m))));
 }
 
 template <typename C, int KIND>
 __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, int njobs,
                                               const C* __restrict__ twpool) {
-    using R = decltype(C{}.x);
+    using R = decltype(re(C{}));
     constexpr bool packed = KIND == kLineRealRows || KIND == kLineLast || KIND == kLineSpecRows;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long src[kMaxLines], dst[kMaxLines];
@@ -723,7 +731,7 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
     load_twiddles(tw, twpool, jb.ap);
     __syncthreads();
     const LineDiv dP(P), dY(Y), dn(nl), df(nf);
-    const C zero{R(0.0), R(0.0)};
+    const C zero = cmake(R(0.0), R(0.0));
     int any = 0;   // forward passes: does this block's input hold anything?
     if constexpr (KIND == kLineRealRows || KIND == kLineSpecRows) {   // two real rows a line, values fastest
         for (int t = threadIdx.x; t < nf * P; t += blockDim.x) {
@@ -733,12 +741,10 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
                 if constexpr (KIND == kLineRealRows) {
                     const float a = jb.in_f[src[2 * c] + x], b = 2 * c + 1 < nl ? jb.in_f[src[2 * c + 1] + x] : 0.f;
                     any |= a != 0.f || b != 0.f;
-                    v.x = to_real(a, R());
-                    v.y = to_real(b, R());
+                    v = cmake(R(a, 0.f), R(b, 0.f));
                 } else {
                     const R* in = reinterpret_cast<const R*>(jb.in);
-                    v.x = in[src[2 * c] + x];
-                    if (2 * c + 1 < nl) v.y = in[src[2 * c + 1] + x];
+                    v = cmake(in[src[2 * c] + x], 2 * c + 1 < nl ? in[src[2 * c + 1] + x] : R(0.0));
                 }
             }
             bufa[pad(t)] = v;
@@ -752,7 +758,7 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
             C a = zero, b = zero;
             if (w < X) {
                 if (jb.in_real) {   // d = 1: the real spectrum itself
-                    a.x = reinterpret_cast<const R*>(jb.in)[src[2 * c] + w];
+                    a = cmake(reinterpret_cast<const R*>(jb.in)[src[2 * c] + w], R(0.0));
                 } else {
                     const C* in = reinterpret_cast<const C*>(jb.in);
                     a = in[src[2 * c] + w * I];
@@ -760,10 +766,11 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
                 }
             }
             if (w == 0 || 2 * w == P) {   // real, but for rounding
-                bufa[pad(c * P + w)] = C{a.x, -b.x};
-            } else {
-                bufa[pad(c * P + w)] = C{a.x - b.y, -(a.y + b.x)};
-                bufa[pad(c * P + P - w)] = C{a.x + b.y, a.y - b.x};
+                bufa[pad(c * P + w)] = cmake(re(a), -re(b));
+            } else {   // conj(a + i b), and a - i b = conj of Z at P - w
+                const C mb = cmi(b);
+                bufa[pad(c * P + w)] = cconj(csub(a, mb));
+                bufa[pad(c * P + P - w)] = cadd(a, mb);
             }
         }
     } else {   // complex lines, line fastest
@@ -774,13 +781,13 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
                 const long long at = src[c] + x * I;
                 if constexpr (KIND == kLineAxis0) {
                     if (jb.in_f)   // d = 1: the counts themselves
-                        v.x = to_real(jb.in_f[at], R());
+                        v = cmake(R(jb.in_f[at], 0.f), R(0.0));
                     else
                         v = reinterpret_cast<const C*>(jb.in)[at];
                 } else {
                     v = reinterpret_cast<const C*>(jb.in)[at];
-                    if constexpr (KIND == kLineInverse) v.y = -v.y;
-                    if constexpr (KIND == kLineForward) any |= v.x.h != 0.f || v.y.h != 0.f;
+                    if constexpr (KIND == kLineInverse) v = cconj(v);
+                    if constexpr (KIND == kLineForward) any |= !czero(v);
                 }
             }
             bufa[pad(c * P + x)] = v;
@@ -809,13 +816,8 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
         const int nh = (nl + 1) / 2;
         for (int t = threadIdx.x; t < nh * P; t += blockDim.x) {
             const int c = dP.div(t), w = t - c * P;
-            const C a = Z[pad(2 * c * P + w)];
-            C v{a.x * a.x + a.y * a.y, R(0.0)};
-            if (2 * c + 1 < nl) {
-                const C b = Z[pad((2 * c + 1) * P + w)];
-                v.y = b.x * b.x + b.y * b.y;
-            }
-            other[pad(t)] = v;
+            other[pad(t)] = cmake(cnorm2(Z[pad(2 * c * P + w)]),
+                                  2 * c + 1 < nl ? cnorm2(Z[pad((2 * c + 1) * P + w)]) : R(0.0));
         }
         Z = smem_fft(other, Z, nh, jb.ap, tw);
     }
@@ -825,9 +827,9 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
             const int c = dY.div(t), y = t - c * Y;
             const int zb = (c >> 1) * P;
             C v = split_pair(c & 1, Z[pad(zb + y)], Z[pad(zb + (y ? P - y : 0))]);
-            if constexpr (KIND != kLineRealRows) v.y = -v.y;
+            if constexpr (KIND != kLineRealRows) v = cconj(v);
             if (KIND == kLineAxis0 && jb.out_r) {   // d = 1
-                const double r = to_double(v.x) * jb.scale;
+                const double r = to_double(re(v)) * jb.scale;
                 jb.out_r[dst[c] + y] = r;
                 jb.out_r32[dst[c] + y] = (float)r;
             } else {
@@ -844,11 +846,10 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
                 int j = jb.ylo + y;   // a lag, |j| < P
                 if (j < 0) j += P;
                 if constexpr (KIND == kLineInverse) {
-                    const C v = Z[pad(c * P + j)];
-                    out[at] = C{v.x, -v.y};
+                    out[at] = cconj(Z[pad(c * P + j)]);
                 } else {
                     const C v = Z[pad((c >> 1) * P + j)];
-                    const double r = to_double((c & 1) ? -v.y : v.x) * jb.scale;
+                    const double r = ((c & 1) ? -to_double(im(v)) : to_double(re(v))) * jb.scale;
                     jb.out_r[at] = r;
                     jb.out_r32[at] = (float)r;
                 }
@@ -858,11 +859,14 @@ __global__ void __launch_bounds__(256) k_line(const LineJob* __restrict__ jobs, 
 }
 
 int line_lines(int kind, int P, long long lines, int nsm) {
-    // Complex lines per CTA: as many as fill kLineSmem (four CTAs an SM, for
-    // lines of a few hundred values), but no more than leave two CTAs an SM
-    // busy over all lines of the launch; at least one.
+    // Complex lines per CTA: as many as fill kLineSmem (eight CTAs of at most 128
+    // threads an SM, for lines of a few hundred values), but no more than leave
+    // two CTAs an SM busy over all lines of the launch; at least one.  Passes of
+    // 48^4 to axis 0 and of 512 data sets with 28 KB and 128 threads 310 and 541
+    // us, 56 KB and 256 threads 317 and 553, 75 KB 331 and 609, 20 KB and 96
+    // threads 312 and 678.
     const bool packed = kind == kLineRealRows || kind == kLineLast || kind == kLineSpecRows;
-    constexpr size_t kLineSmem = 56 * 1024;
+    constexpr size_t kLineSmem = 28 * 1024;
     int f = 1;
     while (f < kMaxLines / 2 && line_smem_bytes(P, f + 1) <= kLineSmem) ++f;
     const long long spread = std::max<long long>(1, (packed ? (lines + 1) / 2 : lines) / (2LL * nsm));
@@ -891,7 +895,7 @@ cudaError_t line_plan(LineJob* jobs_h, int n, int kind, long long* blocks_out, s
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     *blocks_out = blocks;
     *sm_out = sm;
-    *threads_out = std::min(256, std::max(64, (work + 31) / 32 * 32));   // about a butterfly a thread
+    *threads_out = std::min(128, std::max(64, (work + 31) / 32 * 32));   // about a butterfly a thread
     return cudaSuccess;
 }
 

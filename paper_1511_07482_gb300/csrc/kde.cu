@@ -36,34 +36,6 @@ __global__ void __launch_bounds__(256) k_kde_table(KdeDesc g, KdeKernel kn, floa
     }
 }
 
-// Two FP32 values in a 64-bit register pair and the packed operations on
-// them (both halves rounded as the scalar operations round): the FP32 pipes
-// take a packed instruction in two cycles, so arithmetic that fills them
-// leaves every other issue slot to loads and control.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-// a - b: one rounding, as the subtraction's
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack2(-1.f, -1.f), a); }
-
 // The estimate on a tile of 2 BY rows (axis d - 2) by BX * T nodes (axis
 // d - 1) at one index of the outer axes; a thread has T consecutive nodes of
 // two rows (packed pairs, BY rows apart), and KZ threads share each of them,
