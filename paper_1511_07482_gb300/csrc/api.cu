@@ -772,21 +772,28 @@ static int run_graph(kdefft_ctx c, const std::vector<long long>& sig, F&& issue)
     }
     auto it = c->gcache.find(sig);
     if (it == c->gcache.end()) {
+        // a new signature runs at once, and is captured for the next time while
+        // the GPU works on it (captured first and then launched, the first call on
+        // a new data set took 673 us against 568 for psi_4 with its binning,
+        // 969 against 837 for the 4-D plug-in, 616 against 572 for a selection)
+        const int64_t l0 = c->launches;
+        KCHK(issue());
+        if (c->graph_gen != c->buf_gen) return KDEFFT_OK;   // the run reallocated a buffer: keep nothing
+        const int64_t launches = c->launches - l0;
         if (!c->cap_stream) KCU(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
         if (c->gcache.size() >= 64) KCHK(drop_graphs(c));
         // capture on the library's own stream (the caller's may be the legacy
         // default stream, which cannot be captured); replay on the caller's
         cudaStream_t user = c->stream;
-        const int64_t l0 = c->launches;
         KCU(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeRelaxed));
         c->stream = c->cap_stream;
         const int r = issue();
         c->stream = user;
+        c->launches = l0 + launches;
         cudaGraph_t g = nullptr;
         const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
         if (r != KDEFFT_OK) {
             if (g) cudaGraphDestroy(g);
-            c->launches = l0;
             return r;
         }
         KCU(e);
@@ -794,20 +801,11 @@ static int run_graph(kdefft_ctx c, const std::vector<long long>& sig, F&& issue)
         const cudaError_t ei = cudaGraphInstantiate(&ex, g, 0);
         cudaGraphDestroy(g);
         KCU(ei);
-        if (c->graph_gen != c->buf_gen) {   // the capture itself reallocated a buffer: run it once, keep nothing
-            const cudaError_t el = cudaGraphLaunch(ex, c->stream);
-            const cudaError_t es = cudaStreamSynchronize(c->stream);
-            cudaGraphExecDestroy(ex);
-            KCU(el);
-            KCU(es);
-            return KDEFFT_OK;
-        }
-        it = c->gcache.emplace(sig, kdefft_ctx_s::GraphEntry{ex, c->launches - l0}).first;
-        c->launches = l0;
+        c->gcache.emplace(sig, kdefft_ctx_s::GraphEntry{ex, launches});
         c->graphs_captured++;
-    } else {
-        c->graph_replays++;
+        return KDEFFT_OK;
     }
+    c->graph_replays++;
     c->launches += it->second.launches;
     KCU(cudaGraphLaunch(it->second.exec, c->stream));
     return KDEFFT_OK;
