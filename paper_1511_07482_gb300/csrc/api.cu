@@ -2232,12 +2232,17 @@ static int group_order(const ReqSet& rs, const int* ids, int n, int d) {
     return R;
 }
 
-// Points of a FP32 lag tile (per launch, 1024 / 2048 / 4096 points): one
-// bandwidth 10.7 / 12.5 / 16.1 us, plug-in in 4-D 32 / 41 / 58 us, 256 LSCV
-// bandwidths 17 / 15 / 17 us; large batches pay for the smaller tiles (psi_4 of
-// 256 bandwidths on 128^3 78 / 66 / 62 us, 512 data sets x 16 148 / 134 / 135
-// us), a few percent of calls that take 0.6 and 6.6 ms.
-static constexpr long long kLagTile = 1024;
+// Points of a lag tile.  FP64: 256, one per thread (the points are slow on the
+// FP64 pipe: more CTAs in flight).  FP32, by the item's half box alone, so that
+// its sum does not depend on the batch it comes in: small tiles spread a lone
+// bandwidth over SMs, large ones save a large half box its per-tile work.  Per
+// launch with 1024 / 2048 / 4096 points: one bandwidth in 2-D 10.7 / 12.5 / 16.1
+// us, the 4-D plug-in (14 K points) 32 / 41 / 58 us, 256 LSCV bandwidths 17 / 15
+// / 17 us, psi_4 of 256 bandwidths on 128^3 (8 K to 30 K points) 78 / 66 / 62 us.
+static long long lag_tile_points(bool dbl, long long pts) {
+    if (dbl) return 32 * kLagSlices;
+    return pts <= 16384 ? 1024 : pts <= 65536 ? 2048 : 4096;
+}
 
 // A lag work item to be: n consecutive grids of one dataset, covariances and
 // plan, from ids[first] of a run's grid list.  Form: nv Gaussians and all
@@ -2404,10 +2409,6 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
         return groups[a].R != groups[b].R ? groups[a].R < groups[b].R : groups[a].nv < groups[b].nv;
     });
     HermiteIndex& hx = hindex();
-    // fixed tiles, so that an item's sum depends on the item alone, not on
-    // the batch it came in: kLagTile points in FP32, 256 in FP64 (the points
-    // are slow on the FP64 pipe: more CTAs in flight, one point per thread)
-    const long long T = dbl ? 32 * kLagSlices : kLagTile;
     const size_t ni = ord.size();
     LagBatch bt;
     bt.dbl = dbl;
@@ -2429,7 +2430,7 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
         npts[q] = pts;
         int N = 1;   // Hermite values
         for (int i = 1; i <= d; ++i) N = N * (gr.R + i) / i;
-        const long long nt = (pts + T - 1) / T;
+        const long long T = lag_tile_points(dbl, pts), nt = (pts + T - 1) / T;
         tile0[q + 1] = tile0[q] + nt;
         part0[q + 1] = part0[q] + nt * (dbl ? kLagSlices : 1) * gr.sums();
         woff[q + 1] = woff[q] + (long long)nsig * (gr.nv < 0 ? 2 * N : gr.sums());
@@ -2494,7 +2495,7 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
             it.part0 = part0[q];
             it.nout = gr.n;
             it.out0 = out0[q];
-            const long long pts = npts[q];
+            const long long pts = npts[q], T = lag_tile_points(dbl, pts);
             long long f = 0;
             for (long long tq = tile0[q]; tq < tile0[q + 1]; ++tq, f += T)
                 bt.tiles[tq] = LagTile{(int)q, (int)std::min(T, pts - f), f};
@@ -2678,7 +2679,6 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
     if (!c->lag || !lag_single_form(d, f.R, f.nv, f.nsig)) return KDEFFT_ERR_UNSUPPORTED;
     HostTimer hbuild(c, "host:direct");
     auto ds_of = [&](size_t h) { return owner[many ? h : 0]; };
-    const long long T = dbl ? 32 * kLagSlices : kLagTile;
     const int per = dbl ? kLagSlices : 1, nk = f.kernels();
     std::vector<std::array<int, 4>> L(n);
     std::vector<int> tile0(n + 1);
@@ -2695,6 +2695,7 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
             }
             long long pts = L[h][0] + 1;
             for (int k = 1; k < d; ++k) pts *= 2 * L[h][k] + 1;
+            const long long T = lag_tile_points(dbl, pts);
             tile0[h + 1] = (int)((pts + T - 1) / T);
         }
     });
@@ -2755,6 +2756,7 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
             it.out0 = (int)(h * nk);
             long long pts = L[h][0] + 1;
             for (int k = 1; k < d; ++k) pts *= 2 * L[h][k] + 1;
+            const long long T = lag_tile_points(dbl, pts);
             long long at = 0;
             for (int t = tile0[h]; t < tile0[h + 1]; ++t, at += T)
                 tiles[t] = LagTile{(int)h, (int)std::min(T, pts - at), at};
@@ -2763,8 +2765,13 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
     if (!ok) return KDEFFT_ERR_UNSUPPORTED;
     int N = 1;   // Hermite values
     for (int i = 1; i <= d; ++i) N = N * (f.R + i) / i;
-    const double fl = (double)nt * (double)T * (f.nsig * (2.0 * d * d + 3.0 * N) + 12.0 * nk);   // (whole tiles)
-    const double by = (double)nt * (double)T * sizeof(real);
+    double pts_all = 0.0;
+    for (size_t h = 0; h < n; ++h) {
+        double pts = L[h][0] + 1;
+        for (int k = 1; k < d; ++k) pts *= 2 * L[h][k] + 1;
+        pts_all += pts;
+    }
+    const double fl = pts_all * (f.nsig * (2.0 * d * d + 3.0 * N) + 12.0 * nk), by = pts_all * sizeof(real);
     double* hout = (double*)c->h_out.p;
     const std::vector<long long> sig = {10, dbl ? 8 : 4, d, f.R, f.nv, (long long)n, nt, (long long)bytes, (long long)oT,
                                         (long long)oW, (long long)oD, (long long)(uintptr_t)h8, (long long)(uintptr_t)d8,

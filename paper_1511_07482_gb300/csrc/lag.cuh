@@ -267,7 +267,7 @@ __device__ __forceinline__ void lag_tiles(const LagJob<real>& jb) {
         }
         // the item's last block adds its partials: 256 shares (whatever the
         // block's size) of every 256 / NQ-th slot, then a fixed tree
-        __threadfence();
+        if (dbl || threadIdx.x < NO) __threadfence();   // the threads that wrote them
         __syncthreads();
         if (threadIdx.x == 0)
             lastone = atomicAdd(jb.done + tl.item, 1u) == (unsigned)(it.ntile * per) - 1u;
