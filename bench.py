@@ -194,7 +194,7 @@ def roofline_of(kstats, hbm, smmax, src):
 
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("engine.cu", "engine.cuh", "lag.cu", "devutil.cuh"):
+    for f in ("engine.cu", "engine.cuh", "lag.cuh", "devutil.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1511_07482_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
