@@ -2249,7 +2249,8 @@ static long long lag_tile_points(bool dbl, long long pts) {
 // partials of order R (nv >= 0), or dense, two kernels up to order R (nv < 0).
 struct LagGroup {
     int first, n, R, nv;
-    int sums() const {   // kernels that its launch sums (the dense form and merged ones: maybe one more than n)
+    bool two = true;   // no weights on a third covariance
+    int kernels() const {   // of its launch's form (the dense one and merged ones: maybe one more than n)
         return nv < 0 || (R == 0 && nv == 2) ? 2 : n;
     }
 };
@@ -2284,7 +2285,10 @@ static void lag_groups(const ReqSet& rs, const std::vector<int>& ids, int a, int
     for (int i = a + nv; whole && i < b; ++i)
         whole = rs.grids[ids[i]].order == R && rs.grids[ids[i]].place == i - a - nv;
     if (whole && lag_single_form(d, R, nv, rs.specs[g.spec].nsig)) {
-        out.push_back({a, b - a, R, nv});
+        LagGroup gr{a, b - a, R, nv};
+        for (int i = a; i < b; ++i)
+            for (const Term& t : rs.grids[ids[i]].terms) gr.two = gr.two && t.sig < 2;
+        out.push_back(gr);
         return;
     }
     for (int i = a; i < b; i += 2) {
@@ -2345,7 +2349,7 @@ static bool lag_item_sigmas(LagItem<real>& it, const Mat* sig, int nsig) {
 
 // The lag-domain work of one precision in a run, built on the host: the
 // items (LagItem<real>), their tiles and weights, the forms (R, nv, first
-// tile, tiles; one launch each) and the grids in the order of the results.
+// tile, tiles, two covariances; one launch each) and the grids in the order of the results.
 // run_lag builds it; issue_lag uploads and launches the batches of both
 // precisions of a run together.
 struct LagBatch {
@@ -2358,7 +2362,7 @@ struct LagBatch {
     std::vector<float> w32;              // the weights (w64 for FP64)
     std::vector<double> w64;
     std::vector<LagTile> tiles;
-    std::vector<std::array<int, 4>> classes;
+    std::vector<std::array<int, 5>> classes;
     std::vector<int> grids;
     double fl = 0.0, by = 0.0;   // algorithmic flops and bytes of the batch
     template <typename real>
@@ -2406,7 +2410,8 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
     std::vector<size_t> ord(groups.size());
     for (size_t i = 0; i < ord.size(); ++i) ord[i] = i;
     std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) {
-        return groups[a].R != groups[b].R ? groups[a].R < groups[b].R : groups[a].nv < groups[b].nv;
+        const LagGroup &x = groups[a], &y = groups[b];
+        return x.R != y.R ? x.R < y.R : x.nv != y.nv ? x.nv < y.nv : x.two < y.two;
     });
     HermiteIndex& hx = hindex();
     const size_t ni = ord.size();
@@ -2432,11 +2437,12 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
         for (int i = 1; i <= d; ++i) N = N * (gr.R + i) / i;
         const long long T = lag_tile_points(dbl, pts), nt = (pts + T - 1) / T;
         tile0[q + 1] = tile0[q] + nt;
-        part0[q + 1] = part0[q] + nt * (dbl ? kLagSlices : 1) * gr.sums();
-        woff[q + 1] = woff[q] + (long long)nsig * (gr.nv < 0 ? 2 * N : gr.sums());
+        part0[q + 1] = part0[q] + nt * (dbl ? kLagSlices : 1) * lag_sums(d, gr.R, gr.nv, dbl, gr.two);
+        woff[q + 1] = woff[q] + (long long)nsig * (gr.nv < 0 ? 2 * N : gr.kernels());
         out0[q + 1] = out0[q] + gr.n;
-        if (bt.classes.empty() || bt.classes.back()[0] != gr.R || bt.classes.back()[1] != gr.nv)
-            bt.classes.push_back({gr.R, gr.nv, (int)tile0[q], 0});
+        if (bt.classes.empty() || bt.classes.back()[0] != gr.R || bt.classes.back()[1] != gr.nv ||
+            bt.classes.back()[4] != (int)gr.two)
+            bt.classes.push_back({gr.R, gr.nv, (int)tile0[q], 0, (int)gr.two});
         bt.classes.back()[3] += (int)nt;
         bt.fl += (double)pts * (nsig * (2.0 * d * d + 3.0 * N) + 12.0 * gr.n);
         bt.by += (double)pts * sizeof(real);
@@ -2580,7 +2586,7 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
         sig.insert(sig.end(), {bt.dbl ? 8 : 4, bt.d, bt.nitems, (long long)bt.tiles.size(), (long long)lay[b].oI,
                                (long long)lay[b].oT, (long long)lay[b].oW, (long long)lay[b].oD,
                                (long long)lay[b].out0, (long long)lay[b].slot0});
-        for (const auto& cl : bt.classes) sig.insert(sig.end(), {cl[0], cl[1], cl[2], cl[3]});
+        for (const auto& cl : bt.classes) sig.insert(sig.end(), {cl[0], cl[1], cl[2], cl[3], cl[4]});
     }
     // a run with batches of both precisions launches its FP64 batch on the
     // side stream, beside the FP32 one (the two touch disjoint partials,
@@ -2619,6 +2625,7 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
                 auto go = [&](auto zero) -> cudaError_t {
                     using real = decltype(zero);
                     LagJob<real> j = lag_job<real>(c, cl[2], cl[3]);
+                    j.nsum2 = cl[4];
                     j.items = (const LagItem<real>*)(dbase + lay[b].oI);
                     j.tiles = (const LagTile*)(dbase + lay[b].oT);
                     j.wpool = (const real*)(dbase + lay[b].oW);
@@ -2680,6 +2687,9 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
     HostTimer hbuild(c, "host:direct");
     auto ds_of = [&](size_t h) { return owner[many ? h : 0]; };
     const int per = dbl ? kLagSlices : 1, nk = f.kernels();
+    bool two = true;   // no weights on a third covariance
+    for (size_t i = 0; i < f.w.size(); ++i) two = two && (f.w[i] == 0.0 || (int)(i % f.nsig) < 2);
+    const int ns = per * lag_sums(d, f.R, f.nv, dbl, two);   // sums of a tile
     std::vector<std::array<int, 4>> L(n);
     std::vector<int> tile0(n + 1);
     std::atomic<bool> ok{true};
@@ -2723,7 +2733,7 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
     KCHK(staging_wait(c));
     KCHK(c->h_items.ensure(bytes));
     KCHK(c->items.ensure(bytes));
-    KCHK(c->partial.ensure(sizeof(double) * (size_t)nt * per * nk));
+    KCHK(c->partial.ensure(sizeof(double) * (size_t)nt * ns));
     KCHK(flush_reads(c));
     KCHK(c->h_out.ensure(sizeof(double) * n * nk));
     unsigned char* h8 = (unsigned char*)c->h_items.p;
@@ -2751,7 +2761,7 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
             it.sigs = sigs;
             it.tile0 = tile0[h];
             it.ntile = tile0[h + 1] - tile0[h];
-            it.part0 = (long long)tile0[h] * per * nk;
+            it.part0 = (long long)tile0[h] * ns;
             it.nout = nk;
             it.out0 = (int)(h * nk);
             long long pts = L[h][0] + 1;
@@ -2773,13 +2783,14 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
     }
     const double fl = pts_all * (f.nsig * (2.0 * d * d + 3.0 * N) + 12.0 * nk), by = pts_all * sizeof(real);
     double* hout = (double*)c->h_out.p;
-    const std::vector<long long> sig = {10, dbl ? 8 : 4, d, f.R, f.nv, (long long)n, nt, (long long)bytes, (long long)oT,
+    const std::vector<long long> sig = {10, dbl ? 8 : 4, d, f.R, f.nv, two ? 2 : 3, (long long)n, nt, (long long)bytes, (long long)oT,
                                         (long long)oW, (long long)oD, (long long)(uintptr_t)h8, (long long)(uintptr_t)d8,
                                         (long long)(uintptr_t)c->partial.p, (long long)(uintptr_t)hout};
     auto issue = [&]() -> int {
         KCU(cudaMemcpyAsync(d8, h8, bytes, cudaMemcpyHostToDevice, c->stream));
         cudaEvent_t ev = prof_start(c);
         LagJob<real> j = lag_job<real>(c, 0, (int)nt);
+        j.nsum2 = two;
         j.items = (const LagItem<real>*)d8;
         j.tiles = (const LagTile*)(d8 + oT);
         j.wpool = (const real*)(d8 + oW);

@@ -16,5 +16,13 @@ bool lag_single_form(int d, int R, int nv, int nsig) {
     return R == 2 || (R == 4 && nv == 0 && nsig == 1);
 }
 
+int lag_sums(int d, int R, int nv, bool dbl, bool two) {
+    if (nv < 0) return 2;
+    int members = R > 0 ? 1 : 0;
+    for (int i = 1; i < d && R > 0; ++i) members = members * (R + i) / i;
+    if (!dbl) return nv + members;
+    return ((nv > 0 ? 1 : 0) + members) * (R > 2 ? 1 : two ? 2 : MAXSIG);
+}
+
 template cudaError_t launch_lag<float>(int, int, int, const LagJob<float>&, cudaStream_t);
 }  // namespace kdefft

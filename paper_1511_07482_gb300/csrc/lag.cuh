@@ -33,14 +33,21 @@ __device__ __forceinline__ uint32_t inv_div(uint32_t n, uint32_t m, int sh) {
 //             weighted sum over the covariances: LSCV and SCV values and
 //             gradients (R = 2), psi_r (NV = 0, one covariance for R > 2)
 //   NV = -1   two kernels (or one), each any sum of partials up to order R
-template <int D, int R, int NV>
+// SG: covariances that may have weights (a FP64 group without weights on the
+// third one has a kernel of its own).
+template <int D, int R, int NV, int SG>
 struct LagForm {
     static constexpr bool dense = NV < 0;
     static constexpr int N = cx_binom(D + R, D);                          // Hermite values
     static constexpr int N0 = R > 0 ? cx_binom(D + R - 1, D) : 0;         // the first of order R
     static constexpr int NO = dense ? 2 : NV + (R > 0 ? N - N0 : 0);      // kernels
-    static constexpr int NS = (!dense && R > 2) ? 1 : MAXSIG;             // covariances
+    static constexpr int NS = (!dense && R > 2) ? 1 : SG;                 // covariances
     static constexpr int at(int o) { return o < NV ? 0 : N0 + (o - NV); }
+    // FP64 groups sum the Gaussian (if any) and each partial of order R per
+    // covariance, and weigh the sums at the end
+    static constexpr int V = NV > 0 ? 1 : 0;
+    static constexpr int NI = V + (R > 0 ? N - N0 : 0);
+    static constexpr int sum_of(int o) { return o < NV ? 0 : V + (o - NV); }
 };
 // values padded to whole warp reductions: 32s, then a power of two
 __host__ __device__ constexpr int lag_chunk(int left) {
@@ -104,23 +111,31 @@ __device__ __forceinline__ void warp_sums_all(T* v, int lane, Add add, Give shfl
 // that share them are summed from one evaluation (psi_4 in three dimensions: 15
 // kernels from 35 Hermite values, where pairs of kernels evaluated them 8
 // times), covariances without a weight in the group are left out, and the warp
-// reductions take a group's kernels together.
+// reductions take a group's kernels together.  FP64 groups do without what is
+// not a point's own: weights and normalisers apply to the sums of each
+// covariance, and where only Gaussians are asked for, the quadratic form takes
+// the products x_a x_b once for all covariances (SCV values of 5 bandwidths on
+// 61 x 97 x 45 48 -> 42 us, values and gradients of 16 on 256^2 35 -> 31 us).
 // Per launch, against pairs of kernels with the sums of their tiles in a launch
 // of their own (4 to 6 us more): psi_4 of 256 bandwidths on 128^3 78 us (329),
 // 512 data sets x 16 LSCV bandwidths with gradients 122 us (364), SCV with
 // gradients in FP64, 16 bandwidths on 256^2, 36 us (145).
-template <typename real, int D, int R, int NV>
+template <typename real, int D, int R, int NV, int SG>
 __device__ __forceinline__ void lag_tiles(const LagJob<real>& jb) {
-    using F = LagForm<D, R, NV>;
+    using F = LagForm<D, R, NV, SG>;
     constexpr bool dbl = sizeof(real) == 8;
+    constexpr bool late = dbl && !F::dense;   // weights at the end
+    constexpr int NSUM = late ? F::NI * F::NS : F::NO;   // sums of a tile
     constexpr HTab<D, R> ht{};
-    constexpr int N = F::N, NO = F::NO, NP = lag_padded(NO), NS = F::NS;
+    constexpr int N = F::N, NO = F::NO, NP = lag_padded(NSUM), NS = F::NS;
     constexpr int NW = F::dense ? 2 * MAXSIG * N : NO * MAXSIG;
     using Sum = typename std::conditional<dbl, double, DFloat>::type;
     __shared__ real Ws[NW];
     __shared__ __align__(8) LagItem<real> it;
     __shared__ Sum red[dbl ? 1 : 8][dbl ? 1 : NP];
     __shared__ double fin[256];
+    constexpr int NX = (late && R == 0) ? D * (D + 1) / 2 : 1;
+    __shared__ double quad[MAXSIG][NX];   // -x^T Sigma^-1 x / 2 on the products x_a x_b, a <= b
     __shared__ int lastone;
     static_assert(sizeof(LagItem<real>) % 8 == 0, "staged by 8-byte words");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -137,6 +152,13 @@ __device__ __forceinline__ void lag_tiles(const LagJob<real>& jb) {
             const unsigned long long* a = reinterpret_cast<const unsigned long long*>(&src);
             unsigned long long* b = reinterpret_cast<unsigned long long*>(&it);
             for (int t = threadIdx.x; t < (int)(sizeof(LagItem<real>) / 8); t += blockDim.x) b[t] = a[t];
+            if constexpr (late && R == 0) {
+                for (int t = threadIdx.x; t < MAXSIG * NX; t += blockDim.x) {
+                    int k = t % NX, a0 = 0;
+                    while (k >= D - a0) k -= D - a0++;
+                    quad[t / NX][t % NX] = (k == 0 ? -0.5 : -1.0) * src.lam[t / NX][a0 * MAXD + a0 + k];
+                }
+            }
             const int nsig = src.nsig, w_off = src.w_off;
             for (int t = threadIdx.x; t < NW; t += blockDim.x) {
                 if constexpr (F::dense) {   // [kernel][covariance][Hermite index]
@@ -190,65 +212,115 @@ __device__ __forceinline__ void lag_tiles(const LagJob<real>& jb) {
             real x[D];
 #pragma unroll
             for (int k = 0; k < D; ++k) x[k] = it.delta[k] * (real)j[k];
-            real v[NO];
+            if constexpr (late) {
+                double xx[NX];
+                if constexpr (R == 0) {
+                    int k = 0;
 #pragma unroll
-            for (int o = 0; o < NO; ++o) v[o] = real(0);
+                    for (int a = 0; a < D; ++a)
 #pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                if ((sigs >> s) & 1) {
-                    real z[D];
-                    real q = 0;
+                        for (int b = a; b < D; ++b) xx[k++] = x[a] * x[b];
+                }
 #pragma unroll
-                    for (int a = 0; a < D; ++a) {
-                        real zz = 0;
+                for (int s = 0; s < NS; ++s) {
+                    if ((sigs >> s) & 1) {
+                        double z[D], q = 0.0;
+                        if constexpr (R == 0) {
 #pragma unroll
-                        for (int b = 0; b < D; ++b) zz += it.lam[s][a * MAXD + b] * x[b];
-                        z[a] = zz;
-                        q += x[a] * zz;
-                    }
-                    const real e = it.nrm[s] * exp(real(-0.5) * q);
-                    real He[N];
-                    He[0] = real(1);
+                            for (int k = 0; k < NX; ++k) q += quad[s][k] * xx[k];
+                        } else {
 #pragma unroll
-                    for (int t = 1; t < N; ++t) {
-                        real w = z[ht.piv[t]] * He[ht.par[t]];
+                            for (int a = 0; a < D; ++a) {
+                                double zz = 0.0;
 #pragma unroll
-                        for (int r = 0; r < D; ++r)
-                            if (r < ht.nred[t])
-                                w -= real(ht.rc[t][r]) * it.lam[s][ht.piv[t] * MAXD + ht.rj[t][r]] * He[ht.ridx[t][r]];
-                        He[t] = w;
-                    }
-                    if constexpr (F::dense) {
-                        real pa = 0, pb = 0;
-#pragma unroll
-                        for (int t = 0; t < N; ++t) {
-                            pa += Ws[s * N + t] * He[t];
-                            pb += Ws[(MAXSIG + s) * N + t] * He[t];
+                                for (int b = 0; b < D; ++b) zz += it.lam[s][a * MAXD + b] * x[b];
+                                z[a] = zz;
+                                q += x[a] * zz;
+                            }
+                            q *= -0.5;
                         }
-                        v[0] += e * pa;
-                        v[1] += e * pb;
-                    } else {
+                        const double we = wa * exp(q);
+                        if constexpr (F::V > 0) acc[s] += we;
+                        if constexpr (R > 0) {
+                            double He[N];
+                            He[0] = 1.0;
 #pragma unroll
-                        for (int o = 0; o < NO; ++o) v[o] = fma(e, Ws[o * MAXSIG + s] * He[F::at(o)], v[o]);
+                            for (int t = 1; t < N; ++t) {
+                                double w = z[ht.piv[t]] * He[ht.par[t]];
+#pragma unroll
+                                for (int r = 0; r < D; ++r)
+                                    if (r < ht.nred[t])
+                                        w -= double(ht.rc[t][r]) * it.lam[s][ht.piv[t] * MAXD + ht.rj[t][r]] *
+                                             He[ht.ridx[t][r]];
+                                He[t] = w;
+                            }
+#pragma unroll
+                            for (int k = F::V; k < F::NI; ++k)
+                                acc[k * NS + s] = fma(we, He[F::N0 + k - F::V], acc[k * NS + s]);
+                        }
                     }
                 }
-            }
+            } else {
+                real v[NO];
 #pragma unroll
-            for (int o = 0; o < NO; ++o) {
-                if constexpr (dbl) {
-                    acc[o] = fma(wa, v[o], acc[o]);
-                } else {   // two-sum of the pair and the unrounded product
-                    const float s = fmaf(wa, v[o], acc[o].h);
-                    const float b = s - acc[o].h;
-                    acc[o].l += (acc[o].h - (s - b)) + fmaf(wa, v[o], -b);
-                    acc[o].h = s;
+                for (int o = 0; o < NO; ++o) v[o] = real(0);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    if ((sigs >> s) & 1) {
+                        real z[D];
+                        real q = 0;
+#pragma unroll
+                        for (int a = 0; a < D; ++a) {
+                            real zz = 0;
+#pragma unroll
+                            for (int b = 0; b < D; ++b) zz += it.lam[s][a * MAXD + b] * x[b];
+                            z[a] = zz;
+                            q += x[a] * zz;
+                        }
+                        const real e = it.nrm[s] * exp(real(-0.5) * q);
+                        real He[N];
+                        He[0] = real(1);
+#pragma unroll
+                        for (int t = 1; t < N; ++t) {
+                            real w = z[ht.piv[t]] * He[ht.par[t]];
+#pragma unroll
+                            for (int r = 0; r < D; ++r)
+                                if (r < ht.nred[t])
+                                    w -= real(ht.rc[t][r]) * it.lam[s][ht.piv[t] * MAXD + ht.rj[t][r]] * He[ht.ridx[t][r]];
+                            He[t] = w;
+                        }
+                        if constexpr (F::dense) {
+                            real pa = 0, pb = 0;
+#pragma unroll
+                            for (int t = 0; t < N; ++t) {
+                                pa += Ws[s * N + t] * He[t];
+                                pb += Ws[(MAXSIG + s) * N + t] * He[t];
+                            }
+                            v[0] += e * pa;
+                            v[1] += e * pb;
+                        } else {
+#pragma unroll
+                            for (int o = 0; o < NO; ++o) v[o] = fma(e, Ws[o * MAXSIG + s] * He[F::at(o)], v[o]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int o = 0; o < NO; ++o) {
+                    if constexpr (dbl) {
+                        acc[o] = fma(wa, v[o], acc[o]);
+                    } else {   // two-sum of the pair and the unrounded product
+                        const float s = fmaf(wa, v[o], acc[o].h);
+                        const float b = s - acc[o].h;
+                        acc[o].l += (acc[o].h - (s - b)) + fmaf(wa, v[o], -b);
+                        acc[o].h = s;
+                    }
                 }
             }
         }
         double* part = jb.partial + it.part0 +
-                       (long long)NO * ((long long)(tix - it.tile0) * (dbl ? kLagSlices : 1) + (dbl ? s0 + warp : 0));
+                       (long long)NSUM * ((long long)(tix - it.tile0) * (dbl ? kLagSlices : 1) + (dbl ? s0 + warp : 0));
         if constexpr (dbl) {
-            warp_sums_all<0, NO>(
+            warp_sums_all<0, NSUM>(
                 acc, lane, [](double a, double b) { return a + b; },
                 [](double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }, [&](int o, double x) { part[o] = x; });
         } else {
@@ -274,14 +346,16 @@ __device__ __forceinline__ void lag_tiles(const LagJob<real>& jb) {
         __syncthreads();
         if (!lastone) continue;
         __threadfence();
-        constexpr int NQ = NO <= 1 ? 1 : NO <= 2 ? 2 : NO <= 4 ? 4 : NO <= 8 ? 8 : NO <= 16 ? 16 : NO <= 32 ? 32 : 64;
+        constexpr int NQ = NSUM <= 1 ? 1 : NSUM <= 2 ? 2 : NSUM <= 4 ? 4 : NSUM <= 8 ? 8 : NSUM <= 16 ? 16
+                           : NSUM <= 32 ? 32 : 64;
+        static_assert(NSUM <= 64, "a share of the final sum per kernel");
         const int slots = it.ntile * (dbl ? kLagSlices : 1);
         const double* all = jb.partial + it.part0;
         for (int t = threadIdx.x; t < 256; t += blockDim.x) {
             const int o = t % NQ;
             double sum = 0.0;
-            if (o < NO)
-                for (int k = t / NQ; k < slots; k += 256 / NQ) sum += __ldcg(all + (long long)k * NO + o);
+            if (o < NSUM)
+                for (int k = t / NQ; k < slots; k += 256 / NQ) sum += __ldcg(all + (long long)k * NSUM + o);
             fin[t] = sum;
         }
         __syncthreads();
@@ -290,13 +364,22 @@ __device__ __forceinline__ void lag_tiles(const LagJob<real>& jb) {
             __syncthreads();
         }
         for (int o = threadIdx.x; o < NO; o += blockDim.x)
-            if (o < it.nout) jb.out[it.out0 + o] = fin[o] * it.scale;
+            if (o < it.nout) {
+                double v = 0.0;
+                if constexpr (late) {
+                    for (int s = 0; s < NS; ++s)
+                        if ((sigs >> s) & 1) v += (Ws[o * MAXSIG + s] * it.nrm[s]) * fin[F::sum_of(o) * NS + s];
+                } else {
+                    v = fin[o];
+                }
+                jb.out[it.out0 + o] = v * it.scale;
+            }
     }
 }
 
-template <typename real, int D, int R, int NV>
+template <typename real, int D, int R, int NV, int SG>
 __global__ void __launch_bounds__(256) k_lag(const __grid_constant__ LagJob<real> jb) {
-    lag_tiles<real, D, R, NV>(jb);
+    lag_tiles<real, D, R, NV, SG>(jb);
 }
 
 // FP32 groups with d <= 2 are held to 64 registers, four CTAs an SM (512 data
@@ -305,7 +388,7 @@ __global__ void __launch_bounds__(256) k_lag(const __grid_constant__ LagJob<real
 // 82 us against 78, SCV gradients 18 and 15 against 12).
 template <typename real, int D, int R, int NV>
 __global__ void __launch_bounds__(256, 4) k_lag_occ4(const __grid_constant__ LagJob<real> jb) {
-    lag_tiles<real, D, R, NV>(jb);
+    lag_tiles<real, D, R, NV, MAXSIG>(jb);
 }
 
 // dense forms instantiated for (d, R): FP32 d <= 2 up to R = 8, d = 3 up to 6,
@@ -325,8 +408,10 @@ template <typename real, int D, int R, int NV>
 static cudaError_t lag_go(const LagJob<real>& j, cudaStream_t st) {
     if constexpr (sizeof(real) == 4 && D <= 2 && NV >= 0)
         k_lag_occ4<real, D, R, NV><<<j.grid, j.block, 0, st>>>(j);
+    else if (sizeof(real) == 8 && NV >= 0 && R <= 2 && j.nsum2)
+        k_lag<real, D, R, NV, (sizeof(real) == 8 && NV >= 0 && R <= 2) ? 2 : MAXSIG><<<j.grid, j.block, 0, st>>>(j);
     else
-        k_lag<real, D, R, NV><<<j.grid, j.block, 0, st>>>(j);
+        k_lag<real, D, R, NV, MAXSIG><<<j.grid, j.block, 0, st>>>(j);
     return cudaGetLastError();
 }
 
