@@ -2239,9 +2239,12 @@ static int group_order(const ReqSet& rs, const int* ids, int n, int d) {
 // launch with 1024 / 2048 / 4096 points: one bandwidth in 2-D 10.7 / 12.5 / 16.1
 // us, the 4-D plug-in (14 K points) 32 / 41 / 58 us, 256 LSCV bandwidths 17 / 15
 // / 17 us, psi_4 of 256 bandwidths on 128^3 (8 K to 30 K points) 78 / 66 / 62 us.
-static long long lag_tile_points(bool dbl, long long pts) {
+// A dense pair does far more per point than a group, so its small tiles pay up
+// to larger boxes: the plug-in's launch, whose first order has a box of more
+// than 16 K points, takes 45 us with the groups' line and 39 us with its own.
+static long long lag_tile_points(bool dbl, long long pts, bool dense) {
     if (dbl) return 32 * kLagSlices;
-    return pts <= 16384 ? 1024 : pts <= 65536 ? 2048 : 4096;
+    return pts <= (dense ? 65536 : 16384) ? 1024 : pts <= 65536 ? 2048 : 4096;
 }
 
 // A lag work item to be: n consecutive grids of one dataset, covariances and
@@ -2435,7 +2438,7 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
         npts[q] = pts;
         int N = 1;   // Hermite values
         for (int i = 1; i <= d; ++i) N = N * (gr.R + i) / i;
-        const long long T = lag_tile_points(dbl, pts), nt = (pts + T - 1) / T;
+        const long long T = lag_tile_points(dbl, pts, gr.nv < 0), nt = (pts + T - 1) / T;
         tile0[q + 1] = tile0[q] + nt;
         part0[q + 1] = part0[q] + nt * (dbl ? kLagSlices : 1) * lag_sums(d, gr.R, gr.nv, dbl, gr.two);
         woff[q + 1] = woff[q] + (long long)nsig * (gr.nv < 0 ? 2 * N : gr.kernels());
@@ -2501,7 +2504,7 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
             it.part0 = part0[q];
             it.nout = gr.n;
             it.out0 = out0[q];
-            const long long pts = npts[q], T = lag_tile_points(dbl, pts);
+            const long long pts = npts[q], T = lag_tile_points(dbl, pts, gr.nv < 0);
             long long f = 0;
             for (long long tq = tile0[q]; tq < tile0[q + 1]; ++tq, f += T)
                 bt.tiles[tq] = LagTile{(int)q, (int)std::min(T, pts - f), f};
@@ -2705,7 +2708,7 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
             }
             long long pts = L[h][0] + 1;
             for (int k = 1; k < d; ++k) pts *= 2 * L[h][k] + 1;
-            const long long T = lag_tile_points(dbl, pts);
+            const long long T = lag_tile_points(dbl, pts, false);
             tile0[h + 1] = (int)((pts + T - 1) / T);
         }
     });
@@ -2766,7 +2769,7 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
             it.out0 = (int)(h * nk);
             long long pts = L[h][0] + 1;
             for (int k = 1; k < d; ++k) pts *= 2 * L[h][k] + 1;
-            const long long T = lag_tile_points(dbl, pts);
+            const long long T = lag_tile_points(dbl, pts, false);
             long long at = 0;
             for (int t = tile0[h]; t < tile0[h + 1]; ++t, at += T)
                 tiles[t] = LagTile{(int)h, (int)std::min(T, pts - at), at};
