@@ -130,11 +130,11 @@ int kdefft_bin(kdefft_ctx ctx, const double* X, int64_t n, int d,
 /* kdefft_bin for nds datasets of the same d at once (Sec. 4 step 1 for
  * each): X[i] is dataset i's n[i] x d sample (host or device), lo/hi its
  * grid range (nds x d), M its grid (nds x d).  FP32 linear binning runs as
- * three launches over all datasets (binning, conversion, the one-pass
- * covariance) with one synchronisation in total, and the datasets' counts
- * share one allocation (freed with the last of them); other precisions and
- * rules bin one dataset at a time.  out: nds handles.  On error no dataset
- * is created. */
+ * two launches over all datasets (binning with the moments of the
+ * covariance, conversion) with one synchronisation in total, and the
+ * datasets' counts share one allocation (freed with the last of them); other
+ * precisions and rules bin one dataset at a time.  out: nds handles.  On
+ * error no dataset is created. */
 int kdefft_bin_many(kdefft_ctx ctx, int nds, const double* const* X, const int64_t* n, int d,
                     const double* lo, const double* hi, const int64_t* M, const kdefft_opts* opts,
                     kdefft_ds* out);
@@ -364,7 +364,7 @@ int kdefft_set_autotune(kdefft_ctx ctx, int on);
 int kdefft_autocorr(kdefft_ds ds, const int* A, double* out);
 
 /* CUDA graphs (on by default).  A batch's launch sequence (staging copy,
- * kernels, result copy) is captured once into a CUDA graph under its
+ * kernels) is captured once into a CUDA graph under its
  * launch signature -- every device and pinned-host pointer, size, tile
  * count and launch shape -- and replayed when a later batch has the same
  * signature (the work items themselves are data read at replay time).  At

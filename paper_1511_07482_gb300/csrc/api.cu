@@ -3519,13 +3519,10 @@ int kdefft_bin(kdefft_ctx c, const double* X, int64_t n, int d, const double* lo
         c->h2d += (int64_t)(sizeof(double) * n * d);
         dX = (const double*)xbuf.p;
     }
-    // outside counter | block partials of the moments
+    // block partials of the moments
     const int mblk = bin_blocks(n, c->nsm);
     const int nv = d + d * d;
     DevBuf misc(&c->cache);
-    KCHK(misc.ensure(sizeof(double) * (16 + (size_t)mblk * nv)));
-    unsigned long long* dOut = (unsigned long long*)misc.p;
-    double* dPart = (double*)misc.p + 16;
     const bool dbl = o.precision == KDEFFT_FP64;
     // covariance for the normal-scale start point, from moments shifted by the
     // grid's centre (block partials summed in block order: the same start
@@ -3536,22 +3533,21 @@ int kdefft_bin(kdefft_ctx c, const double* X, int64_t n, int d, const double* lo
     std::vector<double> part((size_t)mblk * nv);
     if (!dbl && o.binning != KDEFFT_BIN_SIMPLE) {
         // FP32 linear binning: the launch sequence (zeroing, binning with
-        // the moments, fixed point to FP32, one copy of the outside count and
-        // the moment partials to pinned memory) replays as a CUDA graph when its
+        // the moments, fixed point to FP32) replays as a CUDA graph when its
         // pointers and sizes repeat
         int K = 32;   // fixed point with K fractional bits; a cell's total (<= n 2^K) stays below 2^63
         while (K > 8 && (double)n * std::ldexp(1.0, K) >= std::ldexp(1.0, 63)) --K;
         DevBuf& fix = c->binfix;
         KCHK(fix.ensure(8 * ((size_t)ds->ncells + 1)));   // the accumulators, then the outside counter
         KCHK(ds->counts.ensure(4 * (size_t)ds->ncells));
-        // the outside counter and the moment partials come back in one copy
-        // of the whole work buffer (counter at 0, partials from 16)
+        // the outside counter and the moment partials (counter at 0, partials
+        // from 16) are written to pinned memory by the kernels themselves
         const size_t nres = 16 + (size_t)mblk * nv;
         KCHK(c->h_binres.ensure(sizeof(double) * nres));
         double* hres = (double*)c->h_binres.p;
         std::vector<long long> sig = {4, (long long)(uintptr_t)dX, n, d, K, (long long)(uintptr_t)fix.p,
-                                      (long long)(uintptr_t)ds->counts.p, (long long)(uintptr_t)misc.p,
-                                      (long long)(uintptr_t)hres, mblk, ds->ncells, c->nsm};
+                                      (long long)(uintptr_t)ds->counts.p, (long long)(uintptr_t)hres, mblk,
+                                      ds->ncells, c->nsm};
         for (int k = 0; k < d; ++k) {
             long long bits[3];
             std::memcpy(&bits[0], &g.lo[k], 8);
@@ -3564,12 +3560,11 @@ int kdefft_bin(kdefft_ctx c, const double* X, int64_t n, int d, const double* lo
             KCU(cudaMemsetAsync(acc, 0, 8 * ((size_t)ds->ncells + 1), c->stream));
             cudaEvent_t evb = prof_start(c);
             c->launches++;   // the fixed-point-to-FP32 conversion
-            KCU(launch_bin_fixed(dX, n, g, sh, acc, ds->ncells, acc + ds->ncells, std::ldexp(1.0, K), dPart, c->nsm,
-                                 c->stream));
-            KCU(launch_fix_to_f32(acc, (float*)ds->counts.p, ds->ncells, std::ldexp(1.0, -K), acc + ds->ncells, dOut,
-                                  c->nsm, c->stream));
+            KCU(launch_bin_fixed(dX, n, g, sh, acc, ds->ncells, acc + ds->ncells, std::ldexp(1.0, K), hres + 16,
+                                 c->nsm, c->stream));
+            KCU(launch_fix_to_f32(acc, (float*)ds->counts.p, ds->ncells, std::ldexp(1.0, -K), acc + ds->ncells,
+                                  (unsigned long long*)hres, c->nsm, c->stream));
             prof_stop(c, evb, "bin", (double)n * d * 8.0 + (double)ds->ncells * 4.0, (double)n * (1 << d) * 2.0);
-            KCU(cudaMemcpyAsync(hres, misc.p, sizeof(double) * nres, cudaMemcpyDeviceToHost, c->stream));
             return KDEFFT_OK;
         };
         KCHK(run_graph(c, sig, issue));
@@ -3577,6 +3572,9 @@ int kdefft_bin(kdefft_ctx c, const double* X, int64_t n, int d, const double* lo
         std::memcpy(&nout, hres, sizeof(nout));
         std::memcpy(part.data(), hres + 16, sizeof(double) * mblk * nv);
     } else {
+        KCHK(misc.ensure(sizeof(double) * (16 + (size_t)mblk * nv)));   // outside counter | partials
+        unsigned long long* dOut = (unsigned long long*)misc.p;
+        double* dPart = (double*)misc.p + 16;
         KCU(cudaMemsetAsync(misc.p, 0, sizeof(double) * 16, c->stream));
         KCHK(ds->counts.ensure((dbl ? 8 : 4) * (size_t)ds->ncells));
         // only FP64 linear binning accumulates into the counts themselves; the
