@@ -24,6 +24,7 @@
 // corner weights are FP32 products of the FP64 fractions rounded to FP32: a
 // weight's relative error of a few 2^-24 matches the FP32 rounding of the
 // count itself.  FP64 counts use FP64 weights and FP64 atomics.
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 
@@ -70,6 +71,29 @@ __device__ __forceinline__ bool inside(double x, long long klo, long long khi) {
     return key >= klo && key <= khi;
 }
 
+// v 2^e rounded once to FP32 (ties to even), for results of zero or from 2^-94
+// up.  The leading bit goes to the top, what falls below the upper 32 bits
+// leaves a one in the lowest of them (32 bits round to 24 as the 64 would),
+// and the scale is exact.  The conversion instructions from and to 64-bit
+// integers run at the FP64 rate here, so each costs as much as a product in
+// FP64, which is what the pass is bound by: with them (d + 2^d a point) 1e7
+// points on 512^2 take 363 us instead of 250, 1e6 on 128^3 103 instead of 75,
+// 1e6 on 48^4 142 instead of 119.
+__device__ __forceinline__ float scaled_f32(unsigned long long v, int e) {
+    const unsigned int hi = (unsigned int)(v >> 32);
+    const int n = hi ? __clz(hi) : 32 + __clz((unsigned int)v);
+    v <<= n & 63;   // v = 0 has n = 64 and stays zero
+    const unsigned int top = (unsigned int)(v >> 32) | ((unsigned int)v != 0u ? 1u : 0u);
+    return __uint2float_rn(top) * __int_as_float((159 - n + e) << 23);
+}
+
+// w 2^K rounded to an integer (ties to even), w in [0, 1] and qs = 2^K <= 2^32:
+// a 32-bit conversion, which stops at 2^32 - 1, and one more for 2^32
+__device__ __forceinline__ unsigned long long fixed_weight(float w, float qs) {
+    const float v = w * qs;
+    return (unsigned long long)__float2uint_rn(v) + (v >= 4294967296.f ? 1ULL : 0ULL);
+}
+
 // Cell l = min(floor(t), M - 2) and fraction t - l (1 where t reaches M - 1,
 // which the rounding of delta can push past it) of t >= 0, below 2^31: t is
 // m 2^-sh with a 53-bit m, so the cell is m >> sh and the fraction the bits
@@ -81,7 +105,7 @@ __device__ __forceinline__ int cell_f32(double t, int top, float& f) {
     const int sh = min(1075 - (int)((b >> 52) & 0x7ff), 126);   // the sign of -0 does not matter
     const int s = min(sh, 63);
     int l = (int)(m >> s);
-    f = __ull2float_rn(m & ((1ULL << s) - 1)) * __int_as_float((127 - sh) << 23);
+    f = scaled_f32(m << (64 - s), s - 64 - sh);   // s >= 22: the cell's bits leave at the top
     if (l > top) {
         l = top;
         f = 1.f;
@@ -127,10 +151,11 @@ __device__ __forceinline__ int nearest(double x, double lo, double delta, double
 // pairs, half of them at a time, and a pair adds the two neighbours along the
 // last axis with one instruction: three times out of four they share a sector.
 // What is left is FP64: 2 d operations to locate a point and 2 d + d (d + 1) / 2
-// for its moments, 84 % of the FP64 pipe.  Binning and moments with their
+// for its moments, about 85 % of the FP64 pipe's time for d = 2; on 48^4 the
+// atomics bound it again.  Binning and moments with their
 // launches, against a thread per point with run-time dimensions, FP64
 // comparisons and floor, and a second pass for the moments: 1e7 points on
-// 512^2 363 us (866), 1e6 on 128^3 103 us (206), 1e6 on 48^4 142 us (336);
+// 512^2 250 us (866), 1e6 on 128^3 75 us (206), 1e6 on 48^4 119 us (336);
 // FP64 counts, 1e6 on 256^2 97 us (161).
 template <int D, int KIND, typename acc>
 __device__ __forceinline__ void bin_pass(const double* __restrict__ X, long long n, long long i0, long long stride,
@@ -226,7 +251,7 @@ __device__ __forceinline__ void bin_pass(const double* __restrict__ X, long long
                     }
                     if constexpr (KIND == 0) {
                         w = D == 1 ? last : w * last;
-                        atomicAdd(counts + idx, (acc)__float2ull_rn(w * qs));
+                        atomicAdd(counts + idx, (acc)fixed_weight(w, qs));
                     } else {
                         w = D == 1 ? last : __dmul_rn(w, last);
                         atomicAdd(counts + idx, (acc)w);
@@ -331,24 +356,24 @@ cudaError_t launch_f32_to_f64(const float* src, double* dst, long long n, cudaSt
 // arrays are 16-byte aligned): one correctly rounded conversion and an exact
 // product with a power of two.
 __device__ __forceinline__ void fix_cells(const unsigned long long* __restrict__ src, float* __restrict__ dst,
-                                          long long c, long long n, float unit) {
+                                          long long c, long long n, int e) {
     if (c + 4 <= n) {
         const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(src + c);
         const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(src + c + 2);
-        *reinterpret_cast<float4*>(dst + c) = make_float4(__ull2float_rn(a.x) * unit, __ull2float_rn(a.y) * unit,
-                                                          __ull2float_rn(b.x) * unit, __ull2float_rn(b.y) * unit);
+        *reinterpret_cast<float4*>(dst + c) = make_float4(scaled_f32(a.x, e), scaled_f32(a.y, e),
+                                                          scaled_f32(b.x, e), scaled_f32(b.y, e));
     } else {
-        for (; c < n; ++c) dst[c] = __ull2float_rn(src[c]) * unit;
+        for (; c < n; ++c) dst[c] = scaled_f32(src[c], e);
     }
 }
 
 __global__ void __launch_bounds__(256) k_fix_to_f32(const unsigned long long* __restrict__ src,
-                                                    float* __restrict__ dst, long long n, float unit,
+                                                    float* __restrict__ dst, long long n, int e,
                                                     const unsigned long long* __restrict__ outside,
                                                     unsigned long long* __restrict__ outside_copy) {
     for (long long c = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); c < n;
          c += 4LL * gridDim.x * blockDim.x)
-        fix_cells(src, dst, c, n, unit);
+        fix_cells(src, dst, c, n, e);
     if (blockIdx.x == 0 && threadIdx.x == 0) *outside_copy = *outside;
 }
 
@@ -357,7 +382,7 @@ cudaError_t launch_fix_to_f32(const unsigned long long* src, float* dst, long lo
                               cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const long long b = (n + 1023) / 1024, cap = (long long)nsm * 8;
-    k_fix_to_f32<<<(unsigned)(b < cap ? b : cap), 256, 0, st>>>(src, dst, n, (float)unit, outside, outside_copy);
+    k_fix_to_f32<<<(unsigned)(b < cap ? b : cap), 256, 0, st>>>(src, dst, n, std::ilogb(unit), outside, outside_copy);
     return cudaGetLastError();
 }
 
@@ -446,14 +471,14 @@ __global__ void __launch_bounds__(256) k_bin_many(const BinJob* __restrict__ job
                                        jb.fix, jb.outside, qscale, jb.part + b * (D + D * D));
 }
 
-__global__ void __launch_bounds__(256) k_fix_many(const BinJob* __restrict__ jobs, int njobs, float unit) {
+__global__ void __launch_bounds__(256) k_fix_many(const BinJob* __restrict__ jobs, int njobs, int e) {
     const BinJob& jb = jobs[job_of_warp(njobs, blockIdx.x, [&](int k) { return jobs[k].blk1; })];
     const long long c0 = ((long long)blockIdx.x - jb.blk1) * kCellsPerBlock;
     const long long c1 = c0 + kCellsPerBlock < jb.ncells ? c0 + kCellsPerBlock : jb.ncells;
 #pragma unroll
     for (int r = 0; r < kCellsPerBlock / 1024; ++r) {
         const long long c = c0 + 4LL * (r * 256 + threadIdx.x);
-        if (c < c1) fix_cells(jb.fix, jb.counts, c, c1, unit);
+        if (c < c1) fix_cells(jb.fix, jb.counts, c, c1, e);
     }
 }
 
@@ -479,7 +504,7 @@ cudaError_t launch_bin_many(BinJob* jobs_h, BinJob* jobs_d, int n, int d, double
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_fix_many<<<(unsigned)b1, 256, 0, st>>>(jobs_d, n, (float)(1.0 / qscale));
+    k_fix_many<<<(unsigned)b1, 256, 0, st>>>(jobs_d, n, -std::ilogb(qscale));
     return cudaGetLastError();
 }
 
