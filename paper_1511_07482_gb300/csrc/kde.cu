@@ -304,57 +304,102 @@ cudaError_t launch_kde_grid(const float* counts, const KdeDesc& g, const float* 
 }
 
 // sum_g c_g sum_m w_m phi_{S_m}(x_g - mu_m) for many mixtures (one per
-// bandwidth), nb blocks each: block b of mixture h takes the cells b, b + nb,
-// ... in steps of a block.  Bound by the FP64 pipe (an exponential and a
-// quadratic form per component and cell with counts, about 35 operations), so
-// all mixtures are one launch that fills the SMs; the mixture's last block adds
-// its nb partials in block order.
-// 32 bandwidths, three components, a 101^2 grid: 55 us (512 us in 32 launches,
-// with an upload, a copy back and a host wait each: the call 953 -> 98 us).
+// bandwidth), nb blocks each.  Bound by the FP64 pipe (an exponential and a
+// quadratic form per component and cell with counts, about 30 operations), so
+// all mixtures are one launch that fills the SMs, and lanes are not spent on
+// cells without counts (two thirds of the box around a sample, and more than
+// half of the lanes of the warps that have any): a block queues the cells with
+// counts of its 32 segments of 8 a round and takes 256 of them at a time.  Of
+// every nb segments a block has one, a different one each time: in a fixed
+// order its segments lie in the same columns, and blocks (and with them the
+// SMs, whose blocks differ by multiples of nb) had up to eight times the work
+// of others.
+// The mixture's last block adds its nb partials in block order.
+// 32 bandwidths, three components, a 101^2 grid: 36 us (55 us with a thread per
+// cell; 512 us in 32 launches, with an upload, a copy back and a host wait each).
 template <int D>
 __global__ void __launch_bounds__(256) k_mix_dot(const __grid_constant__ MixJob jb) {
-    __shared__ double mu[kMixMax][D], lam[kMixMax][D * D], amp[kMixMax];
+    constexpr int NQ = D * (D + 1) / 2;
+    __shared__ double mu[kMixMax][D], quad[kMixMax][NQ], amp[kMixMax];
+    __shared__ unsigned int qcell[512];
+    __shared__ float qcount[512];
+    __shared__ int nwarp[8];
     __shared__ double red[8];
     __shared__ int lastone;
     const KdeDesc& g = jb.g;
     const int h = blockIdx.x / jb.nb, b = blockIdx.x % jb.nb, K = jb.ncomp;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const MixComp* comps = jb.comps + (long long)h * K;
     for (int m = threadIdx.x; m < K; m += blockDim.x) {
         for (int k = 0; k < D; ++k) mu[m][k] = comps[m].mu[k];
-        for (int k = 0; k < D * D; ++k) lam[m][k] = comps[m].lam[(k / D) * MAXD + k % D];
+        int v = 0;   // -z^T lam z / 2 on the upper triangle
+        for (int i = 0; i < D; ++i)
+            for (int k = i; k < D; ++k)
+                quad[m][v++] = -0.5 * (i == k ? comps[m].lam[i * MAXD + i]
+                                              : comps[m].lam[i * MAXD + k] + comps[m].lam[k * MAXD + i]);
         amp[m] = comps[m].w * comps[m].nrm;
     }
-    __syncthreads();
     double acc = 0.0;
-    for (long long cell = (long long)b * blockDim.x + threadIdx.x; cell < g.ncells; cell += (long long)jb.nb * blockDim.x) {
-        const float cv = jb.counts[cell];
-        if (cv == 0.f) continue;
+    auto take = [&](unsigned int cell, float cv) {
         double x[D];
-        {
-            long long r = cell;
 #pragma unroll
-            for (int k = D - 1; k >= 0; --k) {
-                const int i = (int)(r % g.M[k]);
-                r /= g.M[k];
-                x[k] = g.lo[k] + g.delta[k] * (double)i;
-            }
+        for (int k = D - 1; k >= 0; --k) {
+            const unsigned int M = (unsigned int)g.M[k], r = cell / M;
+            x[k] = g.lo[k] + g.delta[k] * (double)(int)(cell - r * M);
+            cell = r;
         }
         double f = 0.0;
         for (int m = 0; m < K; ++m) {
             double z[D], q = 0.0;
 #pragma unroll
             for (int k = 0; k < D; ++k) z[k] = x[k] - mu[m][k];
+            int v = 0;
 #pragma unroll
             for (int i = 0; i < D; ++i) {
                 double t = 0.0;
 #pragma unroll
-                for (int k = 0; k < D; ++k) t += lam[m][i * D + k] * z[k];
+                for (int k = i; k < D; ++k) t += quad[m][v++] * z[k];
                 q += z[i] * t;
             }
-            f += amp[m] * exp(-0.5 * q);
+            f += amp[m] * exp(q);
         }
         acc += (double)cv * f;
+    };
+    const int seg = threadIdx.x >> 3;
+    const long long step = 32LL * jb.nb, nseg = (g.ncells + 7) / 8;
+    const long long mine = (long long)seg * jb.nb + (b + (long long)seg * (jb.nb * 5LL / 8)) % jb.nb;
+    int held = 0;   // queued cells, below 256 between rounds
+    for (long long s0 = 0; s0 < nseg; s0 += step) {
+        const long long cell = (s0 + mine) * 8 + (lane & 7);
+        const float cv = cell < g.ncells ? jb.counts[cell] : 0.f;
+        const unsigned int any = __ballot_sync(0xffffffffu, cv != 0.f);
+        if (lane == 0) nwarp[warp] = __popc(any);
+        __syncthreads();   // also: the tables are written, the last round's queue is moved
+        int at = held;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const int n = nwarp[w];
+            if (w < warp) at += n;
+            held += n;
+        }
+        if (cv != 0.f) {
+            at += __popc(any & ((1u << lane) - 1u));
+            qcell[at] = (unsigned int)cell;
+            qcount[at] = cv;
+        }
+        __syncthreads();
+        if (held >= 256) {
+            take(qcell[threadIdx.x], qcount[threadIdx.x]);
+            held -= 256;
+            __syncthreads();
+            if (threadIdx.x < held) {
+                qcell[threadIdx.x] = qcell[256 + threadIdx.x];
+                qcount[threadIdx.x] = qcount[256 + threadIdx.x];
+            }
+        }
     }
+    __syncthreads();
+    if (threadIdx.x < held) take(qcell[threadIdx.x], qcount[threadIdx.x]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
