@@ -68,6 +68,9 @@ static void host_parallel_for(size_t n, size_t grain, F&& fn) {
 static thread_local std::string g_err;
 
 static int fail(int code, const std::string& msg) {
+    // the runtime keeps an error until it is asked for: a launch of the next
+    // call would find it and report it as its own
+    if (code == KDEFFT_ERR_CUDA || code == KDEFFT_ERR_ALLOC) cudaGetLastError();
     g_err = msg;
     return code;
 }

@@ -1,0 +1,85 @@
+"""The library's host code when a CUDA call or a launch fails, without a GPU:
+its objects are linked against a CUDA runtime on the host (fake_cuda.cpp), in
+which kernels do nothing and any call can be made to return an error.  What is
+checked is what the host does next: whether the call fails, and what the one
+after it launches."""
+import glob
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_1511_07482_gb300 import build
+    objs = sorted(glob.glob(os.path.join(build.BUILD, "*.o")))
+    if len(objs) != len(build.SOURCES):
+        pytest.skip("the library is not built")
+    lib = str(tmp_path_factory.mktemp("fake") / "libkdefft_fake.so")
+    subprocess.run([build.nvcc(), "-shared", "-cudart", "none", "-Xcompiler", "-fPIC", "-Xcompiler", "-pthread",
+                    "-o", lib, *objs, os.path.join(HERE, "fake_cuda.cpp")], check=True, capture_output=True)
+    return lib
+
+
+def _run(fake, body):
+    """Run `body` in a process of its own: the library of a process is loaded once."""
+    code = f"import sys; sys.path[:0] = [{ROOT!r}, {HERE!r}]\nfrom test_host_errors_cpu import Fake\nfk = Fake({fake!r})\n{body}"
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+class Fake:
+    def __init__(self, path):
+        from paper_1511_07482_gb300 import _lib
+        self.lib = _lib.load(path)
+        self.lib.fake_log.restype = __import__("ctypes").c_char_p
+
+    def context(self):
+        from paper_1511_07482_gb300 import Context
+        return Context(0, stream=8)   # a handle that the fake's own never equal
+
+    def data(self, ctx, d=2, M=40, **opts):
+        X = np.random.default_rng(1).random((200, d))
+        return ctx.bin(X, np.zeros(d), np.ones(d), [M] * d, **opts)
+
+    def call(self, f, fail=None, nth=1):
+        """(did it raise, did the failure happen, log lines)"""
+        from paper_1511_07482_gb300 import KdefftError
+        self.lib.fake_clear()
+        self.lib.fake_fail((fail or "-").encode(), nth if fail else 0)
+        try:
+            f()
+            raised = False
+        except KdefftError:
+            raised = True
+        hit = self.lib.fake_hits()
+        self.lib.fake_fail(b"-", 0)
+        return raised, bool(hit), self.lib.fake_log().decode().splitlines()
+
+
+@pytest.mark.parametrize("what", ["cudaMemcpyAsync", "cudaMallocHost", "launch", "cudaStreamSynchronize"])
+def test_an_error_ends_with_its_call(fake, what):
+    """The runtime keeps a failed call's error until it is asked for; the next
+    call of the library must not report it as its own."""
+    _run(fake, f"""
+import numpy as np
+failed = 0
+for nth in range(1, 60):
+    ctx = fk.context()
+    ds = fk.data(ctx)
+    raised, hit, log = fk.call(lambda: ds.scv(0.02 * np.eye(2), 0.01 * np.eye(2), grad=True), {what!r}, nth)
+    if raised:
+        failed += 1
+        again, _, log2 = fk.call(lambda: ds.scv(0.02 * np.eye(2), 0.01 * np.eye(2), grad=True))
+        assert not again, (nth, log, log2)
+    ctx.close()
+    if not hit:
+        break
+assert not hit and failed >= 2
+""")
