@@ -2040,6 +2040,19 @@ static int ensure_autocorr_many(kdefft_ctx c, const std::vector<std::pair<kdefft
     for (const Job& jb : jobs)
         for (int k = 0; k < jb.ds->d; ++k) twiddle_offset(c, jb.P[k]);
     KCHK(sync_twiddles(c));
+    // from here to the end of the launch sequence the datasets hold no box: an
+    // error on the way leaves none that was not computed
+    struct Boxes {
+        std::vector<Job>& jobs;
+        bool keep = false;
+        void set(bool whole) {
+            for (const Job& jb : jobs)
+                for (int k = 0; k < 4; ++k) jb.ds->acA[k] = !whole ? -1 : k < jb.ds->d ? jb.A[k] : 0;
+        }
+        ~Boxes() {
+            if (!keep) set(false);
+        }
+    } boxes{jobs};
     size_t pool = 0;
     for (Job& jb : jobs) {
         kdefft_ds ds = jb.ds;
@@ -2170,8 +2183,6 @@ static int ensure_autocorr_many(kdefft_ctx c, const std::vector<std::pair<kdefft
                     lv.push_back(L);
                 }
             }
-        for (const Job& jb : jobs)
-            for (int k = 0; k < 4; ++k) jb.ds->acA[k] = (k < jb.ds->d) ? jb.A[k] : 0;
         if (!c->acjobs_free) KCU(cudaEventSynchronize(c->acjobs_ev));
         const size_t acb = sizeof(LineJob) * all.size();
         KCHK(c->acjobs.ensure(acb));
@@ -2186,6 +2197,7 @@ static int ensure_autocorr_many(kdefft_ctx c, const std::vector<std::pair<kdefft
                                       (long long)lv.size()};
         for (const Launch& L : lv)
             sig.insert(sig.end(), {L.kind, (long long)L.slot, L.n, L.blocks, (long long)L.sm, L.threads, L.pairs ? 1 : 0});
+        boxes.set(true);   // the tail's parameters hold the box
         if (tail) KCHK(tail->prepare(sig));
         auto issue = [&]() -> int {
             KCU(cudaMemcpyAsync(jd, c->h_acjobs.p, acb, cudaMemcpyHostToDevice, c->stream));
@@ -2209,6 +2221,7 @@ static int ensure_autocorr_many(kdefft_ctx c, const std::vector<std::pair<kdefft
             return KDEFFT_OK;
         };
         KCHK(run_graph(c, sig, issue));
+        boxes.keep = true;
         // the pinned table is free again once this work has run
         KCU(cudaEventRecord(c->acjobs_ev, c->stream));
         c->acjobs_free = false;

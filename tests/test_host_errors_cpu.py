@@ -83,3 +83,32 @@ for nth in range(1, 60):
         break
 assert not hit and failed >= 2
 """)
+
+
+@pytest.mark.parametrize("what", ["cudaMalloc", "k_line", "cudaMemcpyAsync"])
+def test_no_box_is_claimed_that_was_not_computed(fake, what):
+    """A call that fails on its way to the count autocorrelation, at whichever
+    step, leaves nothing that the next call would take for computed: one of the
+    two launches all three passes."""
+    _run(fake, f"""
+import numpy as np
+failed = 0
+passes = lambda log: sum("k_line" in l and l.endswith(" 8") for l in log)
+for grown in (False, True):
+    for nth in range(1, 60):
+        ctx = fk.context()
+        ds = fk.data(ctx)
+        if grown:
+            ds.psi(1e-4 * np.eye(2), 2)
+        raised, hit, log = fk.call(lambda: ds.psi(0.02 * np.eye(2), 2), {what!r}, nth)
+        assert hit or not raised
+        if raised:
+            failed += 1
+            again, _, log2 = fk.call(lambda: ds.psi(0.02 * np.eye(2), 2))
+            assert not again and (passes(log) == 3 or passes(log2) == 3), (grown, nth, log, log2)
+        ctx.close()
+        if not hit:
+            break
+    assert not hit and nth > 1
+assert failed >= 4
+""")
