@@ -760,15 +760,46 @@ static int staging_upload(kdefft_ctx c, void* dst, size_t bytes) {
     return KDEFFT_OK;
 }
 
+// Wait for work that an error stopped part way: the copies and launches it
+// did issue read the pinned buffers and write the results' ones, which the next
+// call uses.
+static int issue_or_drain(kdefft_ctx c, int r) {
+    if (r == KDEFFT_OK) return r;
+    if (cudaStreamSynchronize(c->stream) != cudaSuccess) cudaGetLastError();
+    if (c->side && cudaStreamSynchronize(c->side) != cudaSuccess) cudaGetLastError();
+    return r;
+}
+
+// Capture `issue` on the library's own stream (the caller's may be the legacy
+// default stream, which cannot be captured); null where any step of it fails.
+template <typename F>
+static cudaGraphExec_t capture_graph(kdefft_ctx c, F&& issue) {
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t ex = nullptr;
+    if ((c->cap_stream || cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) == cudaSuccess) &&
+        cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
+        cudaStream_t user = c->stream;
+        c->stream = c->cap_stream;
+        const int r = issue();
+        c->stream = user;
+        if (cudaStreamEndCapture(c->cap_stream, &g) == cudaSuccess && r == KDEFFT_OK)
+            if (cudaGraphInstantiate(&ex, g, 0) != cudaSuccess) ex = nullptr;
+        if (g) cudaGraphDestroy(g);
+    }
+    if (!ex) cudaGetLastError();
+    return ex;
+}
+
 // Run the stream work of one batch (`issue`: the copies and launches it
 // enqueues on c->stream) directly, or replay it from a CUDA graph cached
 // under its launch signature `sig` (every pointer, size and launch shape the
 // work depends on; the pinned staging buffers are read when the graph runs,
 // so new contents need no new graph).  Direct while profiling, so that
-// every kernel keeps its own CUDA events.
+// every kernel keeps its own CUDA events.  After an error none of the work is
+// in flight.
 template <typename F>
 static int run_graph(kdefft_ctx c, const std::vector<long long>& sig, F&& issue) {
-    if (!c->graphs || c->prof) return issue();
+    if (!c->graphs || c->prof) return issue_or_drain(c, issue());
     if (c->graph_gen != c->buf_gen) {   // a buffer some graph uses was reallocated
         if (!c->gcache.empty()) KCHK(drop_graphs(c));
         c->graph_gen = c->buf_gen;
@@ -778,34 +809,20 @@ static int run_graph(kdefft_ctx c, const std::vector<long long>& sig, F&& issue)
         // a new signature runs at once, and is captured for the next time while
         // the GPU works on it (captured first and then launched, the first call on
         // a new data set took 673 us against 568 for psi_4 with its binning,
-        // 969 against 837 for the 4-D plug-in, 616 against 572 for a selection)
+        // 969 against 837 for the 4-D plug-in, 616 against 572 for a selection).
+        // The work is on its way by then: a capture that fails leaves no graph,
+        // and the call is none the worse.
         const int64_t l0 = c->launches;
-        KCHK(issue());
+        KCHK(issue_or_drain(c, issue()));
         if (c->graph_gen != c->buf_gen) return KDEFFT_OK;   // the run reallocated a buffer: keep nothing
         const int64_t launches = c->launches - l0;
-        if (!c->cap_stream) KCU(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-        if (c->gcache.size() >= 64) KCHK(drop_graphs(c));
-        // capture on the library's own stream (the caller's may be the legacy
-        // default stream, which cannot be captured); replay on the caller's
-        cudaStream_t user = c->stream;
-        KCU(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeRelaxed));
-        c->stream = c->cap_stream;
-        const int r = issue();
-        c->stream = user;
+        if (c->gcache.size() >= 64 && drop_graphs(c) != KDEFFT_OK) return KDEFFT_OK;
+        cudaGraphExec_t ex = capture_graph(c, issue);
         c->launches = l0 + launches;
-        cudaGraph_t g = nullptr;
-        const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
-        if (r != KDEFFT_OK) {
-            if (g) cudaGraphDestroy(g);
-            return r;
+        if (ex) {
+            c->gcache.emplace(sig, kdefft_ctx_s::GraphEntry{ex, launches});
+            c->graphs_captured++;
         }
-        KCU(e);
-        cudaGraphExec_t ex = nullptr;
-        const cudaError_t ei = cudaGraphInstantiate(&ex, g, 0);
-        cudaGraphDestroy(g);
-        KCU(ei);
-        c->gcache.emplace(sig, kdefft_ctx_s::GraphEntry{ex, launches});
-        c->graphs_captured++;
         return KDEFFT_OK;
     }
     c->graph_replays++;

@@ -28,8 +28,10 @@ def fake(tmp_path_factory):
 
 
 def _run(fake, body):
-    """Run `body` in a process of its own: the library of a process is loaded once."""
-    code = f"import sys; sys.path[:0] = [{ROOT!r}, {HERE!r}]\nfrom test_host_errors_cpu import Fake\nfk = Fake({fake!r})\n{body}"
+    """Run `body` in a process of its own: the library of a process is loaded once
+    (without torch, which takes longer to import than the rest)."""
+    code = (f"import sys; sys.path[:0] = [{ROOT!r}, {HERE!r}]; sys.modules['torch'] = None\n"
+            f"from test_host_errors_cpu import Fake\nfk = Fake({fake!r})\n{body}")
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
 
@@ -111,4 +113,57 @@ for grown in (False, True):
             break
     assert not hit and nth > 1
 assert failed >= 4
+""")
+
+
+CALLS = {"bin": "lambda: fk.data(ctx)", "psi": "lambda: ds.psi(0.02 * I, 2)",
+         "scv": "lambda: ds.scv(0.02 * I, 0.01 * I, grad=True)", "autocorr": "lambda: ds.autocorr([30, 30])",
+         "fft": "lambda: (ctx.set_engine(3), ds.psi(0.02 * I, 2))"}
+
+
+@pytest.mark.parametrize("call", CALLS)
+@pytest.mark.parametrize("what", ["cudaStreamBeginCapture", "cudaStreamEndCapture", "cudaGraphInstantiate"])
+def test_a_failed_capture_is_no_error(fake, call, what):
+    """The work of a new launch sequence is issued before it is captured, so a
+    capture that fails must not fail the call (whose copies and launches are on
+    their way); the sequence is captured the next time."""
+    _run(fake, f"""
+import numpy as np
+I = np.eye(2)
+ctx = fk.context()
+ds = fk.data(ctx)
+n0 = ctx.runtime_stats()["graphs_captured"]
+raised, hit, log = fk.call({CALLS[call]}, {what!r})
+assert hit and not raised, log
+assert not fk.call({CALLS[call]})[0]
+assert ctx.runtime_stats()["graphs_captured"] > n0 or {call == "autocorr"}   # (a box is computed once)
+""")
+
+
+@pytest.mark.parametrize("graphs", [True, False])
+@pytest.mark.parametrize("call", CALLS)
+def test_nothing_is_in_flight_after_an_error(fake, call, graphs):
+    """Where the n-th launch, copy or event of a call fails, the stream is
+    waited for before the call returns: what was issued reads pinned buffers
+    and writes results that the next call uses."""
+    _run(fake, f"""
+import numpy as np
+I = np.eye(2)
+failed = 0
+for what in ("launch", "cudaMemcpyAsync 8", "cudaEventRecordWithFlags", "cudaStreamWaitEvent"):
+    for nth in range(1, 60):
+        ctx = fk.context()
+        ctx.set_graphs({graphs})
+        ds = fk.data(ctx)
+        raised, hit, log = fk.call({CALLS[call]}, what, nth)
+        if raised:
+            failed += 1
+            at = next(i for i, l in enumerate(log) if l.endswith("FAILS"))
+            issued = any(l.startswith(("launch", "cudaMemcpyAsync", "cudaMemsetAsync")) and l.endswith(" 8") for l in log[:at])
+            assert not issued or "cudaStreamSynchronize 8" in log[at:], (what, nth, log)
+        ctx.close()
+        if not hit:
+            break
+    assert not hit
+assert failed >= 2
 """)
