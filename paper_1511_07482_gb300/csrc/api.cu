@@ -4433,11 +4433,13 @@ int kdefft_ise_mixture(kdefft_ds ds, const double* H, int nH, int K, const doubl
         KCU(cudaMemcpyAsync(db, hb, up, cudaMemcpyHostToDevice, c->stream));
         c->h2d += (int64_t)up;
         cudaEvent_t ev = prof_start(c);
-        KCU(launch_mix_dot(mj, nh, c->stream));
+        const cudaError_t le = launch_mix_dot(mj, nh, c->stream);
         prof_stop(c, ev, "mix_dot", 4.0 * (double)ds->ncells * nh, 12.0 * (double)ds->ncells * K * nh);
         int rr = KDEFFT_OK;
-        if (h0 + nh == nH) rr = run(c, rs);
-        KCU(cudaStreamSynchronize(c->stream));   // the pinned table and results, whatever run did
+        if (le == cudaSuccess && h0 + nh == nH) rr = run(c, rs);
+        const cudaError_t se = cudaStreamSynchronize(c->stream);   // the pinned table and results, whatever came of them
+        KCU(le);
+        KCU(se);
         KCHK(rr);
         c->d2h += (int64_t)(sizeof(double) * nh);
         for (int h = 0; h < nh; ++h) v[h0 + h] = mj.out[h] / (double)ds->n;

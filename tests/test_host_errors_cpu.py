@@ -118,7 +118,8 @@ assert failed >= 4
 
 CALLS = {"bin": "lambda: fk.data(ctx)", "psi": "lambda: ds.psi(0.02 * I, 2)",
          "scv": "lambda: ds.scv(0.02 * I, 0.01 * I, grad=True)", "autocorr": "lambda: ds.autocorr([30, 30])",
-         "fft": "lambda: (ctx.set_engine(3), ds.psi(0.02 * I, 2))"}
+         "fft": "lambda: (ctx.set_engine(3), ds.psi(0.02 * I, 2))",
+         "ise": "lambda: ds.ise_mixture(0.02 * I, [1.0], np.zeros(2), I)"}
 
 
 @pytest.mark.parametrize("call", CALLS)
