@@ -753,13 +753,6 @@ static int staging_wait(kdefft_ctx c) {
     return KDEFFT_OK;
 }
 
-static int staging_upload(kdefft_ctx c, void* dst, size_t bytes) {
-    KCU(cudaMemcpyAsync(dst, c->h_items.p, bytes, cudaMemcpyHostToDevice, c->stream));
-    KCU(cudaEventRecord(c->staging_ev, c->stream));
-    c->staging_free = false;
-    return KDEFFT_OK;
-}
-
 // Wait for work that an error stopped part way: the copies and launches it
 // did issue read the pinned buffers and write the results' ones, which the next
 // call uses.
@@ -768,6 +761,22 @@ static int issue_or_drain(kdefft_ctx c, int r) {
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) cudaGetLastError();
     if (c->side && cudaStreamSynchronize(c->side) != cudaSuccess) cudaGetLastError();
     return r;
+}
+
+// An event that marks a pinned buffer free; where it cannot be recorded the
+// work before it is waited for.
+static int record_or_drain(kdefft_ctx c, cudaEvent_t ev) {
+    const cudaError_t e = cudaEventRecord(ev, c->stream);
+    if (e != cudaSuccess) issue_or_drain(c, KDEFFT_ERR_CUDA);
+    KCU(e);
+    return KDEFFT_OK;
+}
+
+static int staging_upload(kdefft_ctx c, void* dst, size_t bytes) {
+    KCU(cudaMemcpyAsync(dst, c->h_items.p, bytes, cudaMemcpyHostToDevice, c->stream));
+    KCHK(record_or_drain(c, c->staging_ev));
+    c->staging_free = false;
+    return KDEFFT_OK;
 }
 
 // Capture `issue` on the library's own stream (the caller's may be the legacy
@@ -2240,7 +2249,7 @@ static int ensure_autocorr_many(kdefft_ctx c, const std::vector<std::pair<kdefft
         KCHK(run_graph(c, sig, issue));
         boxes.keep = true;
         // the pinned table is free again once this work has run
-        KCU(cudaEventRecord(c->acjobs_ev, c->stream));
+        KCHK(record_or_drain(c, c->acjobs_ev));
         c->acjobs_free = false;
         c->h2d += (int64_t)acb;
         tail = nullptr;
