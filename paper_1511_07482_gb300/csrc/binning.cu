@@ -98,15 +98,17 @@ __device__ __forceinline__ unsigned long long fixed_weight(float w, float qs) {
 // which the rounding of delta can push past it) of t >= 0, below 2^31: t is
 // m 2^-sh with a 53-bit m, so the cell is m >> sh and the fraction the bits
 // below, one rounding from FP32 (t < 2^-74 gives a fraction below 2^-73
-// instead of its own, and a weight of zero either way).
+// instead of its own, and a weight of zero either way).  A step below 2^-1024
+// or past the largest double has no finite reciprocal, and t is then infinite
+// or NaN (sh < 22): such a point lies at M - 1, as fmin(t, M - 1) has it.
 __device__ __forceinline__ int cell_f32(double t, int top, float& f) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(t);
     const unsigned long long m = (b & 0xfffffffffffffULL) | 0x10000000000000ULL;
     const int sh = min(1075 - (int)((b >> 52) & 0x7ff), 126);   // the sign of -0 does not matter
-    const int s = min(sh, 63);
+    const int s = min(max(sh, 22), 63);
     int l = (int)(m >> s);
-    f = scaled_f32(m << (64 - s), s - 64 - sh);   // s >= 22: the cell's bits leave at the top
-    if (l > top) {
+    f = scaled_f32(m << (64 - s), s - 64 - max(sh, 22));   // s >= 22: the cell's bits leave at the top
+    if (l > top || sh < 22) {
         l = top;
         f = 1.f;
     }
@@ -117,7 +119,7 @@ __device__ __forceinline__ int cell_f64(double t, int top, double& f) {
     const double u = __dadd_rd(t, 4503599627370496.0);
     int l = (int)__double_as_longlong(u);
     f = __dsub_rn(t, __dsub_rn(u, 4503599627370496.0));
-    if (l > top) {
+    if (l > top || (__double2hiint(t) & 0x7fffffff) >= 0x41e00000) {   // (t infinite or NaN)
         l = top;
         f = 1.0;
     }
@@ -126,14 +128,14 @@ __device__ __forceinline__ int cell_f64(double t, int top, double& f) {
 
 // Nearest node floor(min(t, M - 1) + 1/2) with t the quotient (x - lo) / delta
 // itself.  t * (1 / delta) is within two ulps of it: the division is only
-// needed within 2^-30 of a tie.
+// needed within 2^-30 of a tie (and where there is no finite 1 / delta).
 __device__ __forceinline__ int nearest(double x, double lo, double delta, double inv, int top) {
     const double y = __dsub_rn(x, lo);
     double t = __dmul_rn(y, inv);
     const double h = __dadd_rn(t, 0.5), u = __dadd_rd(h, 4503599627370496.0);
     const double r = __dsub_rn(h, __dsub_rn(u, 4503599627370496.0));   // in [0, 1)
     int l = (int)__double_as_longlong(u);
-    if (r < 1e-9 || r > 1.0 - 1e-9) {
+    if (!(r >= 1e-9 && r <= 1.0 - 1e-9)) {   // (NaN too)
         t = fmin(__ddiv_rn(y, delta), (double)(top + 1));
         l = (int)floor(__dadd_rn(t, 0.5));
     }
