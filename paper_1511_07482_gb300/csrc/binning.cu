@@ -94,6 +94,19 @@ __device__ __forceinline__ unsigned long long fixed_weight(float w, float qs) {
     return (unsigned long long)__float2uint_rn(v) + (v >= 4294967296.f ? 1ULL : 0ULL);
 }
 
+// A fixed-point weight added to a histogram in shared memory by two 32-bit
+// additions, the carry from the low word's own sum (integer sums: any order
+// gives the same bits).  A 64-bit addition retries where lanes meet on a cell,
+// so that concentrated samples were slow: 4e6 points, all of them or half of
+// them in one cell, 1-D on 700 nodes 487 and 272 us (75 and 76 this way; 80 ->
+// 76 spread over the grid), sorted ones 215 (74), 2-D on 100^2 681 and 367 (126).
+__device__ __forceinline__ void add_shared(unsigned long long* p, unsigned long long w) {
+    unsigned int* q = reinterpret_cast<unsigned int*>(p);   // low word first
+    const unsigned int lo = (unsigned int)w, old = atomicAdd(q, lo);
+    const unsigned int hi = (unsigned int)(w >> 32) + (old + lo < lo ? 1u : 0u);
+    if (hi) atomicAdd(q + 1, hi);
+}
+
 // Cell l = min(floor(t), M - 2) and fraction t - l (1 where t reaches M - 1,
 // which the rounding of delta can push past it) of t >= 0, below 2^31: t is
 // m 2^-sh with a 53-bit m, so the cell is m >> sh and the fraction the bits
@@ -145,7 +158,8 @@ __device__ __forceinline__ int nearest(double x, double lo, double delta, double
 // ------------------------------------------------------------ the pass
 // Points i0 + threadIdx.x, + stride, .. below n: their counts into `counts`
 // (kind 0: fixed point, kind 1: FP64, kind 2: whole points), and the block's
-// sums of x - s and (x - s)(x - s)^T to part.
+// sums of x - s and (x - s)(x - s)^T to part.  SHARED: `counts` is a histogram
+// in shared memory.
 //
 // A linear-binned point is 2^d 64-bit atomic additions to scattered cells,
 // and what L2 is limited by is the 32-byte sectors they touch (58 G/s on
@@ -159,7 +173,7 @@ __device__ __forceinline__ int nearest(double x, double lo, double delta, double
 // comparisons and floor, and a second pass for the moments: 1e7 points on
 // 512^2 250 us (866), 1e6 on 128^3 75 us (206), 1e6 on 48^4 119 us (336);
 // FP64 counts, 1e6 on 256^2 97 us (161).
-template <int D, int KIND, typename acc>
+template <int D, int KIND, bool SHARED, typename acc>
 __device__ __forceinline__ void bin_pass(const double* __restrict__ X, long long n, long long i0, long long stride,
                                          const BinAxes& ax, const double* __restrict__ shift, acc* counts,
                                          unsigned long long* __restrict__ outside, double qscale,
@@ -253,7 +267,10 @@ __device__ __forceinline__ void bin_pass(const double* __restrict__ X, long long
                     }
                     if constexpr (KIND == 0) {
                         w = D == 1 ? last : w * last;
-                        atomicAdd(counts + idx, (acc)fixed_weight(w, qs));
+                        if constexpr (SHARED)
+                            add_shared(counts + idx, fixed_weight(w, qs));
+                        else
+                            atomicAdd(counts + idx, (acc)fixed_weight(w, qs));
                     } else {
                         w = D == 1 ? last : __dmul_rn(w, last);
                         atomicAdd(counts + idx, (acc)w);
@@ -329,9 +346,9 @@ __global__ void __launch_bounds__(256) k_bin(const double* __restrict__ X, long 
     const long long i0 = (long long)blockIdx.x * blockDim.x, stride = (long long)gridDim.x * blockDim.x;
     double* out = part + (size_t)blockIdx.x * (D + D * D);
     if (smem_cells)
-        bin_pass<D, KIND, acc>(X, n, i0, stride, ax, sh.s, hist, outside, qscale, out);
+        bin_pass<D, KIND, true, acc>(X, n, i0, stride, ax, sh.s, hist, outside, qscale, out);
     else
-        bin_pass<D, KIND, acc>(X, n, i0, stride, ax, sh.s, counts, outside, qscale, out);
+        bin_pass<D, KIND, false, acc>(X, n, i0, stride, ax, sh.s, counts, outside, qscale, out);
     if (smem_cells) {
         __syncthreads();
         for (unsigned int c = threadIdx.x; c < smem_cells; c += blockDim.x) {
@@ -469,8 +486,8 @@ template <int D>
 __global__ void __launch_bounds__(256) k_bin_many(const BinJob* __restrict__ jobs, int njobs, double qscale) {
     const BinJob& jb = jobs[job_of_warp(njobs, blockIdx.x, [&](int k) { return jobs[k].blk0; })];
     const long long b = (long long)blockIdx.x - jb.blk0;
-    bin_pass<D, 0, unsigned long long>(jb.X, jb.n, b * blockDim.x, (long long)jb.mblk * blockDim.x, jb.ax, jb.shift,
-                                       jb.fix, jb.outside, qscale, jb.part + b * (D + D * D));
+    bin_pass<D, 0, false, unsigned long long>(jb.X, jb.n, b * blockDim.x, (long long)jb.mblk * blockDim.x, jb.ax, jb.shift,
+                                              jb.fix, jb.outside, qscale, jb.part + b * (D + D * D));
 }
 
 __global__ void __launch_bounds__(256) k_fix_many(const BinJob* __restrict__ jobs, int njobs, int e) {
