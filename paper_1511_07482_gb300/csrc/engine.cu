@@ -869,8 +869,13 @@ int line_lines(int kind, int P, long long lines, int nsm) {
     constexpr size_t kLineSmem = 28 * 1024;
     int f = 1;
     while (f < kMaxLines / 2 && line_smem_bytes(P, f + 1) <= kLineSmem) ++f;
+    // Two lines along axis 0 share an inverse where two fit, lines 2 i and 2 i + 1
+    // whatever else is in the launch: a data set's lags are the same bits alone
+    // and in a batch.
+    const bool two = kind == kLineAxis0 && f >= 2;
     const long long spread = std::max<long long>(1, (packed ? (lines + 1) / 2 : lines) / (2LL * nsm));
     f = (int)std::min<long long>(f, spread);
+    if (two) f = std::max(2, f & ~1);
     return packed ? 2 * f : f;
 }
 
