@@ -2446,9 +2446,11 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
         KCHK(ensure_autocorr_many(c, rq));
     }
     HostTimer hbuild(c, "host:lag_build");
-    // single Gaussians join the pairs of Gaussians, if there are any, in one launch
+    // single Gaussians join the pairs of Gaussians, if there are any, in one
+    // launch (FP64, whose sums are per covariance: the same bits in either form;
+    // in FP32 a value would depend on what shares its batch)
     bool two = false;
-    for (const LagGroup& gr : groups) two = two || (gr.R == 0 && gr.nv == 2);
+    for (const LagGroup& gr : groups) two = two || (dbl && gr.R == 0 && gr.nv == 2);
     for (LagGroup& gr : groups)
         if (two && gr.R == 0 && gr.nv == 1) gr.nv = 2;
     // forms, contiguous

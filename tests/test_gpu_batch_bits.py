@@ -4,7 +4,7 @@ sets take whole points: FP64 atomics sum the linear weights in any order.)"""
 import numpy as np
 import pytest
 
-from paper_1511_07482_gb300 import BIN_SIMPLE, FP64, LSCV, synthetic
+from paper_1511_07482_gb300 import BIN_SIMPLE, FP64, L_FULL, LSCV, synthetic
 
 pytestmark = pytest.mark.gpu
 
@@ -40,4 +40,21 @@ def test_lags_alone_and_in_a_batch(d, M, count, prec):
         for ds in dss:
             ds.close()
     alone.close()
+    ctx.close()
+
+
+@pytest.mark.parametrize("prec", [{}, {"precision": FP64, "binning": BIN_SIMPLE}])
+def test_values_beside_leave_one_out(prec):
+    """One Gaussian (Eq. 10) and two (Eq. 8) a bandwidth in one batch, supports
+    of several hundred tiles."""
+    from paper_1511_07482_gb300 import Context
+    ws = [synthetic.small_case(n=800, d=2, M=[1000, 900 + i], seed=60 + i, n_candidates=12) for i in range(3)]
+    ctx = Context(0)
+    dss = [ctx.bin(w.X, w.lo, w.hi, w.M, exact_loo=i % 2, L_basis=L_FULL, **prec) for i, w in enumerate(ws)]
+    Hs = [np.stack(w.H) * 30.0 for w in ws]
+    vals = [ds.lscv(h) for ds, h in zip(dss, Hs)]
+    v = ctx.batch_lscv(dss, Hs, grad=False)
+    assert np.array_equal(v, np.concatenate(vals))
+    for ds in dss:
+        ds.close()
     ctx.close()
