@@ -2294,7 +2294,7 @@ static long long lag_tile_points(bool dbl, long long pts, bool dense) {
 // partials of order R (nv >= 0), or dense, two kernels up to order R (nv < 0).
 struct LagGroup {
     int first, n, R, nv;
-    bool two = true;   // no weights on a third covariance
+    int covs = 0;   // covariances of its FP64 kernel (lag_covs)
     int kernels() const {   // of its launch's form (the dense one and merged ones: maybe one more than n)
         return nv < 0 || (R == 0 && nv == 2) ? 2 : n;
     }
@@ -2332,7 +2332,8 @@ static void lag_groups(const ReqSet& rs, const std::vector<int>& ids, int a, int
     if (whole && lag_single_form(d, R, nv, rs.specs[g.spec].nsig)) {
         LagGroup gr{a, b - a, R, nv};
         for (int i = a; i < b; ++i)
-            for (const Term& t : rs.grids[ids[i]].terms) gr.two = gr.two && t.sig < 2;
+            for (const Term& t : rs.grids[ids[i]].terms) gr.covs = std::max(gr.covs, t.sig + 1);
+        gr.covs = lag_covs(R, nv, gr.covs);
         out.push_back(gr);
         return;
     }
@@ -2394,7 +2395,7 @@ static bool lag_item_sigmas(LagItem<real>& it, const Mat* sig, int nsig) {
 
 // The lag-domain work of one precision in a run, built on the host: the
 // items (LagItem<real>), their tiles and weights, the forms (R, nv, first
-// tile, tiles, two covariances; one launch each) and the grids in the order of the results.
+// tile, tiles, covariances; one launch each) and the grids in the order of the results.
 // run_lag builds it; issue_lag uploads and launches the batches of both
 // precisions of a run together.
 struct LagBatch {
@@ -2458,7 +2459,7 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
     for (size_t i = 0; i < ord.size(); ++i) ord[i] = i;
     std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) {
         const LagGroup &x = groups[a], &y = groups[b];
-        return x.R != y.R ? x.R < y.R : x.nv != y.nv ? x.nv < y.nv : x.two < y.two;
+        return x.R != y.R ? x.R < y.R : x.nv != y.nv ? x.nv < y.nv : x.covs < y.covs;
     });
     HermiteIndex& hx = hindex();
     const size_t ni = ord.size();
@@ -2484,12 +2485,12 @@ static int run_lag(kdefft_ctx c, ReqSet& rs, const std::vector<int>& ids, std::v
         for (int i = 1; i <= d; ++i) N = N * (gr.R + i) / i;
         const long long T = lag_tile_points(dbl, pts, gr.nv < 0), nt = (pts + T - 1) / T;
         tile0[q + 1] = tile0[q] + nt;
-        part0[q + 1] = part0[q] + nt * (dbl ? kLagSlices : 1) * lag_sums(d, gr.R, gr.nv, dbl, gr.two);
+        part0[q + 1] = part0[q] + nt * (dbl ? kLagSlices : 1) * lag_sums(d, gr.R, gr.nv, dbl, gr.covs);
         woff[q + 1] = woff[q] + (long long)nsig * (gr.nv < 0 ? 2 * N : gr.kernels());
         out0[q + 1] = out0[q] + gr.n;
         if (bt.classes.empty() || bt.classes.back()[0] != gr.R || bt.classes.back()[1] != gr.nv ||
-            bt.classes.back()[4] != (int)gr.two)
-            bt.classes.push_back({gr.R, gr.nv, (int)tile0[q], 0, (int)gr.two});
+            bt.classes.back()[4] != gr.covs)
+            bt.classes.push_back({gr.R, gr.nv, (int)tile0[q], 0, gr.covs});
         bt.classes.back()[3] += (int)nt;
         bt.fl += (double)pts * (nsig * (2.0 * d * d + 3.0 * N) + 12.0 * gr.n);
         bt.by += (double)pts * sizeof(real);
@@ -2672,7 +2673,7 @@ static int issue_lag(kdefft_ctx c, ReqSet& rs, std::vector<LagBatch>& bts) {
                 auto go = [&](auto zero) -> cudaError_t {
                     using real = decltype(zero);
                     LagJob<real> j = lag_job<real>(c, cl[2], cl[3]);
-                    j.nsum2 = cl[4];
+                    j.covs = cl[4];
                     j.items = (const LagItem<real>*)(dbase + lay[b].oI);
                     j.tiles = (const LagTile*)(dbase + lay[b].oT);
                     j.wpool = (const real*)(dbase + lay[b].oW);
@@ -2734,9 +2735,11 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
     HostTimer hbuild(c, "host:direct");
     auto ds_of = [&](size_t h) { return owner[many ? h : 0]; };
     const int per = dbl ? kLagSlices : 1, nk = f.kernels();
-    bool two = true;   // no weights on a third covariance
-    for (size_t i = 0; i < f.w.size(); ++i) two = two && (f.w[i] == 0.0 || (int)(i % f.nsig) < 2);
-    const int ns = per * lag_sums(d, f.R, f.nv, dbl, two);   // sums of a tile
+    int covs = 0;
+    for (size_t i = 0; i < f.w.size(); ++i)
+        if (f.w[i] != 0.0) covs = std::max(covs, (int)(i % f.nsig) + 1);
+    covs = lag_covs(f.R, f.nv, covs);
+    const int ns = per * lag_sums(d, f.R, f.nv, dbl, covs);   // sums of a tile
     std::vector<std::array<int, 4>> L(n);
     std::vector<int> tile0(n + 1);
     std::atomic<bool> ok{true};
@@ -2830,14 +2833,14 @@ static int direct_lag(kdefft_ctx c, const std::vector<kdefft_ds>& owner, bool ma
     }
     const double fl = pts_all * (f.nsig * (2.0 * d * d + 3.0 * N) + 12.0 * nk), by = pts_all * sizeof(real);
     double* hout = (double*)c->h_out.p;
-    const std::vector<long long> sig = {10, dbl ? 8 : 4, d, f.R, f.nv, two ? 2 : 3, (long long)n, nt, (long long)bytes, (long long)oT,
+    const std::vector<long long> sig = {10, dbl ? 8 : 4, d, f.R, f.nv, covs, (long long)n, nt, (long long)bytes, (long long)oT,
                                         (long long)oW, (long long)oD, (long long)(uintptr_t)h8, (long long)(uintptr_t)d8,
                                         (long long)(uintptr_t)c->partial.p, (long long)(uintptr_t)hout};
     auto issue = [&]() -> int {
         KCU(cudaMemcpyAsync(d8, h8, bytes, cudaMemcpyHostToDevice, c->stream));
         cudaEvent_t ev = prof_start(c);
         LagJob<real> j = lag_job<real>(c, 0, (int)nt);
-        j.nsum2 = two;
+        j.covs = covs;
         j.items = (const LagItem<real>*)d8;
         j.tiles = (const LagTile*)(d8 + oT);
         j.wpool = (const real*)(d8 + oW);

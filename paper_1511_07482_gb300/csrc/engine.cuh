@@ -260,9 +260,11 @@ int lag_table_size(int d, int R, bool dbl);
 bool lag_single_form(int d, int R, int nv, int nsig);
 // Sums that a launch of a form keeps per slot (tile or slice): its kernels in
 // FP32 and in the dense form; in FP64 the Gaussian (if any) and each partial of
-// order R once per covariance, of which the kernel takes two (two: no item of
-// the launch has weights on the third) or three (one for R > 2).
-int lag_sums(int d, int R, int nv, bool dbl, bool two);
+// order R once per covariance, of which the kernel takes covs (one for R > 2).
+int lag_sums(int d, int R, int nv, bool dbl, int covs);
+// The covariances that the FP64 kernel of a form takes where the items' weights
+// lie on the first n: one (psi_2), two or three.
+int lag_covs(int R, int nv, int n);
 // One launch of the lag kernel over tiles [t0, t0 + ntiles) of a batch (one
 // form): items, tiles and weights of the batch.  FP64 lag tiles hold
 // 32 * kLagSlices points, one per thread, in kLagSlices warp slices, so a
@@ -276,7 +278,7 @@ struct LagJob {
     const LagItem<real>* items;
     const LagTile* tiles;
     int t0, ntiles, grid;
-    int nsum2;                        // FP64 groups: no weights on the third covariance
+    int covs;                         // FP64 groups: covariances of the kernel (lag_covs)
     int block;                        // 256; FP64 also 32, 64 or 128 (slices per CTA = block / 32)
     const real* wpool;
     double* partial;

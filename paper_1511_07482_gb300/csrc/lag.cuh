@@ -34,7 +34,7 @@ __device__ __forceinline__ uint32_t inv_div(uint32_t n, uint32_t m, int sh) {
 //             gradients (R = 2), psi_r (NV = 0, one covariance for R > 2)
 //   NV = -1   two kernels (or one), each any sum of partials up to order R
 // SG: covariances that may have weights (a FP64 group without weights on the
-// third one has a kernel of its own).
+// third one has a kernel of its own, and psi_2, which has one covariance, too).
 template <int D, int R, int NV, int SG>
 struct LagForm {
     static constexpr bool dense = NV < 0;
@@ -408,7 +408,9 @@ template <typename real, int D, int R, int NV>
 static cudaError_t lag_go(const LagJob<real>& j, cudaStream_t st) {
     if constexpr (sizeof(real) == 4 && D <= 2 && NV >= 0)
         k_lag_occ4<real, D, R, NV><<<j.grid, j.block, 0, st>>>(j);
-    else if (sizeof(real) == 8 && NV >= 0 && R <= 2 && j.nsum2)
+    else if (sizeof(real) == 8 && NV == 0 && R == 2 && j.covs == 1)   // (4-D: 48 us a call, 55 with two)
+        k_lag<real, D, R, NV, (sizeof(real) == 8 && NV == 0 && R == 2) ? 1 : MAXSIG><<<j.grid, j.block, 0, st>>>(j);
+    else if (sizeof(real) == 8 && NV >= 0 && R <= 2 && j.covs == 2)
         k_lag<real, D, R, NV, (sizeof(real) == 8 && NV >= 0 && R <= 2) ? 2 : MAXSIG><<<j.grid, j.block, 0, st>>>(j);
     else
         k_lag<real, D, R, NV, MAXSIG><<<j.grid, j.block, 0, st>>>(j);
