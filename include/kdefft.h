@@ -265,7 +265,15 @@ int kdefft_lscv_r(kdefft_ds ds, const double* H, int nH, int r, double* val);
  * with sqrt(H_kk) >= delta_k / 2 (bandwidths finer than half a bin are not
  * resolved by the binned objective, which is unbounded below as H -> 0 when
  * bins hold several points); trial points outside it are rejected by the line
- * search.  Steps change the Cholesky diagonal by at most a factor e. */
+ * search.  Steps change the Cholesky diagonal by at most a factor e.
+ * Limit: the device-resident d = 2 search of SCV (FP32 datasets) forms its
+ * kernel as phi_2G times a factor.  Where the box of lags reaches so far along
+ * 2G's narrow axis that phi_2G falls below FP32's range (strongly correlated
+ * samples; normal ones at a correlation of 0.9 on 256 x 256) the factor
+ * overflows, the product has no value and every start is rejected:
+ * KDEFFT_ERR_ARG, "no start point inside the search domain".
+ * kdefft_set_engine(ctx, KDEFFT_ENGINE_HOST_SELECT) searches them from the
+ * host. */
 int kdefft_select_H(kdefft_ds ds, int method, const double* H0, const double* G,
                     int n_starts, int max_iter, double* H_out, double* f_out,
                     int64_t* n_evals);
@@ -356,9 +364,10 @@ int kdefft_set_autotune(kdefft_ctx ctx, int on);
  * Eq. 25's double sum) on the half box j_0 in [0, A_0], |j_k| <= A_k
  * (k >= 1), A_k <= M_k - 1: out holds prod_{k>=1} (2 A_k + 1) x (A_0 + 1)
  * FP64 values, layout [j_{d-1}]..[j_1][j_0] (j_0 fastest, index j_k + A_k
- * for k >= 1); a_{-j} = a_j gives the other half.  Computed in FP64 from the
- * count spectrum at the smallest 2^a 3^b 5^c padding >= M_k + A_k (cached on
- * the dataset and reused by the lag-domain engine).  out: host.  Errors:
+ * for k >= 1); a_{-j} = a_j gives the other half.  Computed
+ * through the count spectrum at the smallest 2^a 3^b 5^c padding >= M_k + A_k,
+ * in FP32 pairs (about 44 bits) for FP32 datasets and in FP64 for FP64 ones
+ * (cached on the dataset and reused by the lag-domain engine).  out: host.  Errors:
  * KDEFFT_ERR_ARG for A outside [0, M_k - 1], KDEFFT_ERR_UNSUPPORTED when that
  * padding exceeds 4096 on an axis. */
 int kdefft_autocorr(kdefft_ds ds, const int* A, double* out);

@@ -2003,10 +2003,11 @@ static int ensure_spectra(kdefft_ctx c, const std::vector<std::pair<kdefft_ds, s
 // ============================================================ lag-domain engine
 // Largest radix of the FP32-pair transforms.  A pair butterfly is a long
 // chain of dependent FP32 operations, so small radices (more threads busy
-// per stage, shorter chains) win: measured for the count spectrum and
-// autocorrelation of a 256^2 grid at P = 384 (n = 1e5), 42 µs with radices up
-// to 5, 55 µs up to 8, 84 µs up to 16 (the FP64 passes: 81 µs); 128^3 at
-// P = 180 (n = 1e6): 405, 406, 494 µs (FP64: 921 µs).
+// per stage, shorter chains, 48 to 64 registers instead of 128) win.  Measured
+// with a transform a line in passes of 256 threads, before k_line: 256^2 at
+// P = 384 42 us with radices up to 5, 55 up to 8, 84 up to 16; 128^3 at P = 180
+// 405, 406, 494 us.  k_line has the radices up to 5 only; larger ones have not
+// been measured in it.
 static constexpr int kPairRadix = 5;
 
 // Work that follows the autocorrelation passes on the stream (the device
@@ -3099,9 +3100,9 @@ static int run(kdefft_ctx c, ReqSet& rs) {
     std::vector<LagBatch> lagq;
     int r = run_requests<double>(c, rs, s64, lagq);
     if (r == KDEFFT_OK) r = run_requests<float>(c, rs, s32, lagq);
-    // the lag batches of both precisions: one upload, one launch sequence,
-    // one copy back, one wait (also on an error, as the pending reads point
-    // into rs)
+    // the lag batches of both precisions: one upload, one launch sequence
+    // (whose last blocks write the values to pinned memory), one wait (also on
+    // an error, as the pending reads point into rs)
     if (r == KDEFFT_OK) r = issue_lag(c, rs, lagq);
     const int f = flush_reads(c);
     return r != KDEFFT_OK ? r : f;

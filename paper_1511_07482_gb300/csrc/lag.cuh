@@ -117,9 +117,9 @@ __device__ __forceinline__ void warp_sums_all(T* v, int lane, Add add, Give shfl
 // the products x_a x_b once for all covariances (SCV values of 5 bandwidths on
 // 61 x 97 x 45 48 -> 42 us, values and gradients of 16 on 256^2 35 -> 31 us).
 // Per launch, against pairs of kernels with the sums of their tiles in a launch
-// of their own (4 to 6 us more): psi_4 of 256 bandwidths on 128^3 78 us (329),
+// of their own (4 to 6 us more): psi_4 of 256 bandwidths on 128^3 67 us (329),
 // 512 data sets x 16 LSCV bandwidths with gradients 122 us (364), SCV with
-// gradients in FP64, 16 bandwidths on 256^2, 36 us (145).
+// gradients in FP64, 16 bandwidths on 256^2, 31 us (145).
 template <typename real, int D, int R, int NV, int SG>
 __device__ __forceinline__ void lag_tiles(const LagJob<real>& jb) {
     using F = LagForm<D, R, NV, SG>;
@@ -384,8 +384,9 @@ __global__ void __launch_bounds__(256) k_lag(const __grid_constant__ LagJob<real
 
 // FP32 groups with d <= 2 are held to 64 registers, four CTAs an SM (512 data
 // sets x 16 bandwidths 122 us, against 148 with the compiler's 75); with d = 3
-// the same cap (or three CTAs) is slower than the compiler's 126 (psi_4 91 and
-// 82 us against 78, SCV gradients 18 and 15 against 12).
+// the same cap (or three CTAs) is slower than the compiler's 126 (psi_4 with
+// tiles of 1024 points 91 and 82 us against 78, SCV gradients 18 and 15 against
+// 12).
 template <typename real, int D, int R, int NV>
 __global__ void __launch_bounds__(256, 4) k_lag_occ4(const __grid_constant__ LagJob<real> jb) {
     lag_tiles<real, D, R, NV, MAXSIG>(jb);
